@@ -353,10 +353,11 @@ helm_status helm_profile_read(helm_handle *h, int ncls, int *launches, double *m
 /* ---- cycle tuning (kernel choices; no counterpart in the paper) ----
  * The arithmetic of Algorithm 1 is fixed by helm_mg_params; these choices only pick which
  * kernels carry it out, and every choice gives the same cycle up to FP32 rounding order.
- *   tail_levels    the coarsest levels (>= 2, or 0 for none) fused into one single-block
- *                  shared-memory launch; -1 = as many as fit (at most 4 levels, each with at
- *                  most 4096 unknowns, all in 200 KB of shared memory).  Values above what
- *                  fits are clamped.
+ *   tail_levels    the coarsest levels (>= 2, or 0 for none) fused into one launch of a thread-
+ *                  block cluster, every level in distributed shared memory; -1 = as many as fit
+ *                  (at most 6 levels, each with at most 8192 unknowns, 16384 in 2D complex64,
+ *                  in 200 KB a block).
+ *                  Values above what fits are clamped.
  *   level_tile[l]  level l (0 = finest) of a 2D complex64 V(2,2) omega-Jacobi cycle runs its
  *                  two pre-sweeps + residual + full weighting, and its prolongation + two
  *                  post-sweeps, as two temporally blocked launches with tile shape
@@ -381,10 +382,9 @@ typedef enum {
 typedef struct {
     int tail_levels;
     int level_tile[HELM_MAX_LEVELS];
-    int cluster_levels;  /* 2D complex64: the coarsest levels (>= 2, 0 = off) in one launch of a
-                            thread-block cluster, every level in distributed shared memory;
-                            takes precedence over tail_levels; clamped to what fits (200 KB per
-                            block, at most 6 levels) */
+    int cluster_levels;  /* 2D complex64: the same fused tail with a depth of its own (>= 2, 0 = off)
+                            on cluster_ctas blocks; takes precedence over tail_levels; clamped to
+                            what fits (200 KB per block, at most 6 levels) */
     int cluster_ctas;    /* blocks (SMs) of that cluster: 8 or 16 */
     int cluster_halo;    /* rows each block of the cluster keeps beyond its slab of every level:
                             1 = one halo row, a cluster barrier after every sweep and transfer;

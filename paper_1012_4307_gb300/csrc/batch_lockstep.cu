@@ -249,9 +249,9 @@ helm_status build(BatchLockstep *L, int m) {
                 if (mb.first == p && mb.second < HELM_MAX_LEVELS) t.level_tile[mb.second] = ph.tile;
         helm_status st = helm_set_tuning(h, &t);
         if (st != HELM_OK) return st;
-        if (p == 0) L->deep = ctail_deep(h);
-        if (ctail_deep(h) != L->deep) return helm_fail(HELM_ERR_ARG, "the problems' cluster tails differ");
-        if (!ctail_image(h, false, L->deep)) return helm_fail(HELM_ERR_NOMEM, "cluster-tail image of problem %d", p);
+        if (p == 0) L->deep = h->tail[0].deep;
+        if (h->tail[0].deep != L->deep) return helm_fail(HELM_ERR_ARG, "the problems' cluster tails differ");
+        if (!ctail_image(h, 0, L->deep)) return helm_fail(HELM_ERR_NOMEM, "cluster-tail image of problem %d", p);
         CKR(cudaStreamSynchronize(h->stream));
     }
     CKR(cudaMalloc((void **)&L->active, P * sizeof(int)));
@@ -297,7 +297,7 @@ helm_status build(BatchLockstep *L, int m) {
         E.b_top = h->lv[t0].b32;
         E.u_top = t0 == 0 ? (float2 *)h->Z : h->lv[t0].u32;
         E.ustride = t0 == 0 ? h->np : 0;
-        E.img = ctail_image(h, false, L->deep);
+        E.img = ctail_image(h, 0, L->deep);
         E.active = L->active + p;
         BVec &V = vec[p];
         V.n = h->np;

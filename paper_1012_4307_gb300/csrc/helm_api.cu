@@ -361,47 +361,53 @@ helm_status helm_create_impl(const helm_grid *grid, double theta, const double *
         k2l.swap(k2c);
         for (int a = 0; a < 3; a++) nl[a] = nc[a];
     }
-    // coarse tail: the longest run of levels ending at the coarsest with at most
-    // TAIL_MAX_UNKNOWNS interior nodes each (and at most MAX_TAIL_LEVELS levels)
-    if (mg->kind != HELM_PC_NONE) {
-        const int nlev = (int)h->lv.size();
-        for (int pass = 0; pass < 2; pass++) {
-            const size_t es = pass == 0 ? sizeof(float2) : sizeof(double2);
-            int top = nlev - 1;
-            while (top > 0 && nlev - top < MAX_TAIL_LEVELS) {
-                const LevelDev &L = h->lv[top - 1];
-                const double ni = (double)(L.n[0] - 2) * (L.n[1] - 2) * (dim == 3 ? (double)(L.n[2] - 2) : 1.0);
-                int n[MAX_TAIL_LEVELS][3];
-                for (int l = top - 1; l < nlev; l++)
-                    for (int a = 0; a < 3; a++) n[l - top + 1][a] = h->lv[l].n[a];
-                if (ni > TAIL_MAX_UNKNOWNS || mg_tail_smem_bytes_nodes(dim, nlev - top + 1, n, h->nu_c, es) > TAIL_SMEM_BYTES)
-                    break;
-                top--;
-            }
-            // a lone coarsest level keeps its dense-solve kernel
-            (pass == 0 ? h->tail_top32 : h->tail_top64) = nlev - top >= 2 ? top : -1;
-        }
-    }
     h->tune.tail_levels = -1;
     for (int l = 0; l < HELM_MAX_LEVELS; l++) h->tune.level_tile[l] = HELM_TILE_32x8;
     h->tune.cluster_levels = 0;
     h->tune.cluster_ctas = 16;
     h->tune.cluster_halo = 3;
-    // how many coarsest levels a cluster tail can hold (2D only)
-    if (mg->kind != HELM_PC_NONE && dim == 2) {
+    if (mg->kind != HELM_PC_NONE) {
         const int nlev = (int)h->lv.size();
-        for (int k = 0; k < 2; k++) {
-            const int nc = k ? 16 : 8;
-            int fit = 0;
-            for (int nt = 2; nt <= std::min(nlev, MAX_CT_LEVELS); nt++) {
-                int n[MAX_CT_LEVELS][3];
-                for (int q = 0; q < nt; q++)
-                    for (int a = 0; a < 3; a++) n[q][a] = h->lv[nlev - nt + q].n[a];
-                unsigned off[MAX_CT_LEVELS][7], obc, oz;
-                if (mg_ctail_layout(nt, n, nc, h->nu_c, off, &obc, &oz) <= CT_SMEM_BYTES) fit = nt;
+        // shared memory per block of a tail over the nt coarsest levels
+        auto tail_bytes = [&](int nt, int nc, size_t es) {
+            int n[MAX_CT_LEVELS][3];
+            for (int q = 0; q < nt; q++)
+                for (int a = 0; a < 3; a++) n[q][a] = h->lv[nlev - nt + q].n[a];
+            unsigned off[MAX_CT_LEVELS][8], obc, oz;
+            return mg_ctail_layout(dim, es, nt, n, nc, h->nu_c, off, &obc, &oz);
+        };
+        // the fused tail: the longest run of levels ending at the coarsest that fit (a lone
+        // coarsest level keeps its dense-solve kernel) with at most tail_max_unknowns interior nodes
+        // each, on 16 blocks, or 8 where the device runs no cluster of 16
+        for (int prec = 0; prec < 2; prec++) {
+            const size_t es = prec == 0 ? sizeof(float2) : sizeof(double2);
+            const double most = tail_max_unknowns(dim, es);
+            for (int nc = 16; nc >= 8 && h->tail_built[prec] < 0; nc -= 8) {
+                int fit = 0;
+                size_t bytes = 0;
+                for (int nt = 2; nt <= std::min(nlev, MAX_CT_LEVELS); nt++) {
+                    const LevelDev &L = h->lv[nlev - nt];
+                    const double ni = (double)(L.n[0] - 2) * (L.n[1] - 2) * (dim == 3 ? (double)(L.n[2] - 2) : 1.0);
+                    const size_t b = tail_bytes(nt, nc, es);
+                    if (ni > most || b > CT_SMEM_BYTES) break;
+                    fit = nt;
+                    bytes = b;
+                }
+                if (fit < 2) continue;
+                if ((prec == 0 ? mg_ctail_max_clusters<float>(dim, nc, bytes)
+                               : mg_ctail_max_clusters<double>(dim, nc, bytes)) < 1)
+                    continue;
+                h->tail_built[prec] = nlev - fit;
+                h->tail_ctas[prec] = nc;
             }
-            h->ctail_fit[k] = fit;
         }
+        // how many coarsest levels a cluster tail chosen by the tuning can hold (2D only, every
+        // level with an odd number of rows)
+        if (dim == 2 && h->lv[nlev - 1].n[1] % 2 == 1)
+            for (int k = 0; k < 2; k++)
+                for (int nt = 2; nt <= std::min(nlev, MAX_CT_LEVELS); nt++)
+                    if (tail_bytes(nt, k ? 16 : 8, sizeof(float2)) <= CT_SMEM_BYTES) h->ctail_fit[k] = nt;
+        helm_refresh_tails(h, true);
     }
     CKC(cudaStreamSynchronize(s));
     *out = h;
@@ -560,70 +566,85 @@ static cudaError_t coarse_solve(helm_handle *h, LevelDev &L, const typename CT<R
     return launch_dense_solve<R>(L.n, h->dim, h->nu_c, LvBuf<R>::minv(h), b, u, h->stream);
 }
 
+// Key of a tail's image.
+static int image_key(int top, int nc, bool deep, int prec) { return top * 64 + nc + (deep ? 4096 : 0) + (prec ? 8192 : 0); }
+
+const void *ctail_image(const helm_handle *h, int prec, bool deep) {
+    const helm_handle::Tail &T = h->tail[prec];
+    if (T.top < 0) return nullptr;
+    const int key = image_key(T.top, T.nc, deep, prec);
+    for (const auto &e : h->ctail_img)
+        if (e.first == key) return e.second;
+    return nullptr;
+}
+
+// Builds the image of the selected tail unless the handle has it.  A failure leaves the tail without
+// an image: the deep-halo kernel is then not used, and the other builds its blocks' memory itself.
+template <typename R> static void build_image(helm_handle *h, bool deep) {
+    const int prec = sizeof(R) == sizeof(float) ? 0 : 1;
+    const helm_handle::Tail &T = h->tail[prec];
+    if (T.top < 0 || ctail_image(h, prec, deep)) return;
+    const int nt = (int)h->lv.size() - T.top;
+    DevOp<R> ops[MAX_CT_LEVELS];
+    for (int k = 0; k < nt; k++) ops[k] = LvBuf<R>::op(h->lv[T.top + k]);
+    void *img = nullptr;
+    cudaError_t e = cudaErrorInvalidValue;
+    if constexpr (sizeof(R) == sizeof(float)) {
+        if (deep) e = build_mg_chalo_image(nt, ops, h->minv32, h->nu_c, T.nc, &img, h->stream);
+    }
+    if (!deep)
+        e = build_mg_ctail_image<R>(h->dim, nt, ops, LvBuf<R>::minv(h), h->nu_c, (R)h->mg.omega, T.nc, &img, h->stream);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    try {
+        h->ctail_img.reserve(h->ctail_img.size() + 1);
+        h->owned.push_back(img);
+        h->ctail_img.push_back({image_key(T.top, T.nc, deep, prec), img});
+    } catch (...) {
+        cudaFree(img);
+    }
+}
+
+void helm_refresh_tails(helm_handle *h, bool build) {
+    const helm_mg_params &m = h->mg;
+    const helm_tuning &t = h->tune;
+    h->tail[0] = h->tail[1] = helm_handle::Tail{};
+    if (m.kind == HELM_PC_NONE) return;
+    const int nlev = (int)h->lv.size();
+    for (int prec = 0; prec < 2; prec++) {
+        helm_handle::Tail &T = h->tail[prec];
+        // a cluster tail named by the tuning (2D complex64) goes before the fused tail
+        const int named = prec == 0 && h->dim == 2 && t.cluster_levels >= 2
+                              ? std::min(t.cluster_levels, h->ctail_fit[t.cluster_ctas == 16 ? 1 : 0]) : 0;
+        if (named >= 2) {
+            T.top = nlev - named;
+            T.nc = t.cluster_ctas;
+        } else if (h->tail_built[prec] >= 0 && t.tail_levels != 0) {
+            const int built = nlev - h->tail_built[prec];
+            T.top = nlev - (t.tail_levels < 0 ? built : std::min(built, t.tail_levels));
+            T.nc = h->tail_ctas[prec];
+        }
+        if (T.top >= 0 && prec == 0 && h->dim == 2 && t.cluster_halo == 3 && m.smoother == HELM_SMOOTH_JACOBI &&
+            m.gamma_f == 1 && m.gamma_c == 1 && m.nu1 <= 2 && m.nu2 <= 2) {
+            DevOp<float> ops[MAX_CT_LEVELS];
+            for (int l = T.top; l < nlev; l++) ops[l - T.top] = h->lv[l].M32;
+            T.deep = mg_chalo_bytes(nlev - T.top, ops, h->nu_c, T.nc) > 0;
+        }
+    }
+    if (!build) return;
+    if (h->tail[0].deep) {
+        build_image<float>(h, true);
+        if (!ctail_image(h, 0, true)) h->tail[0].deep = false;
+    }
+    if (!h->tail[0].deep) build_image<float>(h, false);
+    build_image<double>(h, false);
+}
+
 // u <- MG(l, M_l, b, u, nu1, nu2, C, gf, gc).  'zero' means u = 0 on entry (not read).
 // The result always ends in u.  Level l uses its own t buffer as the Jacobi partner; coarse
 // levels use their own b (restricted residual) and u (error) buffers.
-// First level of the fused tail under the handle's tuning (-1: no tail): the built (largest
-// fitting) tail shortened to tune.tail_levels levels.
-template <typename R> int tail_top(const helm_handle *h) {
-    const int built = sizeof(R) == sizeof(float) ? h->tail_top32 : h->tail_top64;
-    const int want = h->tune.tail_levels;
-    if (built < 0 || want == 0) return -1;
-    if (want < 0) return built;
-    const int last = (int)h->lv.size() - 1;
-    const int top = std::max(built, last - want + 1);
-    return last - top + 1 >= 2 ? top : -1;
-}
-template int tail_top<float>(const helm_handle *);
-template int tail_top<double>(const helm_handle *);
-
-const void *ctail_image(helm_handle *h, bool build, bool deep) {
-    const int top = ctail_top(h);
-    if (top < 0) return nullptr;
-    const int nc = h->tune.cluster_ctas, key = top * 32 + nc + (deep ? 1024 : 0);
-    for (const auto &e : h->ctail_img)
-        if (e.first == key) return e.second;
-    if (!build) return nullptr;
-    const int nt = (int)h->lv.size() - top;
-    DevOp<float> ops[MAX_CT_LEVELS];
-    for (int k = 0; k < nt; k++) ops[k] = h->lv[top + k].M32;
-    void *img = nullptr;
-    if ((deep ? build_mg_chalo_image(nt, ops, h->minv32, h->nu_c, nc, &img, h->stream)
-              : build_mg_ctail_image(nt, ops, h->minv32, h->nu_c, nc, &img, h->stream)) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    try {
-        h->owned.push_back(img);
-        h->ctail_img.push_back({key, img});
-    } catch (...) {
-        cudaFree(img);
-        return nullptr;
-    }
-    return img;
-}
-
-bool ctail_deep(const helm_handle *h) {
-    if (h->tune.cluster_halo != 3) return false;
-    const int top = ctail_top(h);
-    const helm_mg_params &m = h->mg;
-    if (top < 0 || m.smoother != HELM_SMOOTH_JACOBI || m.gamma_f != 1 || m.gamma_c != 1 || m.nu1 > 2 || m.nu2 > 2)
-        return false;
-    const int nt = (int)h->lv.size() - top;
-    DevOp<float> ops[MAX_CT_LEVELS];
-    for (int k = 0; k < nt; k++) ops[k] = h->lv[top + k].M32;
-    return mg_chalo_bytes(nt, ops, h->nu_c, h->tune.cluster_ctas) > 0;
-}
-
-int ctail_top(const helm_handle *h) {
-    const int want = h->tune.cluster_levels;
-    if (h->dim != 2 || want < 2 || h->mg.kind == HELM_PC_NONE) return -1;
-    const int fit = h->ctail_fit[h->tune.cluster_ctas == 16 ? 1 : 0];
-    const int nt = std::min(want, fit);
-    if (nt < 2) return -1;
-    return (int)h->lv.size() - nt;
-}
-
 template <typename R>
 static cudaError_t cycle(helm_handle *h, int l, const typename CT<R>::T *b, typename CT<R>::T *u, bool zero, int gf,
                          int gc) {
@@ -631,45 +652,29 @@ static cudaError_t cycle(helm_handle *h, int l, const typename CT<R>::T *b, type
     LevelDev &L = h->lv[l];
     const int last = (int)h->lv.size() - 1;
     if (l == last) return coarse_solve<R>(h, L, b, u);
-    if constexpr (sizeof(R) == sizeof(float)) {
-        if (l == ctail_top(h)) {
-            // levels l..last in one launch of a thread-block cluster
-            const int nt = last - l + 1;
-            DevOp<float> ops[MAX_CT_LEVELS];
-            double bytes = 0;
-            for (int k = 0; k < nt; k++) {
-                ops[k] = h->lv[l + k].M32;
-                bytes += interior(h->lv[l + k], h->dim) * sizeof(float2) * 8.0;
-            }
-            ProfScope ps(h, HELM_K_COARSE, bytes + (double)h->nu_c * h->nu_c * sizeof(float2), 0);
-            if (zero && ctail_deep(h)) {
-                const void *img = ctail_image(h, !h->capturing, true);
-                if (img)
-                    return launch_mg_chalo(nt, ops, b, u, h->minv32, h->nu_c, h->mg.nu1, h->mg.nu2,
-                                           (float)h->mg.omega, h->tune.cluster_ctas, img, h->stream);
-            }
-            return launch_mg_ctail(nt, ops, b, u, h->minv32, h->nu_c, h->mg.nu1, h->mg.nu2,
-                                   h->mg.smoother == HELM_SMOOTH_RB, (float)h->mg.omega, zero ? 1 : 0, gf, gc,
-                                   h->tune.cluster_ctas, ctail_image(h, !h->capturing, false), h->stream);
-        }
-    }
-    if (l == tail_top<R>(h)) {
-        // levels l..last in one fused single-block launch
+    constexpr int prec = sizeof(R) == sizeof(float) ? 0 : 1;
+    if (l == h->tail[prec].top) {
+        // levels l..last in one launch of a thread-block cluster
+        const helm_handle::Tail &T = h->tail[prec];
         const int nt = last - l + 1;
-        DevOp<R> ops[MAX_TAIL_LEVELS];
-        typename CT<R>::T *bb[MAX_TAIL_LEVELS], *uu[MAX_TAIL_LEVELS], *tt[MAX_TAIL_LEVELS];
+        DevOp<R> ops[MAX_CT_LEVELS];
         double bytes = 0;
         for (int k = 0; k < nt; k++) {
-            LevelDev &Lk = h->lv[l + k];
-            ops[k] = LvBuf<R>::op(Lk);
-            bb[k] = k == 0 ? const_cast<typename CT<R>::T *>(b) : LvBuf<R>::b(Lk);
-            uu[k] = k == 0 ? u : LvBuf<R>::u(Lk);
-            tt[k] = LvBuf<R>::t(Lk);
-            bytes += interior(Lk, h->dim) * sizeof(typename CT<R>::T) * 8.0;
+            ops[k] = LvBuf<R>::op(h->lv[l + k]);
+            bytes += interior(h->lv[l + k], h->dim) * sizeof(C) * 8.0;
         }
-        ProfScope ps(h, HELM_K_COARSE, bytes + (double)h->nu_c * h->nu_c * sizeof(typename CT<R>::T), 0);
-        return launch_mg_tail<R>(h->dim, nt, ops, bb, uu, tt, LvBuf<R>::minv(h), h->nu_c, h->mg.nu1, h->mg.nu2,
-                                 h->mg.smoother == HELM_SMOOTH_RB, (R)h->mg.omega, gf, gc, zero ? 1 : 0, h->stream);
+        ProfScope ps(h, HELM_K_COARSE, bytes + (double)h->nu_c * h->nu_c * sizeof(C), 0);
+        if constexpr (prec == 0) {
+            if (zero && T.deep) {
+                const void *img = ctail_image(h, 0, true);
+                if (img)
+                    return launch_mg_chalo(nt, ops, b, u, h->minv32, h->nu_c, h->mg.nu1, h->mg.nu2,
+                                           (float)h->mg.omega, T.nc, img, h->stream);
+            }
+        }
+        return launch_mg_ctail<R>(h->dim, nt, ops, b, u, LvBuf<R>::minv(h), h->nu_c, h->mg.nu1, h->mg.nu2,
+                                  h->mg.smoother == HELM_SMOOTH_RB, (R)h->mg.omega, zero ? 1 : 0, gf, gc, T.nc,
+                                  ctail_image(h, prec, false), h->stream);
     }
     const double es = sizeof(C), rs = sizeof(R), ni = interior(L, h->dim), nd = h->dim == 3 ? 8.0 : 4.0;
     if constexpr (sizeof(R) == sizeof(float)) {

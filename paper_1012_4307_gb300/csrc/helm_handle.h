@@ -68,12 +68,18 @@ struct helm_handle {
     double2 *wts[3] = {nullptr, nullptr, nullptr};  // dual-volume weights per axis
 
     std::vector<LevelDev> lv;
-    // first level handled by the fused coarse-tail kernel, per precision (-1: none); chosen so
-    // the tail's vectors fit in shared memory
-    int tail_top32 = -1, tail_top64 = -1;  // first level of the fused tail (-1: none), as built
+    // the deepest fused coarse tail the handle offers, per precision (0: complex64, 1: complex128):
+    // its first level (-1: none) and blocks per cluster
+    int tail_built[2] = {-1, -1}, tail_ctas[2] = {16, 16};
     helm_tuning tune{};                      // kernel choices (see helm_set_tuning)
     int ctail_fit[2] = {0, 0};               // most coarsest levels a cluster tail of 8 / 16 blocks holds
-    // initial shared-memory images of the cluster tail, keyed by first level * 32 + blocks
+    // the fused tail that the tuning selects, per precision (helm_refresh_tails)
+    struct Tail {
+        int top = -1;      // first level (-1: none)
+        int nc = 16;       // blocks per cluster
+        bool deep = false; // cycles from zero run the deep-halo kernel (complex64 2D V-cycles)
+    } tail[2];
+    // initial shared-memory images of the tails, keyed by first level, blocks, kernel and precision
     // (device memory, also listed in owned)
     std::vector<std::pair<int, void *>> ctail_img;
     int nu_c = 0;
@@ -180,18 +186,13 @@ cudaError_t precondition_pair(helm_handle *h, const float4 *v, const double2 *al
 // there by the delayed-CGS2 update pass), and that buffer.
 cudaError_t precondition_level0_c64(helm_handle *h, float2 *z);
 float2 *level0_rhs_c64(helm_handle *h);
-// First level of the fused coarse tail of a precision-R cycle under the handle's tuning (-1: none).
-template <typename R> int tail_top(const helm_handle *h);
-// First level of the cluster tail (2D complex64 cycles) under the handle's tuning (-1: none).
-int ctail_top(const helm_handle *h);
-// Whether the cluster tail of a cycle from zero runs as the deep-halo kernel under the handle's
-// tuning (cluster_halo 3, a V-cycle of omega-Jacobi with at most two sweeps each way, levels that
-// fit).
-bool ctail_deep(const helm_handle *h);
-// The initial shared-memory image of the cluster tail (deep: of the deep-halo kernel) for the
-// current tuning (null: no tail, or not built and build false); built on the handle's stream,
-// outside graph capture.
-const void *ctail_image(helm_handle *h, bool build, bool deep);
+// Recomputes h->tail for the handle's tuning; with build, also builds the initial shared-memory
+// images its cycles use (allocates device memory and launches on the handle's stream; outside graph
+// capture).
+void helm_refresh_tails(helm_handle *h, bool build);
+// The initial shared-memory image of a complex64 (prec 0) or complex128 (1) tail (deep: of the
+// deep-halo kernel); null if it was not built.
+const void *ctail_image(const helm_handle *h, int prec, bool deep);
 
 // Lockstep engine of helm_solve_batch (batch_lockstep.cu): every phase of an FGMRES step is one
 // launch over all problems.  lockstep_eligible tells whether the batch's configuration is one it

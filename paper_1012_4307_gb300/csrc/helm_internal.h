@@ -20,8 +20,11 @@ __host__ __device__ __forceinline__ float2 mk(float a, float b) { return make_fl
 __host__ __device__ __forceinline__ double2 mk(double a, double b) { return make_double2(a, b); }
 template <typename C> __host__ __device__ __forceinline__ C cadd(C a, C b) { return mk(a.x + b.x, a.y + b.y); }
 template <typename C> __host__ __device__ __forceinline__ C csub(C a, C b) { return mk(a.x - b.x, a.y - b.y); }
+// a b with its roundings written out (one product rounded, the other inside the fma), so that
+// every kernel forms it alike: left to the compiler's contraction, two kernels that must agree bit
+// for bit can round different products.
 template <typename C> __host__ __device__ __forceinline__ C cmul(C a, C b) {
-    return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+    return mk(fma(a.x, b.x, -(a.y * b.y)), fma(a.x, b.y, a.y * b.x));
 }
 // acc + a*b
 template <typename C> __host__ __device__ __forceinline__ C cfma(C a, C b, C acc) {
@@ -34,14 +37,14 @@ template <typename C> __host__ __device__ __forceinline__ C cfmac(C a, C b, C ac
 template <typename C, typename R> __host__ __device__ __forceinline__ C cscale(C a, R s) { return mk(a.x * s, a.y * s); }
 // 1 / a = conj(a) / |a|^2 (one real division)
 template <typename C> __host__ __device__ __forceinline__ C cinv(C a) {
-    const auto d = a.x * a.x + a.y * a.y;
+    const auto d = fma(a.x, a.x, a.y * a.y);
     const auto r = decltype(d)(1) / d;
     return mk(a.x * r, -a.y * r);
 }
 // 1 / a for complex64 with the fast approximate reciprocal (__fdividef, about 2 ulp): used
 // where the result only enters a complex64 smoother update.
 __device__ __forceinline__ float2 cinv_fast(float2 a) {
-    const float r = __fdividef(1.0f, a.x * a.x + a.y * a.y);
+    const float r = __fdividef(1.0f, fmaf(a.x, a.x, a.y * a.y));
     return make_float2(a.x * r, -a.y * r);
 }
 // dst[q] = src[q] for q < n (src global and unchanged during the kernel, dst this block's
@@ -207,63 +210,40 @@ cudaError_t launch_pre2_restrict(const DevOp<float> &op, int tile, float omega, 
 cudaError_t launch_prolong_post2(const DevOp<float> &op, int tile, float omega, const float2 *b, const float2 *u_in,
                                  float2 *u_out, const float2 *ec, cudaStream_t s);
 
-// Fused coarse tail: Algorithm 1 on levels 0..nlev-1 of the given arrays (level 0 = the
-// tail's top, nlev - 1 = the coarsest, solved with minv) inside one thread block.  zero: the
-// top-level iterate u[0] starts at 0 (not read).  Levels with at most TAIL_MAX_UNKNOWNS
-// interior nodes, MAX_TAIL_LEVELS at most, go to the tail.
-constexpr int MAX_TAIL_LEVELS = 4;
-constexpr int TAIL_MAX_UNKNOWNS = 4096;
-constexpr size_t TAIL_SMEM_BYTES = 200 * 1024;  // b, u, t of every tail level in shared memory
-// Dynamic shared memory of the fused tail: the coarsest solve's compact right-hand side
-// (nu_c values, rounded up to even), b, u, t of every tail level, then every tail level's
-// coefficient triples and k^2 (each k^2 array padded to 16 bytes).
-inline size_t mg_tail_smem_bytes_nodes(int dim, int nlev, const int (*n)[3], int nu_c, size_t es) {
-    size_t bytes = (size_t)((nu_c + 1) & ~1) * es;
-    for (int l = 0; l < nlev; l++) {
-        const size_t np = (size_t)n[l][0] * n[l][1] * (dim == 3 ? n[l][2] : 1);
-        bytes += 3 * es * np;                                                  // b, u, t
-        bytes += 3 * es * (size_t)(n[l][0] + n[l][1] + (dim == 3 ? n[l][2] : 0));  // coefficients
-        bytes += (np * (es / 2) + 15) & ~(size_t)15;                           // k^2
-    }
-    return bytes;
-}
-template <typename R>
-inline size_t mg_tail_smem_bytes(int dim, int nlev, const DevOp<R> *ops, int nu_c, size_t es) {
-    int n[MAX_TAIL_LEVELS][3];
-    for (int l = 0; l < nlev && l < MAX_TAIL_LEVELS; l++)
-        for (int a = 0; a < 3; a++) n[l][a] = ops[l].n[a];
-    return mg_tail_smem_bytes_nodes(dim, nlev < MAX_TAIL_LEVELS ? nlev : MAX_TAIL_LEVELS, n, nu_c, es);
-}
-template <typename R>
-cudaError_t launch_mg_tail(int dim, int nlev, const DevOp<R> *ops, typename CT<R>::T *const *b,
-                           typename CT<R>::T *const *u, typename CT<R>::T *const *t, const typename CT<R>::T *minv,
-                           int nu_c, int nu1, int nu2, int rb, R omega, int gf, int gc, int zero, cudaStream_t s);
-// Cluster tail (kernels_ctail.cu): the coarsest nlev levels of a 2D complex64 cycle in one
-// launch of a cluster of nc = 8 or 16 thread blocks, every level in distributed shared memory
-// (rows split into slabs).  b_top / u_top: the first of those levels' right-hand side and result
-// (global; u_top is the initial guess unless zero).
+// Fused coarse tail (kernels_ctail.cu): Algorithm 1 on the coarsest nlev levels in one launch of a
+// cluster of nc = 8 or 16 thread blocks, every level in distributed shared memory (rows -- grid
+// lines in 2D, planes in 3D -- split into slabs).  b_top / u_top: the first of those levels'
+// right-hand side and result (global; u_top is the initial guess unless zero).
 constexpr int MAX_CT_LEVELS = 6;
 constexpr int MAX_CT_BLOCKS = 16;      // blocks per cluster at most
 constexpr int CT_BLOCK_THREADS = 512;  // threads per block of a cluster tail
 constexpr size_t CT_SMEM_BYTES = 200 * 1024;
+// Largest level (interior nodes) of the fused tail where the tuning names no depth: below it the
+// cluster (16 of the 152 SMs) is faster than a launch per phase over the whole GPU.  Measured per
+// cycle on GB300 with the level above the line in / out of the tail: 2D complex64 129^2 24.7 / 27.2
+// us (V(2,2) on 129^2) but 161^2 30.3 / 27.4; 2D complex128 81^2 86 / 106 us (161^2), 129^2 does not
+// fit; 3D 21^3 43.1 / 45.9 us complex64 and 235 / 317 us complex128 (41^3), but 25^3 47.2 / 46.3.
+constexpr int tail_max_unknowns(int dim, size_t es) { return dim == 2 && es == sizeof(float2) ? 16384 : 8192; }
 // Nested row slabs of the tail levels: block r owns the interior rows B[l][r] .. B[l][r+1]-1 of
-// level l (level 0 in runs of ceil((ny - 2) / nc) rows, B[l+1][r] = (B[l][r] + 1) / 2).  False
-// unless every level has odd ny and the next has (ny + 1) / 2.
-bool mg_ctail_bounds(int nlev, const int (*n)[3], int nc, int (*B)[MAX_CT_BLOCKS + 1]);
+// level l (level 0 in runs of ceil((rows - 2) / nc), B[l+1][r] = (B[l][r] + 1) / 2).  False
+// unless every level but the last has an odd number of rows and the next has half of them.
+bool mg_ctail_bounds(int dim, int nlev, const int (*n)[3], int nc, int (*B)[MAX_CT_BLOCKS + 1]);
 // Rows of the coarsest inverse each warp stages in the dense phase, and their shared-memory
-// bytes (0 when above 64 KB: the rows are then read from global memory).
+// bytes (0 when above 64 KB: the rows are then read from global memory); es: bytes of a value.
 int mg_ctail_minv_rows(int nc, int nu_c);
-size_t mg_ctail_minv_stage_bytes(int nc, int nu_c);
-size_t mg_ctail_layout(int nlev, const int (*n)[3], int nc, int nu_c, unsigned (*off)[7], unsigned *obc,
-                       unsigned *ominv);
-// img: the blocks' initial shared memory from build_mg_ctail_image for the same levels and nc
+size_t mg_ctail_minv_stage_bytes(int nc, int nu_c, size_t es);
+size_t mg_ctail_layout(int dim, size_t es, int nlev, const int (*n)[3], int nc, int nu_c, unsigned (*off)[8],
+                       unsigned *obc, unsigned *ominv);
+// img: the blocks' initial shared memory from build_mg_ctail_image for the same levels, omega and nc
 // (null: each launch builds it itself); *out is device memory the caller frees.
-cudaError_t launch_mg_ctail(int nlev, const DevOp<float> *ops, const float2 *b_top, float2 *u_top,
-                            const float2 *minv, int nu_c, int nu1, int nu2, int rb, float omega, int zero, int gf,
-                            int gc, int nc, const void *img, cudaStream_t s);
-cudaError_t build_mg_ctail_image(int nlev, const DevOp<float> *ops, const float2 *minv, int nu_c, int nc, void **out,
-                                 cudaStream_t s);
-int mg_ctail_max_clusters(int nc, size_t bytes);
+template <typename R>
+cudaError_t launch_mg_ctail(int dim, int nlev, const DevOp<R> *ops, const typename CT<R>::T *b_top,
+                            typename CT<R>::T *u_top, const typename CT<R>::T *minv, int nu_c, int nu1, int nu2, int rb,
+                            R omega, int zero, int gf, int gc, int nc, const void *img, cudaStream_t s);
+template <typename R>
+cudaError_t build_mg_ctail_image(int dim, int nlev, const DevOp<R> *ops, const typename CT<R>::T *minv, int nu_c,
+                                 R omega, int nc, void **out, cudaStream_t s);
+template <typename R> int mg_ctail_max_clusters(int dim, int nc, size_t bytes);
 // Deep-halo cluster tail (kernels_chalo.cu): the same levels for a V-cycle of omega-Jacobi with
 // nu1, nu2 <= 2 sweeps from a zero guess, each block keeping three rows beyond its slab so that
 // each level needs one cluster barrier down and one up.  img (required): the blocks' initial

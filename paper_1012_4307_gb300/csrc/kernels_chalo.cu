@@ -414,7 +414,8 @@ size_t mg_chalo_layout(int nlev, const int (*n)[3], int nc, int nu_c, unsigned (
                        unsigned *ominv) {
     auto al = [](size_t b) { return (b + 15) & ~(size_t)15; };
     int B[MAX_CT_LEVELS][MAX_CT_BLOCKS + 1];
-    if (nlev < 2 || nlev > MAX_CT_LEVELS || !mg_ctail_bounds(nlev, n, nc, B)) return ~(size_t)0;
+    if (nlev < 2 || nlev > MAX_CT_LEVELS || n[nlev - 1][1] % 2 == 0 || !mg_ctail_bounds(2, nlev, n, nc, B))
+        return ~(size_t)0;
     size_t p = 0;
     for (int l = 0; l < nlev; l++) {
         const int nx = n[l][0];
@@ -441,7 +442,7 @@ size_t mg_chalo_layout(int nlev, const int (*n)[3], int nc, int nu_c, unsigned (
     *obc = (unsigned)p;
     p += al((size_t)nu_c * sizeof(float2));
     *ominv = (unsigned)p;
-    p += al(mg_ctail_minv_stage_bytes(nc, nu_c));
+    p += al(mg_ctail_minv_stage_bytes(nc, nu_c, sizeof(float2)));
     return p;
 }
 
@@ -455,7 +456,7 @@ static size_t chalo_args(int nlev, const DevOp<float> *ops, const float2 *minv, 
     const size_t bytes = mg_chalo_layout(nlev, n, nc, nu_c, off, &obc, &ominv);
     if (bytes > CT_SMEM_BYTES) return 0;
     int B[MAX_CT_LEVELS][MAX_CT_BLOCKS + 1];
-    if (!mg_ctail_bounds(nlev, n, nc, B)) return 0;
+    if (!mg_ctail_bounds(2, nlev, n, nc, B)) return 0;
     A = HArgs{};
     for (int l = 0; l < nlev; l++) {
         HLevel &L = A.lv[l];
@@ -475,7 +476,7 @@ static size_t chalo_args(int nlev, const DevOp<float> *ops, const float2 *minv, 
     A.minv = minv;
     A.obc = obc;
     A.ominv = ominv;
-    A.mrow = mg_ctail_minv_stage_bytes(nc, nu_c) ? mg_ctail_minv_rows(nc, nu_c) : 0;
+    A.mrow = mg_ctail_minv_stage_bytes(nc, nu_c, sizeof(float2)) ? mg_ctail_minv_rows(nc, nu_c) : 0;
     A.total = (unsigned)bytes;
     return bytes;
 }

@@ -37,32 +37,25 @@ template <typename R> __host__ __device__ OpView<R> view(const DevOp<R> &op) {
     return v;
 }
 
-// Coefficient load: the read-only global path (ld.global.nc) for operators in global memory,
-// a plain (generic) load when the operator's arrays may live in shared memory.
-template <bool GLOBAL, typename T> __device__ __forceinline__ T ldc(const T *p) {
-    if constexpr (GLOBAL) return __ldg(p);
-    else return *p;
-}
-
 // Off-diagonal part of the stencil at p (neighbours along x and y; z handled by callers that
-// march in k) and the diagonal entry.  GLOBAL: the coefficient arrays are in global memory.
-template <typename R, int DIM, typename CX, bool GLOBAL = true>
+// march in k) and the diagonal entry.
+template <typename R, int DIM, typename CX>
 __device__ __forceinline__ typename CT<R>::T stencil(const OpView<R> &o, const CX *__restrict__ x, size_t p,
                                                     int i, int j, int k, typename CT<R>::T xm_z,
                                                     typename CT<R>::T xc, typename CT<R>::T xp_z,
                                                     typename CT<R>::T &diag) {
     typedef typename CT<R>::T C;
     const size_t sy = (size_t)o.nx;
-    C cw = ldc<GLOBAL>(&o.cx[3 * i]), cc = ldc<GLOBAL>(&o.cx[3 * i + 1]), ce = ldc<GLOBAL>(&o.cx[3 * i + 2]);
+    C cw = __ldg(&o.cx[3 * i]), cc = __ldg(&o.cx[3 * i + 1]), ce = __ldg(&o.cx[3 * i + 2]);
     C acc = cmul(cw, to_c(x[p - 1], R()));
     acc = cfma(ce, to_c(x[p + 1], R()), acc);
     C d = cc;
-    cw = ldc<GLOBAL>(&o.cy[3 * j]); cc = ldc<GLOBAL>(&o.cy[3 * j + 1]); ce = ldc<GLOBAL>(&o.cy[3 * j + 2]);
+    cw = __ldg(&o.cy[3 * j]); cc = __ldg(&o.cy[3 * j + 1]); ce = __ldg(&o.cy[3 * j + 2]);
     acc = cfma(cw, to_c(x[p - sy], R()), acc);
     acc = cfma(ce, to_c(x[p + sy], R()), acc);
     d = cadd(d, cc);
     if (DIM == 3) {
-        cw = ldc<GLOBAL>(&o.cz[3 * k]); cc = ldc<GLOBAL>(&o.cz[3 * k + 1]); ce = ldc<GLOBAL>(&o.cz[3 * k + 2]);
+        cw = __ldg(&o.cz[3 * k]); cc = __ldg(&o.cz[3 * k + 1]); ce = __ldg(&o.cz[3 * k + 2]);
         acc = cfma(cw, xm_z, acc);
         acc = cfma(ce, xp_z, acc);
         d = cadd(d, cc);
@@ -73,7 +66,7 @@ __device__ __forceinline__ typename CT<R>::T stencil(const OpView<R> &o, const C
 }
 
 // (M x)_p for a point whose z neighbours are loaded here (used by the restriction kernel).
-template <typename R, int DIM, typename CX, bool GLOBAL = true>
+template <typename R, int DIM, typename CX>
 __device__ __forceinline__ typename CT<R>::T apply_point(const OpView<R> &o, const CX *__restrict__ x, int i, int j,
                                                         int k, typename CT<R>::T &diag) {
     typedef typename CT<R>::T C;
@@ -81,7 +74,7 @@ __device__ __forceinline__ typename CT<R>::T apply_point(const OpView<R> &o, con
     const size_t p = (size_t)i + (size_t)o.nx * ((size_t)j + (size_t)o.ny * k);
     C xm = mk(R(0), R(0)), xp = mk(R(0), R(0));
     if (DIM == 3) { xm = to_c(x[p - sz], R()); xp = to_c(x[p + sz], R()); }
-    return stencil<R, DIM, CX, GLOBAL>(o, x, p, i, j, k, xm, to_c(x[p], R()), xp, diag);
+    return stencil<R, DIM, CX>(o, x, p, i, j, k, xm, to_c(x[p], R()), xp, diag);
 }
 
 // Thread preamble: interior (i, j) and the k range of this thread.
@@ -789,265 +782,6 @@ __global__ void __launch_bounds__(Tile<TCX, TCY>::NT, 4) k_prolong_post2_b(const
                                  (o.ny + 1) / 2, blockIdx.x, blockIdx.y);
 }
 
-// ------------------------------------------------------------------------------ coarse tail
-// The coarse levels of a cycle (a few thousand unknowns or fewer) are launch- and latency-
-// bound when every sweep is its own grid.  k_mg_tail runs Algorithm 1 from the tail's top
-// level down to the exact coarsest solve and back inside ONE thread block, with every level's
-// b, u, t in shared memory (the host picks the tail depth so they fit): the top level's
-// right-hand side is copied in, its result copied out (interior nodes only).  Phases are
-// block-wide loops (warps over grid rows, lanes over x) separated by __syncthreads().  Same
-// arithmetic as the per-level kernels.
-constexpr int TAIL_THREADS = 512;
-
-template <typename R> struct TailLevelDev {
-    OpView<R> o;
-    typename CT<R>::T *b, *u, *t;
-};
-
-template <typename R> struct TailArgs {
-    TailLevelDev<R> lv[MAX_TAIL_LEVELS];
-    int nlev, nu_c, nu1, nu2, rb;
-    R omega;
-    const typename CT<R>::T *minv;
-    typename CT<R>::T *bc;  // compact right-hand side of the coarsest solve (shared memory)
-};
-
-// f(i, j, k) for every interior node of a level; warps take rows (j, k), lanes take i.
-template <int DIM, typename F>
-__device__ __forceinline__ void for_interior(int nx, int ny, int nz, F f) {
-    const int mx = nx - 2, my = ny - 2, rows = my * (DIM == 3 ? nz - 2 : 1);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int r = warp; r < rows; r += nw) {
-        const int j = 1 + (DIM == 3 ? r % my : r);
-        const int k = DIM == 3 ? 1 + r / my : 0;
-        for (int i = 1 + lane; i <= mx; i += 32) f(i, j, k);
-    }
-}
-
-template <typename R, int DIM>
-__device__ void tail_smooth(const TailArgs<R> &A, const TailLevelDev<R> &L, int sweeps, typename CT<R>::T **cur,
-                            typename CT<R>::T **oth, bool zero) {
-    typedef typename CT<R>::T C;
-    const OpView<R> &o = L.o;
-    const size_t sz = (size_t)o.nx * o.ny;
-    auto at = [&](int i, int j, int k) { return (size_t)i + (size_t)o.nx * ((size_t)j + (size_t)o.ny * k); };
-    if (zero && (sweeps == 0 || A.rb)) {
-        C *u = *cur;
-        for_interior<DIM>(o.nx, o.ny, o.nz, [&](int i, int j, int k) { u[at(i, j, k)] = mk(R(0), R(0)); });
-        __syncthreads();
-    }
-    for (int s = 0; s < sweeps; s++) {
-        if (A.rb) {
-            for (int colour = 0; colour < 2; colour++) {
-                C *u = *cur;
-                for_interior<DIM>(o.nx, o.ny, o.nz, [&](int i, int j, int k) {
-                    if (((i + j + k) & 1) != colour) return;
-                    const size_t p = at(i, j, k);
-                    C xm = mk(R(0), R(0)), xp = mk(R(0), R(0));
-                    if (DIM == 3) { xm = u[p - sz]; xp = u[p + sz]; }
-                    const C xc = u[p];
-                    C d;
-                    const C mu = stencil<R, DIM, C, false>(o, u, p, i, j, k, xm, xc, xp, d);
-                    u[p] = cadd(xc, cscale(cmul(csub(L.b[p], mu), cinv(d)), A.omega));
-                });
-                __syncthreads();
-            }
-        } else {
-            const bool z0 = zero && s == 0;
-            const C *u = *cur;
-            C *un = *oth;
-            for_interior<DIM>(o.nx, o.ny, o.nz, [&](int i, int j, int k) {
-                const size_t p = at(i, j, k);
-                if (z0) {
-                    C d = cadd(cadd(o.cx[3 * i + 1], o.cy[3 * j + 1]), cadd(cscale(o.bk, o.k2[p]), o.c));
-                    if (DIM == 3) d = cadd(d, o.cz[3 * k + 1]);
-                    un[p] = cscale(cmul(L.b[p], cinv(d)), A.omega);
-                } else {
-                    C xm = mk(R(0), R(0)), xp = mk(R(0), R(0));
-                    if (DIM == 3) { xm = u[p - sz]; xp = u[p + sz]; }
-                    const C xc = u[p];
-                    C d;
-                    const C mu = stencil<R, DIM, C, false>(o, u, p, i, j, k, xm, xc, xp, d);
-                    un[p] = cadd(xc, cscale(cmul(csub(L.b[p], mu), cinv(d)), A.omega));
-                }
-            });
-            __syncthreads();
-            C *t = *cur;
-            *cur = *oth;
-            *oth = t;
-        }
-    }
-}
-
-// Exact coarsest solve u = Minv b: gather b's unknowns (natural order) into a compact array,
-// one warp per row of Minv (coalesced, 8 loads in flight per lane), scatter the rows.
-template <typename R, int DIM>
-__device__ void tail_dense(const TailArgs<R> &A, const TailLevelDev<R> &L) {
-    typedef typename CT<R>::T C;
-    const int mx = L.o.nx - 2, my = L.o.ny - 2, nu = A.nu_c;
-    auto node = [&](int c) {
-        const int i = 1 + c % mx, j = 1 + (c / mx) % my, k = DIM == 3 ? 1 + c / (mx * my) : 0;
-        return (size_t)i + (size_t)L.o.nx * ((size_t)j + (size_t)L.o.ny * k);
-    };
-    for (int c = threadIdx.x; c < nu; c += blockDim.x) A.bc[c] = L.b[node(c)];
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    for (int row = warp; row < nu; row += nwarp) {
-        const C *mrow = A.minv + (size_t)row * nu;
-        C acc = mk(R(0), R(0));
-#pragma unroll 8
-        for (int c = lane; c < nu; c += 32) acc = cfma(mrow[c], A.bc[c], acc);
-        for (int off = 16; off > 0; off >>= 1) {
-            acc.x += __shfl_down_sync(0xffffffffu, acc.x, off);
-            acc.y += __shfl_down_sync(0xffffffffu, acc.y, off);
-        }
-        if (lane == 0) L.u[node(row)] = acc;
-    }
-    __syncthreads();
-}
-
-// Level LVL of the tail (compile-time depth, so no device recursion and no stack growth).
-template <typename R, int DIM, int LVL>
-__device__ void tail_cycle(const TailArgs<R> &A, bool zero, int gf, int gc) {
-    typedef typename CT<R>::T C;
-    constexpr int l = LVL;
-    const TailLevelDev<R> &L = A.lv[l];
-    if (l == A.nlev - 1) {
-        tail_dense<R, DIM>(A, L);
-        return;
-    }
-    if constexpr (LVL + 1 < MAX_TAIL_LEVELS) {
-    C *cur = L.u, *oth = L.t;
-    tail_smooth<R, DIM>(A, L, A.nu1, &cur, &oth, zero);
-    const TailLevelDev<R> &Lc = A.lv[l + 1];
-    // residual + full weighting into the next level's right-hand side
-    {
-        const C *uc = cur;
-        for_interior<DIM>(Lc.o.nx, Lc.o.ny, Lc.o.nz, [&](int I, int J, int K) {
-            C acc = mk(R(0), R(0));
-            for (int dk = (DIM == 3 ? -1 : 0); dk <= (DIM == 3 ? 1 : 0); dk++) {
-                const R wk = DIM == 3 ? (dk == 0 ? R(0.5) : R(0.25)) : R(1);
-                const int k = DIM == 3 ? 2 * K + dk : 0;
-#pragma unroll
-                for (int dj = -1; dj <= 1; dj++) {
-                    const R wj = wk * (dj == 0 ? R(0.5) : R(0.25));
-                    const int j = 2 * J + dj;
-#pragma unroll
-                    for (int di = -1; di <= 1; di++) {
-                        const R w = wj * (di == 0 ? R(0.5) : R(0.25));
-                        const int i = 2 * I + di;
-                        const size_t p = (size_t)i + (size_t)L.o.nx * ((size_t)j + (size_t)L.o.ny * k);
-                        C d;
-                        const C mu = apply_point<R, DIM, C, false>(L.o, uc, i, j, k, d);
-                        acc = cadd(acc, cscale(csub(L.b[p], mu), w));
-                    }
-                }
-            }
-            Lc.b[(size_t)I + (size_t)Lc.o.nx * ((size_t)J + (size_t)Lc.o.ny * K)] = acc;
-        });
-        __syncthreads();
-    }
-    if (l + 1 == A.nlev - 1) {
-        tail_dense<R, DIM>(A, Lc);
-    } else {
-        for (int i = 1; i <= gc; i++) {
-            if (i == 1) tail_cycle<R, DIM, LVL + 1>(A, true, gf, gc);
-            else tail_cycle<R, DIM, LVL + 1>(A, false, gc, gf);
-        }
-    }
-    // prolongation + correction
-    {
-        const int nx = L.o.nx, ny = L.o.ny, ncx = Lc.o.nx, ncy = Lc.o.ny;
-        C *uf = cur;
-        for_interior<DIM>(nx, ny, L.o.nz, [&](int i, int j, int k) {
-            const int kk0 = DIM == 3 ? k >> 1 : 0, kk1 = DIM == 3 ? (k + 1) >> 1 : 0;
-            C acc = mk(R(0), R(0));
-            int cnt = 0;
-            for (int kk = kk0; kk <= kk1; kk++)
-                for (int jj = j >> 1; jj <= (j + 1) >> 1; jj++)
-                    for (int ii = i >> 1; ii <= (i + 1) >> 1; ii++) {
-                        acc = cadd(acc, Lc.u[(size_t)ii + (size_t)ncx * ((size_t)jj + (size_t)ncy * kk)]);
-                        cnt++;
-                    }
-            const size_t p = (size_t)i + (size_t)nx * ((size_t)j + (size_t)ny * k);
-            uf[p] = cadd(uf[p], cscale(acc, R(1) / R(cnt)));
-        });
-        __syncthreads();
-    }
-    tail_smooth<R, DIM>(A, L, A.nu2, &cur, &oth, false);
-    if (cur != L.u) {
-        const C *src = cur;
-        for_interior<DIM>(L.o.nx, L.o.ny, L.o.nz, [&](int i, int j, int k) {
-            const size_t p = (size_t)i + (size_t)L.o.nx * ((size_t)j + (size_t)L.o.ny * k);
-            L.u[p] = src[p];
-        });
-        __syncthreads();
-    }
-    }  // LVL + 1 < MAX_TAIL_LEVELS
-}
-
-// Dynamic shared memory: [compact coarsest rhs | per level: b, u, t | per level: coefficient
-// triples, k^2].  A.lv[0].b / u hold the
-// caller's global top-level vectors; zero != 0 means the top-level iterate starts at 0.
-template <typename R, int DIM>
-__global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail(TailArgs<R> A, int gf, int gc, int zero) {
-    pdl_enter();
-    typedef typename CT<R>::T C;
-    extern __shared__ __align__(16) unsigned char tail_smem[];
-    __shared__ TailArgs<R> S;
-    if (threadIdx.x == 0) {
-        S = A;
-        C *p = (C *)tail_smem;
-        S.bc = p;
-        p += (A.nu_c + 1) & ~1;
-        for (int l = 0; l < A.nlev; l++) {
-            const size_t np = (size_t)A.lv[l].o.nx * A.lv[l].o.ny * (DIM == 3 ? A.lv[l].o.nz : 1);
-            S.lv[l].b = p; p += np;
-            S.lv[l].u = p; p += np;
-            S.lv[l].t = p; p += np;
-        }
-        // then every level's coefficient triples and k^2 (read by every phase)
-        for (int l = 0; l < A.nlev; l++) {
-            OpView<R> &o = S.lv[l].o;
-            const size_t np = (size_t)o.nx * o.ny * (DIM == 3 ? o.nz : 1);
-            o.cx = p; p += 3 * o.nx;
-            o.cy = p; p += 3 * o.ny;
-            if (DIM == 3) { o.cz = p; p += 3 * o.nz; }
-            o.k2 = (const R *)p;
-            p = (C *)((unsigned char *)p + ((np * sizeof(R) + 15) & ~(size_t)15));
-        }
-    }
-    __syncthreads();
-    {
-        const TailLevelDev<R> &last = S.lv[S.nlev - 1];
-        const C *end = last.t + (size_t)last.o.nx * last.o.ny * (DIM == 3 ? last.o.nz : 1);
-        const size_t total = end - (const C *)tail_smem;
-        for (size_t q = threadIdx.x; q < total; q += blockDim.x) ((C *)tail_smem)[q] = mk(R(0), R(0));
-        for (int l = 0; l < S.nlev; l++) {
-            const OpView<R> &g = A.lv[l].o, &o = S.lv[l].o;
-            const size_t np = (size_t)g.nx * g.ny * (DIM == 3 ? g.nz : 1);
-            for (int q = threadIdx.x; q < 3 * g.nx; q += blockDim.x) const_cast<C *>(o.cx)[q] = g.cx[q];
-            for (int q = threadIdx.x; q < 3 * g.ny; q += blockDim.x) const_cast<C *>(o.cy)[q] = g.cy[q];
-            if (DIM == 3)
-                for (int q = threadIdx.x; q < 3 * g.nz; q += blockDim.x) const_cast<C *>(o.cz)[q] = g.cz[q];
-            for (size_t q = threadIdx.x; q < np; q += blockDim.x) const_cast<R *>(o.k2)[q] = g.k2[q];
-        }
-    }
-    __syncthreads();
-    const OpView<R> &o = A.lv[0].o;
-    for_interior<DIM>(o.nx, o.ny, o.nz, [&](int i, int j, int k) {
-        const size_t p = (size_t)i + (size_t)o.nx * ((size_t)j + (size_t)o.ny * k);
-        S.lv[0].b[p] = A.lv[0].b[p];
-        if (!zero) S.lv[0].u[p] = A.lv[0].u[p];
-    });
-    __syncthreads();
-    tail_cycle<R, DIM, 0>(S, zero != 0, gf, gc);
-    for_interior<DIM>(o.nx, o.ny, o.nz, [&](int i, int j, int k) {
-        const size_t p = (size_t)i + (size_t)o.nx * ((size_t)j + (size_t)o.ny * k);
-        A.lv[0].u[p] = S.lv[0].u[p];
-    });
-}
-
 // Planes per thread of a 3D z-marching kernel: kmax, halved while the grid would have fewer than
 // `target` blocks (small levels: more, shorter chains instead of a few long ones).
 static int z_chunk(size_t tiles_xy, int planes, int kmax, size_t target) {
@@ -1164,46 +898,6 @@ cudaError_t launch_dense_solve(const int n[3], int dim, int nu, const typename C
     launch_pdl(k_dense_solve<R>, cdiv(nu, warps), threads, 0, s, n[0], n[1], dim == 3 ? n[2] : 1, dim, nu, minv, b, u);
     return cudaGetLastError();
 }
-
-template <typename R>
-cudaError_t launch_mg_tail(int dim, int nlev, const DevOp<R> *ops, typename CT<R>::T *const *b,
-                           typename CT<R>::T *const *u, typename CT<R>::T *const *t, const typename CT<R>::T *minv,
-                           int nu_c, int nu1, int nu2, int rb, R omega, int gf, int gc, int zero, cudaStream_t s) {
-    if (nlev < 2 || nlev > MAX_TAIL_LEVELS) return cudaErrorInvalidValue;
-    TailArgs<R> A{};
-    for (int l = 0; l < nlev; l++) {
-        A.lv[l].o = view(ops[l]);
-        if (dim != 3) A.lv[l].o.nz = 1;
-        A.lv[l].b = b[l];
-        A.lv[l].u = u[l];
-        A.lv[l].t = t[l];
-    }
-    A.nlev = nlev;
-    A.nu_c = nu_c;
-    A.nu1 = nu1;
-    A.nu2 = nu2;
-    A.rb = rb;
-    A.omega = omega;
-    A.minv = minv;
-    const size_t bytes = mg_tail_smem_bytes(dim, nlev, ops, nu_c, sizeof(typename CT<R>::T));
-    if (bytes > TAIL_SMEM_BYTES) return cudaErrorInvalidValue;
-    static bool attr_set[2] = {false, false};
-    if (!attr_set[dim == 3]) {
-        cudaError_t e = dim == 3 ? cudaFuncSetAttribute(k_mg_tail<R, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TAIL_SMEM_BYTES)
-                                 : cudaFuncSetAttribute(k_mg_tail<R, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TAIL_SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        attr_set[dim == 3] = true;
-    }
-    if (dim == 3) launch_pdl(k_mg_tail<R, 3>, 1, TAIL_THREADS, bytes, s, A, gf, gc, zero);
-    else launch_pdl(k_mg_tail<R, 2>, 1, TAIL_THREADS, bytes, s, A, gf, gc, zero);
-    return cudaGetLastError();
-}
-template cudaError_t launch_mg_tail<float>(int, int, const DevOp<float> *, float2 *const *, float2 *const *,
-                                           float2 *const *, const float2 *, int, int, int, int, float, int, int, int,
-                                           cudaStream_t);
-template cudaError_t launch_mg_tail<double>(int, int, const DevOp<double> *, double2 *const *, double2 *const *,
-                                            double2 *const *, const double2 *, int, int, int, int, double, int, int,
-                                            int, cudaStream_t);
 
 // Tile shapes (coarse nodes per block) of the temporally blocked kernels, by tile index (the
 // wavefront, HELM_TILE_WAVE, has none).

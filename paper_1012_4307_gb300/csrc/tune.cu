@@ -49,7 +49,7 @@ extern "C" helm_status helm_set_tuning(helm_handle *h, const helm_tuning *t) {
         return helm_fail(HELM_ERR_ARG, "invalid tuning (tail or cluster levels, cluster blocks or halo, or a tile)");
     h->tune = *t;
     helm_drop_graphs(h);
-    ctail_image(h, true, ctail_deep(h));
+    helm_refresh_tails(h, true);
     return HELM_OK;
 }
 
@@ -89,7 +89,7 @@ extern "C" helm_status helm_autotune(helm_handle *h, helm_prec prec, int reps, h
     // skipped
     auto time_it = [&](const helm_tuning &t, bool soft = false) -> double {
         h->tune = t;
-        ctail_image(h, true, ctail_deep(h));
+        helm_refresh_tails(h, true);
         cudaStream_t keep_s = h->stream;
         cudaGraph_t g = nullptr;
         cudaGraphExec_t ge = nullptr;
@@ -132,7 +132,7 @@ extern "C" helm_status helm_autotune(helm_handle *h, helm_prec prec, int reps, h
     helm_tuning cur = keep;
     double cur_ms = 0.0;
     const int last = (int)h->lv.size() - 1;
-    const int built = c64 ? h->tail_top32 : h->tail_top64;
+    const int built = h->tail_built[c64 ? 0 : 1];
     const int max_tail = built < 0 ? 0 : last - built + 1;
     const bool blockable = c64 && h->dim == 2 && h->mg.smoother == HELM_SMOOTH_JACOBI && h->mg.nu1 == 2 &&
                            h->mg.nu2 == 2;
@@ -161,8 +161,9 @@ extern "C" helm_status helm_autotune(helm_handle *h, helm_prec prec, int reps, h
                     ops[q] = h->lv[last - cl + 1 + q].M32;
                     for (int a = 0; a < 3; a++) n[q][a] = ops[q].n[a];
                 }
-                unsigned off[MAX_CT_LEVELS][7], obc, oz;
-                if (mg_ctail_max_clusters(nc, mg_ctail_layout(cl, n, nc, h->nu_c, off, &obc, &oz)) < 1) continue;
+                unsigned off[MAX_CT_LEVELS][8], obc, oz;
+                const size_t bytes = mg_ctail_layout(2, sizeof(float2), cl, n, nc, h->nu_c, off, &obc, &oz);
+                if (mg_ctail_max_clusters<float>(2, nc, bytes) < 1) continue;
                 const size_t deep_bytes = vj2 ? mg_chalo_bytes(cl, ops, h->nu_c, nc) : 0;
                 for (int halo : {1, 3}) {
                     if (cl == cur.cluster_levels && nc == cur.cluster_ctas && halo == cur.cluster_halo) continue;
@@ -201,11 +202,8 @@ extern "C" helm_status helm_autotune(helm_handle *h, helm_prec prec, int reps, h
         // per level above the tails, greedily from the finest: separate launches or a tile shape
         if (blockable) {
             h->tune = cur;
-            const int top = tail_top<float>(h), ctop = ctail_top(h);
-            int stop = last;
-            if (top >= 0) stop = std::min(stop, top);
-            if (ctop >= 0) stop = std::min(stop, ctop);
-            stop = std::min(stop, HELM_MAX_LEVELS);
+            helm_refresh_tails(h, false);
+            const int stop = std::min(h->tail[0].top >= 0 ? h->tail[0].top : last, HELM_MAX_LEVELS);
             for (int l = 0; l < stop && st == HELM_OK; l++) {
                 for (int tile = HELM_TILE_NONE; tile < HELM_TILE_COUNT && st == HELM_OK; tile++) {
                     if (tile == cur.level_tile[l]) continue;
@@ -227,7 +225,7 @@ extern "C" helm_status helm_autotune(helm_handle *h, helm_prec prec, int reps, h
     h->prof.on = prof;
     h->tune = st == HELM_OK ? cur : keep;
     helm_drop_graphs(h);
-    ctail_image(h, true, ctail_deep(h));
+    helm_refresh_tails(h, true);
     if (st != HELM_OK) return st;
     if (best) *best = cur;
     if (best_ms) *best_ms = cur_ms;

@@ -1,0 +1,56 @@
+"""Kernels that are chosen by size, precision or smoother, at the edges of their ranges, against the
+oracle's cycle: the same bounds as the per-level kernels (1e-12 in complex128: a cycle's roundings
+amplified by the coarsest solve; 2e-5 in complex64)."""
+import numpy as np
+import pytest
+
+from helpers import gpu_handle, oracle_pair, rel_l2, to_gpu, to_np
+from paper_1012_4307_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+TOL = {"c128": 1e-12, "c64": 2e-5}
+
+
+@pytest.fixture(scope="module")
+def helm():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1012_4307_gb300 import helm as H
+    H.load()
+    return H
+
+
+def problem(n, coarsest_n):
+    """Nodes n per axis (x first); k^2 cut from the square or cubic well field."""
+    dim = len(n)
+    k2 = W.k2_well_growth(dim, max(n), kh_max=0.5)[tuple(slice(0, m) for m in reversed(n))]
+    shape = tuple(reversed(n))
+    return W.Problem("paths", dim, list(n), np.ascontiguousarray(k2), np.zeros(shape, complex), coarsest_n=coarsest_n)
+
+
+def check_cycle(helm, oracle, n, coarsest_n, prec, smoother, nu, gamma, tunings=({},)):
+    P = problem(n, coarsest_n)
+    h = gpu_handle(helm, P, pc="csg", prec=prec, smoother=smoother, nu=nu, gamma=gamma)
+    A, M = oracle_pair(oracle, P)
+    v = W.random_field(tuple(reversed(n)), 51)
+    ref = oracle.MG(M, coarsest_n, nu[0], nu[1], 0.8, smoother).cycle(v, None, *gamma)
+    dtype = torch.complex64 if prec == "c64" else torch.complex128
+    for t in tunings:
+        if t:
+            helm.helm_set_tuning(h, t)
+        z = helm.mg_precondition(h, to_gpu(v), dtype)
+        assert rel_l2(to_np(z), ref) <= TOL[prec], t
+
+
+@pytest.mark.parametrize("prec", ["c64", "c128"])
+@pytest.mark.parametrize("smoother,nu,gamma", [("jacobi", (2, 2), (1, 1)), ("jacobi", (1, 2), (1, 3)),
+                                               ("rb", (1, 1), (2, 2)), ("jacobi", (0, 1), (1, 1))])
+@pytest.mark.parametrize("n,coarsest_n", [((65, 65), 17), ((81, 41), 17), ((41, 81), 11), ((43, 35), 21),
+                                          ((17, 17, 17), 9), ((21, 13, 17), 6), ((13, 21, 33), 9)])
+def test_fused_tail_any_cycle(helm, oracle, n, coarsest_n, prec, smoother, nu, gamma):
+    """The coarse tail on a thread-block cluster at every depth: lines and planes as rows, more
+    blocks than rows, coarsest grids with an even number of rows, red-black and F / W cycles."""
+    check_cycle(helm, oracle, n, coarsest_n, prec, smoother, nu, gamma, [dict(tail_levels=t) for t in (-1, 2, 3, 4, 0)])
