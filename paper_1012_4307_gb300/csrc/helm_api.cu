@@ -308,8 +308,14 @@ helm_status helm_create_impl(const helm_grid *grid, double theta, const double *
         if (dim == 2) {  // 1 / diagonal for the temporally blocked smoothers
             float2 *di = nullptr;
             CKC(dalloc(&di, L.np, h->owned));
-            CKC(launch_diag_inv(L.M32, di, s));
+            CKC(launch_diag_inv<float>(L.M32, dim, (float)mg->omega, di, s));
             L.M32.dinv = di;
+        }
+        if (mg->kind != HELM_PC_NONE) {  // omega / diagonal for the complex128 sweeps
+            double2 *di = nullptr;
+            CKC(dalloc(&di, L.np, h->owned));
+            CKC(launch_diag_inv<double>(L.M64, dim, mg->omega, di, s));
+            L.M64.dinv = di;
         }
         CKC(dalloc(&L.b64, L.np, h->owned)); CKC(dalloc(&L.u64, L.np, h->owned));
         CKC(dalloc(&L.t64, L.np, h->owned)); CKC(dalloc(&L.b32, L.np, h->owned));
@@ -538,14 +544,10 @@ static cudaError_t smooth(helm_handle *h, int l, int sweeps, const typename CT<R
         return cudaSuccess;
     }
     if (h->mg.smoother == HELM_SMOOTH_RB) {
-        if (zero) {
-            ProfScope ps(h, HELM_K_VECTOR, L.np * es, 0);
-            CKE(launch_zero(L.np, *cur, h->stream));
-        }
         for (int s = 0; s < sweeps; s++) {
             for (int colour = 0; colour < 2; colour++) {
                 ProfScope ps(h, cls, 0.5 * ni * (3 * es + rs), 0);
-                CKE(launch_rb<R>(op, h->dim, om, b, *cur, colour, h->stream));
+                CKE(launch_rb<R>(op, h->dim, om, b, *cur, colour, zero && s == 0, h->stream));
             }
         }
         return cudaSuccess;
@@ -709,27 +711,48 @@ static cudaError_t cycle(helm_handle *h, int l, const typename CT<R>::T *b, type
             return launch_prolong_post2(L.M32, tile, (float)h->mg.omega, b, L.t32, u, ec, h->stream);
         }
     }
-    C *cur = u, *oth = LvBuf<R>::t(L);
-    CKE(smooth<R>(h, l, h->mg.nu1, b, &cur, &oth, zero));
     LevelDev &Lc = h->lv[l + 1];
-    {
-        ProfScope ps(h, HELM_K_RESTRICT, ni * (2 * es + rs + es / nd), 0);
-        CKE(launch_residual_restrict<R>(LvBuf<R>::op(L), h->dim, b, cur, LvBuf<R>::b(Lc), h->stream));
-    }
+    // the coarse correction: Lc's right-hand side in, its error out
     C *ec = LvBuf<R>::u(Lc);
-    if (l + 1 == last) {
-        CKE(coarse_solve<R>(h, Lc, LvBuf<R>::b(Lc), ec));
-    } else {
+    auto coarse = [&]() -> cudaError_t {
+        if (l + 1 == last) return coarse_solve<R>(h, Lc, LvBuf<R>::b(Lc), ec);
         for (int i = 1; i <= gc; i++) {
             if (i == 1) CKE(cycle<R>(h, l + 1, LvBuf<R>::b(Lc), ec, true, gf, gc));
             else CKE(cycle<R>(h, l + 1, LvBuf<R>::b(Lc), ec, false, gc, gf));
         }
+        return cudaSuccess;
+    };
+    const int cls = l == 0 ? HELM_K_SMOOTH_FINE : HELM_K_SMOOTH_COARSE;
+    const int nu1 = h->mg.nu1, nu2 = h->mg.nu2, rb = h->mg.smoother == HELM_SMOOTH_RB;
+    // 2D levels with one or two sweeps each way: the way down (sweeps, residual, full weighting; the
+    // iterate to this level's t) and the way up (correction, sweeps; t -> u) as one launch each.  A
+    // complex64 level whose tuning asks for separate launches gets them.
+    const bool separate = prec == 0 && l < HELM_MAX_LEVELS && h->tune.level_tile[l] == HELM_TILE_NONE;
+    if (!separate && tile2d_ok(L.n, h->dim, nu1) && tile2d_ok(L.n, h->dim, nu2)) {
+        const DevOp<R> &op = LvBuf<R>::op(L);
+        const double ds = es, sweep = ni * (3 * es + rs);
+        {
+            ProfScope ps(h, cls, ni * ((zero ? 2 : 3) * es + ds + rs + es / nd), 0,
+                         nu1 * sweep - (zero ? ni * es : 0) + ni * (2 * es + rs + es / nd));
+            CKE(launch_tile_pre<R>(op, (R)h->mg.omega, nu1, rb, b, zero ? nullptr : u, LvBuf<R>::t(L), LvBuf<R>::b(Lc),
+                                   h->stream));
+        }
+        CKE(coarse());
+        ProfScope ps(h, cls, ni * (3 * es + ds + es / nd), 0, nu2 * sweep + ni * (2 * es + es / nd));
+        return launch_tile_post<R>(op, (R)h->mg.omega, nu2, rb, b, LvBuf<R>::t(L), u, ec, h->stream);
     }
+    C *cur = u, *oth = LvBuf<R>::t(L);
+    CKE(smooth<R>(h, l, nu1, b, &cur, &oth, zero));
+    {
+        ProfScope ps(h, HELM_K_RESTRICT, ni * (2 * es + rs + es / nd), 0);
+        CKE(launch_residual_restrict<R>(LvBuf<R>::op(L), h->dim, b, cur, LvBuf<R>::b(Lc), h->stream));
+    }
+    CKE(coarse());
     {
         ProfScope ps(h, HELM_K_PROLONG, ni * (2 * es + es / nd), 0);
         CKE(launch_prolong_add<R>(L.n, h->dim, ec, cur, h->stream, LvBuf<R>::op(L).gate));
     }
-    CKE(smooth<R>(h, l, h->mg.nu2, b, &cur, &oth, false));
+    CKE(smooth<R>(h, l, nu2, b, &cur, &oth, false));
     if (cur != u) CKE(cudaMemcpyAsync(u, cur, L.np * sizeof(C), cudaMemcpyDeviceToDevice, h->stream));
     return cudaSuccess;
 }

@@ -82,8 +82,9 @@ template <typename R> struct DevOp {
     const C *coef[3];
     const R *k2;
     C bk, c;
-    // 2D complex64 levels: 1 / (diagonal of M) at every node (0 off the interior), formed once
-    // by launch_diag_inv for the temporally blocked smoothers; null otherwise
+    // formed once by launch_diag_inv (0 off the interior): 2D complex64 levels 1 / (diagonal of M)
+    // for the temporally blocked smoothers; complex128 levels omega / (diagonal of M), which every
+    // complex128 sweep uses; null otherwise
     const C *dinv = nullptr;
     // device flag (null: none): when it is set at launch, this level's smoothing, residual and
     // transfer kernels return at once (the fused coarse-tail kernels do not test it).  Set only
@@ -175,9 +176,10 @@ cudaError_t launch_residual(const DevOp<R> &op, int dim, const CB *b, const type
 template <typename R, typename CB>
 cudaError_t launch_jacobi(const DevOp<R> &op, int dim, R omega, const CB *b, const typename CT<R>::T *u_in,
                           typename CT<R>::T *u_out, cudaStream_t s);
-// one colour of omega-red-black Jacobi, in place; colour 0 = (i+j+k) even.
+// one colour of omega-red-black Jacobi, in place; colour 0 = (i+j+k) even.  zero: the iterate is 0
+// on entry to the sweep (its interior is not read: colour 0, then colour 1, fill it).
 template <typename R, typename CB>
-cudaError_t launch_rb(const DevOp<R> &op, int dim, R omega, const CB *b, typename CT<R>::T *u, int colour,
+cudaError_t launch_rb(const DevOp<R> &op, int dim, R omega, const CB *b, typename CT<R>::T *u, int colour, int zero,
                       cudaStream_t s);
 // rc = FW(b - M u) on the coarse grid (fine nodes op.n, coarse nodes (n+1)/2).
 template <typename R, typename CB>
@@ -203,8 +205,24 @@ cudaError_t launch_pre2_wave(const DevOp<float> &op, float omega, const float2 *
                              cudaStream_t s);
 cudaError_t launch_post2_wave(const DevOp<float> &op, float omega, const float2 *b, const float2 *u_in, float2 *u_out,
                               const float2 *ec, cudaStream_t s);
-// dinv = 1 / (diagonal of M) at every node of a 2D level (0 off the interior)
-cudaError_t launch_diag_inv(const DevOp<float> &op, float2 *dinv, cudaStream_t s);
+// dinv = 1 / (diagonal of M) (complex64) or omega / (diagonal of M) (complex128) at every node of a
+// level (0 off the interior)
+template <typename R>
+cudaError_t launch_diag_inv(const DevOp<R> &op, int dim, R omega, typename CT<R>::T *dinv, cudaStream_t s);
+// A 2D level's way down and way up in one launch each, any precision and smoother
+// (kernels_tile2d.cu), nu = 1 or 2 sweeps (tile2d_ok):
+//   pre:  u_out = sweeps of M u = b from u_in (null: zero), rc = FW(b - M u_out)
+//   post: u_out = sweeps of (u_in + P ec)
+// u_in != u_out.
+bool tile2d_ok(const int n[3], int dim, int nu);
+template <typename R>
+cudaError_t launch_tile_pre(const DevOp<R> &op, R omega, int nu, int rb, const typename CT<R>::T *b,
+                            const typename CT<R>::T *u_in, typename CT<R>::T *u_out, typename CT<R>::T *rc,
+                            cudaStream_t s);
+template <typename R>
+cudaError_t launch_tile_post(const DevOp<R> &op, R omega, int nu, int rb, const typename CT<R>::T *b,
+                             const typename CT<R>::T *u_in, typename CT<R>::T *u_out, const typename CT<R>::T *ec,
+                             cudaStream_t s);
 cudaError_t launch_pre2_restrict(const DevOp<float> &op, int tile, float omega, const float2 *b, float2 *u_out,
                                  float2 *rc, cudaStream_t s);
 cudaError_t launch_prolong_post2(const DevOp<float> &op, int tile, float omega, const float2 *b, const float2 *u_in,

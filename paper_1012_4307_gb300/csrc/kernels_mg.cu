@@ -38,28 +38,33 @@ template <typename R> __host__ __device__ OpView<R> view(const DevOp<R> &op) {
 }
 
 // Off-diagonal part of the stencil at p (neighbours along x and y; z handled by callers that
-// march in k) and the diagonal entry.
+// march in k).
+template <typename R, int DIM, typename CX>
+__device__ __forceinline__ typename CT<R>::T offdiag(const OpView<R> &o, const CX *__restrict__ x, size_t p, int i,
+                                                    int j, int k, typename CT<R>::T xm_z, typename CT<R>::T xp_z) {
+    typedef typename CT<R>::T C;
+    const size_t sy = (size_t)o.nx;
+    C acc = cmul(__ldg(&o.cx[3 * i]), to_c(x[p - 1], R()));
+    acc = cfma(__ldg(&o.cx[3 * i + 2]), to_c(x[p + 1], R()), acc);
+    acc = cfma(__ldg(&o.cy[3 * j]), to_c(x[p - sy], R()), acc);
+    acc = cfma(__ldg(&o.cy[3 * j + 2]), to_c(x[p + sy], R()), acc);
+    if (DIM == 3) {
+        acc = cfma(__ldg(&o.cz[3 * k]), xm_z, acc);
+        acc = cfma(__ldg(&o.cz[3 * k + 2]), xp_z, acc);
+    }
+    return acc;
+}
+
+// (M x)_p and the diagonal entry.
 template <typename R, int DIM, typename CX>
 __device__ __forceinline__ typename CT<R>::T stencil(const OpView<R> &o, const CX *__restrict__ x, size_t p,
                                                     int i, int j, int k, typename CT<R>::T xm_z,
                                                     typename CT<R>::T xc, typename CT<R>::T xp_z,
                                                     typename CT<R>::T &diag) {
     typedef typename CT<R>::T C;
-    const size_t sy = (size_t)o.nx;
-    C cw = __ldg(&o.cx[3 * i]), cc = __ldg(&o.cx[3 * i + 1]), ce = __ldg(&o.cx[3 * i + 2]);
-    C acc = cmul(cw, to_c(x[p - 1], R()));
-    acc = cfma(ce, to_c(x[p + 1], R()), acc);
-    C d = cc;
-    cw = __ldg(&o.cy[3 * j]); cc = __ldg(&o.cy[3 * j + 1]); ce = __ldg(&o.cy[3 * j + 2]);
-    acc = cfma(cw, to_c(x[p - sy], R()), acc);
-    acc = cfma(ce, to_c(x[p + sy], R()), acc);
-    d = cadd(d, cc);
-    if (DIM == 3) {
-        cw = __ldg(&o.cz[3 * k]); cc = __ldg(&o.cz[3 * k + 1]); ce = __ldg(&o.cz[3 * k + 2]);
-        acc = cfma(cw, xm_z, acc);
-        acc = cfma(ce, xp_z, acc);
-        d = cadd(d, cc);
-    }
+    const C acc = offdiag<R, DIM>(o, x, p, i, j, k, xm_z, xp_z);
+    C d = cadd(__ldg(&o.cx[3 * i + 1]), __ldg(&o.cy[3 * j + 1]));
+    if (DIM == 3) d = cadd(d, __ldg(&o.cz[3 * k + 1]));
     d = cadd(d, cadd(cscale(o.bk, o.k2[p]), o.c));
     diag = d;
     return cfma(d, xc, acc);
@@ -133,6 +138,10 @@ __global__ void __launch_bounds__(BX *BY) k_jacobi(OpView<R> o, R omega, const C
     INTERIOR_IJ(o);
     if (ZERO) {
         for (int k = k0; k < k1; k++, p += sz) {
+            if constexpr (sizeof(R) == sizeof(double)) {
+                un[p] = cmul(to_c(b[p], R()), o.dinv[p]);
+                continue;
+            }
             C d;
             // diagonal only: the stencil of the zero vector
             d = cadd(cadd(__ldg(&o.cx[3 * i + 1]), __ldg(&o.cy[3 * j + 1])), cadd(cscale(o.bk, o.k2[p]), o.c));
@@ -145,10 +154,15 @@ __global__ void __launch_bounds__(BX *BY) k_jacobi(OpView<R> o, R omega, const C
     if (DIM == 3) xm = u[p - sz];
     for (int k = k0; k < k1; k++, p += sz) {
         if (DIM == 3) xp = u[p + sz];
-        C d;
-        C mu = stencil<R, DIM>(o, u, p, i, j, k, xm, xc, xp, d);
-        C res = csub(to_c(b[p], R()), mu);
-        un[p] = cadd(xc, cscale(cmul(res, cinv(d)), omega));
+        if constexpr (sizeof(R) == sizeof(double)) {
+            const C r = csub(to_c(b[p], R()), offdiag<R, DIM>(o, u, p, i, j, k, xm, xp));
+            un[p] = cfma(o.dinv[p], r, cscale(xc, R(1) - omega));
+        } else {
+            C d;
+            C mu = stencil<R, DIM>(o, u, p, i, j, k, xm, xc, xp, d);
+            C res = csub(to_c(b[p], R()), mu);
+            un[p] = cadd(xc, cscale(cmul(res, cinv(d)), omega));
+        }
         if (DIM == 3) { xm = xc; xc = xp; }
     }
 }
@@ -174,6 +188,37 @@ __global__ void __launch_bounds__(BX *BY) k_jacobi3(OpView<R> o, R omega, const 
     const C cwx = __ldg(&o.cx[3 * i]), ccx = __ldg(&o.cx[3 * i + 1]), cex = __ldg(&o.cx[3 * i + 2]);
     const C cwy = __ldg(&o.cy[3 * j]), ccy = __ldg(&o.cy[3 * j + 1]), cey = __ldg(&o.cy[3 * j + 2]);
     C bq = to_c(b[p], R());
+    if constexpr (sizeof(R) == sizeof(double)) {
+        // complex128: bound by the FP64 units, so the sweep takes omega / D as formed once
+        // (34 operations per node instead of about 67)
+        C wq = o.dinv[p];
+        if (gv) return;
+        if (ZERO) {
+            for (int k = k0; k < k1; k++, p += sz) un[p] = cmul(to_c(b[p], R()), o.dinv[p]);
+            return;
+        }
+        C xm = u[p - sz], xc = u[p], xp = u[p + sz];
+        for (int k = k0; k < k1; k++, p += sz) {
+            C xp2 = xp, bn = bq, wn = wq;
+            const C xw = u[p - 1], xe = u[p + 1], xs = u[p - sy], xn = u[p + sy];
+            if (k + 1 < k1) {
+                xp2 = u[p + 2 * sz];
+                bn = to_c(b[p + sz], R());
+                wn = o.dinv[p + sz];
+            }
+            C acc = cmul(cwx, xw);
+            acc = cfma(cex, xe, acc);
+            acc = cfma(cwy, xs, acc);
+            acc = cfma(cey, xn, acc);
+            acc = cfma(__ldg(&o.cz[3 * k]), xm, acc);
+            acc = cfma(__ldg(&o.cz[3 * k + 2]), xp, acc);
+            un[p] = cfma(wq, csub(bq, acc), cscale(xc, R(1) - omega));
+            xm = xc;
+            xc = xp;
+            xp = xp2; bq = bn; wq = wn;
+        }
+        return;
+    } else {
     R kq = o.k2[p];
     if (gv) return;
     if (ZERO) {
@@ -225,11 +270,19 @@ __global__ void __launch_bounds__(BX *BY) k_jacobi3(OpView<R> o, R omega, const 
         xc = xp;
         xw = xw2; xe = xe2; xs = xs2; xn = xn2; xp = xp2; bq = bn; kq = kn;
     }
+    }  // complex64
 }
 
-// one colour of omega-red-black Jacobi, in place: threads map to every other x node.
-template <typename R, int DIM, typename CB>
-__global__ void __launch_bounds__(BX *BY) k_rb(OpView<R> o, R omega, const CB *__restrict__ b, typename CT<R>::T *u, int colour) {
+// one colour of omega-red-black Jacobi, in place: threads map to every other x node and march kc
+// planes.  FROM: the iterate on entry is given (RB_ANY), zero everywhere and not read (RB_ZERO: the
+// first colour of a sweep from zero is pointwise), or zero on this colour and not read there
+// (RB_OWN_ZERO: the second colour).  complex128 takes omega / D as formed once (see k_jacobi3).
+// Measured, 193 x 129 x 97 complex128 V(1,1) cycle: 1318 us with the diagonal assembled and divided by
+// at every node, a zero fill before the first sweep and chunks of 8 planes on every level, 719 us so.
+enum { RB_ANY, RB_ZERO, RB_OWN_ZERO };
+template <typename R, int DIM, typename CB, int FROM>
+__global__ void __launch_bounds__(BX *BY) k_rb(OpView<R> o, R omega, const CB *__restrict__ b, typename CT<R>::T *u, int colour,
+                                               int kc) {
     pdl_enter();
     if (o.gate && *o.gate) return;
     typedef typename CT<R>::T C;
@@ -237,18 +290,26 @@ __global__ void __launch_bounds__(BX *BY) k_rb(OpView<R> o, R omega, const CB *_
     const int j = blockIdx.y * BY + threadIdx.y + 1;
     if (j > o.ny - 2) return;
     int k0 = 0, k1 = 1;
-    if (DIM == 3) { k0 = blockIdx.z * KCHUNK + 1; k1 = min(k0 + KCHUNK, o.nz - 1); }
+    if (DIM == 3) { k0 = blockIdx.z * kc + 1; k1 = min(k0 + kc, o.nz - 1); }
     const size_t sz = (size_t)o.nx * o.ny;
+#pragma unroll 2
     for (int k = k0; k < k1; k++) {
         const int i = 2 * t + 1 + ((1 + j + k + colour) & 1);
         if (i > o.nx - 2) continue;
         const size_t p = (size_t)i + (size_t)o.nx * ((size_t)j + (size_t)o.ny * k);
-        C xm = mk(R(0), R(0)), xp = mk(R(0), R(0));
-        if (DIM == 3) { xm = u[p - sz]; xp = u[p + sz]; }
-        C xc = u[p];
-        C d;
-        C mu = stencil<R, DIM>(o, u, p, i, j, k, xm, xc, xp, d);
-        u[p] = cadd(xc, cscale(cmul(csub(to_c(b[p], R()), mu), cinv(d)), omega));
+        C xm = mk(R(0), R(0)), xp = xm, xc = xm, w, acc = xm;
+        if (FROM != RB_ZERO && DIM == 3) { xm = u[p - sz]; xp = u[p + sz]; }
+        if (FROM == RB_ANY) xc = u[p];
+        if constexpr (sizeof(R) == sizeof(double)) {
+            w = o.dinv[p];
+        } else {
+            C d = cadd(__ldg(&o.cx[3 * i + 1]), __ldg(&o.cy[3 * j + 1]));
+            if (DIM == 3) d = cadd(d, __ldg(&o.cz[3 * k + 1]));
+            w = cscale(cinv(cadd(d, cadd(cscale(o.bk, o.k2[p]), o.c))), omega);
+        }
+        C r = to_c(b[p], R());
+        if (FROM != RB_ZERO) r = csub(r, offdiag<R, DIM>(o, u, p, i, j, k, xm, xp));
+        u[p] = FROM == RB_ANY ? cfma(w, r, cscale(xc, R(1) - omega)) : cmul(w, r);
     }
 }
 
@@ -845,11 +906,22 @@ cudaError_t launch_jacobi(const DevOp<R> &op, int dim, R omega, const CB *bb, co
 }
 
 template <typename R, typename CB>
-cudaError_t launch_rb(const DevOp<R> &op, int dim, R omega, const CB *bb, typename CT<R>::T *u, int colour,
+cudaError_t launch_rb(const DevOp<R> &op, int dim, R omega, const CB *bb, typename CT<R>::T *u, int colour, int zero,
                       cudaStream_t s) {
-    dim3 g(cdiv((op.n[0] - 1) / 2, BX), cdiv(op.n[1] - 2, BY), dim == 3 ? cdiv(op.n[2] - 2, KCHUNK) : 1), b(BX, BY);
-    if (dim == 3) launch_pdl(k_rb<R, 3, CB>, g, b, 0, s, view(op), omega, bb, u, colour);
-    else launch_pdl(k_rb<R, 2, CB>, g, b, 0, s, view(op), omega, bb, u, colour);
+    dim3 g(cdiv((op.n[0] - 1) / 2, BX), cdiv(op.n[1] - 2, BY)), b(BX, BY);
+    // planes per thread: chunks of 8 left most of the chip idle on small levels (33 us a colour)
+    const int kc = dim == 3 ? z_chunk((size_t)g.x * g.y, op.n[2] - 2, KCHUNK, 152 * 10) : 1;
+    if (dim == 3) g.z = cdiv(op.n[2] - 2, kc);
+    auto go = [&](auto kernel) { return launch_pdl(kernel, g, b, 0, s, view(op), omega, bb, u, colour, kc); };
+    if (dim == 3) {
+        if (!zero) go(k_rb<R, 3, CB, RB_ANY>);
+        else if (colour == 0) go(k_rb<R, 3, CB, RB_ZERO>);
+        else go(k_rb<R, 3, CB, RB_OWN_ZERO>);
+    } else {
+        if (!zero) go(k_rb<R, 2, CB, RB_ANY>);
+        else if (colour == 0) go(k_rb<R, 2, CB, RB_ZERO>);
+        else go(k_rb<R, 2, CB, RB_OWN_ZERO>);
+    }
     return cudaGetLastError();
 }
 
@@ -1043,7 +1115,7 @@ template <typename C> cudaError_t launch_zero(size_t n, C *x, cudaStream_t s) {
     template cudaError_t launch_jacobi<R, CT<R>::T>(const DevOp<R> &, int, R, const CT<R>::T *, const CT<R>::T *, \
                                                      CT<R>::T *, cudaStream_t);                                 \
     template cudaError_t launch_rb<R, CT<R>::T>(const DevOp<R> &, int, R, const CT<R>::T *, CT<R>::T *, int,     \
-                                                 cudaStream_t);                                                 \
+                                                 int, cudaStream_t);                                            \
     template cudaError_t launch_residual_restrict<R, CT<R>::T>(const DevOp<R> &, int, const CT<R>::T *,          \
                                                                 const CT<R>::T *, CT<R>::T *, cudaStream_t);    \
     template cudaError_t launch_prolong_add<R>(const int *, int, const CT<R>::T *, CT<R>::T *, cudaStream_t,      \
@@ -1064,23 +1136,30 @@ template cudaError_t launch_zero<float2>(size_t, float2 *, cudaStream_t);
 
 // ------------------------------------------------------------------------------ 1 / diagonal
 namespace {
-__global__ void k_diag_inv(OpView<float> o, float2 *__restrict__ dinv) {
+template <typename R> __global__ void k_diag_inv(OpView<R> o, int dim, R omega, typename CT<R>::T *__restrict__ dinv) {
     pdl_enter();
-    const size_t n = (size_t)o.nx * o.ny;
+    typedef typename CT<R>::T C;
+    const size_t sz = (size_t)o.nx * o.ny, n = sz * (dim == 3 ? o.nz : 1);
     for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < n; p += (size_t)gridDim.x * blockDim.x) {
-        const int x = (int)(p % o.nx), y = (int)(p / o.nx);
-        float2 v = make_float2(0.f, 0.f);
-        if (x >= 1 && x <= o.nx - 2 && y >= 1 && y <= o.ny - 2) {
-            const float2 d = cadd(cadd(o.cx[3 * x + 1], o.cy[3 * y + 1]), cadd(cscale(o.bk, o.k2[p]), o.c));
-            v = cinv_fast(d);
+        const int k = (int)(p / sz), x = (int)(p % o.nx), y = (int)(p % sz / o.nx);
+        C v = mk(R(0), R(0));
+        if (x >= 1 && x <= o.nx - 2 && y >= 1 && y <= o.ny - 2 && (dim == 2 || (k >= 1 && k <= o.nz - 2))) {
+            C d = cadd(o.cx[3 * x + 1], o.cy[3 * y + 1]);
+            if (dim == 3) d = cadd(d, o.cz[3 * k + 1]);
+            d = cadd(d, cadd(cscale(o.bk, o.k2[p]), o.c));
+            if constexpr (sizeof(R) == sizeof(float)) v = cinv_fast(d);
+            else v = cscale(cinv(d), omega);
         }
         dinv[p] = v;
     }
 }
 }  // namespace
 
-cudaError_t launch_diag_inv(const DevOp<float> &op, float2 *dinv, cudaStream_t s) {
-    const size_t n = (size_t)op.n[0] * op.n[1];
-    launch_pdl(k_diag_inv, (unsigned)std::min<size_t>(cdiv(n, 256), 152 * 8), 256, 0, s, view(op), dinv);
+template <typename R>
+cudaError_t launch_diag_inv(const DevOp<R> &op, int dim, R omega, typename CT<R>::T *dinv, cudaStream_t s) {
+    const size_t n = (size_t)op.n[0] * op.n[1] * (dim == 3 ? op.n[2] : 1);
+    launch_pdl(k_diag_inv<R>, (unsigned)std::min<size_t>(cdiv(n, 256), 152 * 8), 256, 0, s, view(op), dim, omega, dinv);
     return cudaGetLastError();
 }
+template cudaError_t launch_diag_inv<float>(const DevOp<float> &, int, float, float2 *, cudaStream_t);
+template cudaError_t launch_diag_inv<double>(const DevOp<double> &, int, double, double2 *, cudaStream_t);

@@ -54,3 +54,25 @@ def test_fused_tail_any_cycle(helm, oracle, n, coarsest_n, prec, smoother, nu, g
     """The coarse tail on a thread-block cluster at every depth: lines and planes as rows, more
     blocks than rows, coarsest grids with an even number of rows, red-black and F / W cycles."""
     check_cycle(helm, oracle, n, coarsest_n, prec, smoother, nu, gamma, [dict(tail_levels=t) for t in (-1, 2, 3, 4, 0)])
+
+
+@pytest.mark.parametrize("prec", ["c64", "c128"])
+@pytest.mark.parametrize("smoother,nu,gamma", [("jacobi", (1, 2), (1, 1)), ("jacobi", (2, 1), (1, 3)),
+                                               ("jacobi", (2, 2), (2, 2)), ("rb", (1, 1), (1, 1)),
+                                               ("rb", (2, 1), (1, 2)), ("rb", (1, 2), (1, 1)),
+                                               ("jacobi", (3, 0), (1, 1)), ("rb", (0, 3), (1, 1))])
+@pytest.mark.parametrize("n,coarsest_n", [((67, 35), 34), ((35, 67), 34), ((9, 5), 5), ((161, 97), 17), ((257, 193), 17)])
+def test_2d_level_tiles(helm, oracle, n, coarsest_n, prec, smoother, nu, gamma):
+    """A level's way down and way up as one launch each: coarse interiors that fill the tiles exactly
+    and that leave remainders, the smallest level, every tile shape, sweeps from zero and from a
+    guess; more or fewer than one or two sweeps take the separate kernels."""
+    check_cycle(helm, oracle, n, coarsest_n, prec, smoother, nu, gamma, [dict(tail_levels=0)])
+
+
+@pytest.mark.parametrize("prec", ["c64", "c128"])
+@pytest.mark.parametrize("smoother,nu,gamma", [("jacobi", (1, 2), (1, 1)), ("rb", (1, 1), (1, 2)), ("rb", (2, 0), (1, 1))])
+@pytest.mark.parametrize("n,coarsest_n", [((33, 17, 65), 9), ((17, 65, 33), 9), ((65, 33, 25), 9)])
+def test_3d_level_kernels(helm, oracle, n, coarsest_n, prec, smoother, nu, gamma):
+    """The 3D sweeps (omega / D formed once in complex128), red-black from zero and from a guess, with
+    chunks of one to eight planes."""
+    check_cycle(helm, oracle, n, coarsest_n, prec, smoother, nu, gamma, [dict(tail_levels=0)])
