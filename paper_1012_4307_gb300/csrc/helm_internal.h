@@ -357,16 +357,18 @@ cudaError_t launch_zero(size_t n, C *x, cudaStream_t s);
 int blas_nblocks(size_t n);
 // Gram-Schmidt passes (gate: device int; the kernel returns at once when *gate == 0).
 // partials[i * G + b] = sum conj(V_i) w (i < nv) and partials[nv * G + b] = (||w||^2, 0),
-// G = blas_nblocks(n).
+// G = mdot_nblocks(n, nv) (at most blas_nblocks(n), which it is for nv = 0: the norm alone, no gate).
+int mdot_nblocks(size_t n, int nv);
 cudaError_t launch_mdot_norm(size_t n, const double2 *V, size_t ldv, int nv, const double2 *w, double2 *partials,
                              const int *gate, cudaStream_t s);
 // w -= sum_i V_i h_i, then partials[b] = (||w||^2, 0)   (h on device)
 cudaError_t launch_update_norm(size_t n, const double2 *V, size_t ldv, int nv, const double2 *h, double2 *w,
                                double2 *partials, const int *gate, cudaStream_t s);
 // out[i] (mode 0: =, 1: +=, 2: (sqrt(re), 0)) = fixed-order sum of partials of vector i; with
-// host_out (pinned host memory), host_out[i] = the real part of out[i] as well
+// host_out (pinned host memory), host_out[i] = the real part of out[i] as well; with out2, out2[i] =
+// the plain sum too
 cudaError_t launch_reduce(const double2 *partials, int nblk, int nv, double2 *out, int mode, const int *gate,
-                          cudaStream_t s, double *host_out = nullptr);
+                          cudaStream_t s, double *host_out = nullptr, double2 *out2 = nullptr);
 // Same two passes in double-FP32 arithmetic on float-pair vectors (kernels_gs_df.cu): node q
 // of such a vector is the float4 (re.hi, re.lo, im.hi, im.lo).  Dot-pass partials use
 // G = gs_df_nblocks(n) blocks per vector, update-pass partials gs_df_update_nblocks(n).
@@ -412,8 +414,9 @@ cudaError_t launch_pair_to_c128(size_t n, const float4 *v, const double2 *alpha,
 // *hnorm: ||w||^2 in, ||w'|| out; *flag = (||w'|| < eta ||w||); *count += flag
 cudaError_t launch_reduce_decide(const double2 *partials, int nblk, double2 *hnorm, int *flag, int *count, double eta,
                                  cudaStream_t s);
-// y = x * (1 / scale[0].x)
-cudaError_t launch_scale_inv(size_t n, const double2 *x, const double2 *scale, double2 *y, cudaStream_t s);
+// y = x * (1 / scale[0].x); with b_out, b_out = y rounded to complex64 as well
+cudaError_t launch_scale_inv(size_t n, const double2 *x, const double2 *scale, double2 *y, float2 *b_out,
+                             cudaStream_t s);
 // x += sum_c y_c Z_c  (Z c64 or c128, ldz stride); with alpha (c64 only) the weights are
 // y_c / alpha[c].x for c >= 1 (columns that hold alpha_c z_c)
 template <typename CZ>
@@ -434,16 +437,27 @@ cudaError_t launch_cycle_start(double2 *g, int len, const double2 *beta, int *st
 // y = H(0:k,0:k)^{-1} g(0:k)  (upper triangular back substitution)
 cudaError_t launch_backsolve(const double2 *H, int ldh, int k, const double2 *g, double2 *y, cudaStream_t s);
 
-// Bi-CGSTAB vector updates (FP64)
-// p = r + beta (p - omega v), beta and omega from dev scalars
-cudaError_t launch_bicg_p(size_t n, const double2 *r, const double2 *v, const double2 *sc, double2 *p,
+// Bi-CGSTAB (FP64).  sc: the device scalar block (k_bicg_scalars); partials: at least 4
+// blas_nblocks(n) doubles; ticket: a device counter at 0 between launches; host: two pinned doubles.
+// p = r + beta (p - omega v); b_out (may be null) = p rounded to complex64
+cudaError_t launch_bicg_p(size_t n, const double2 *r, const double2 *v, const double2 *sc, double2 *p, float2 *b_out,
                           cudaStream_t s);
-// generic: y = a*x + b*y with device complex scalars a, b (pointers into a scalar block)
-cudaError_t launch_axpby(size_t n, const double2 *a, const double2 *x, const double2 *b, double2 *y,
-                         cudaStream_t s);
+// stage 1: <rh, v> (a = rh, b = v), then alpha; stage 2: <t, s> and <t, t> (a = t, b = s), then omega
+cudaError_t launch_bicg_dots(int stage, size_t n, const double2 *a, const double2 *b, double2 *sc, double2 *partials,
+                             unsigned *ticket, cudaStream_t s);
+// s = r - alpha v; host = (||s||, breakdown flag); b_out (may be null) = s rounded to complex64
+cudaError_t launch_bicg_s(size_t n, const double2 *r, const double2 *v, double2 *sc, double2 *so, float2 *b_out,
+                          double2 *partials, unsigned *ticket, double *host, cudaStream_t s);
+// x += alpha y + omega z; r = s - omega t; rho = <rh, r>, then beta; host = (||r||, breakdown flag
+// before that step)
+template <typename CY>
+cudaError_t launch_bicg_xr(size_t n, const CY *y, const CY *z, const double2 *so, const double2 *t, const double2 *rh,
+                           double2 *sc, double2 *x, double2 *r, double2 *partials, unsigned *ticket, double *host,
+                           cudaStream_t s);
+// y += a x with a device complex scalar a
 template <typename CY>
 cudaError_t launch_axpy_mixed(size_t n, const double2 *a, const CY *x, double2 *y, cudaStream_t s);
-// scalar kernels of Bi-CGSTAB (device-side scalar algebra, no host round trip)
+// scalar steps of Bi-CGSTAB as a launch of their own (0: beta, 3: initial values)
 cudaError_t launch_bicg_scalars(int stage, double2 *sc, cudaStream_t s);
 
 // adjoint helpers

@@ -3,7 +3,7 @@
 // fixed reduction tree, so repeated runs give bit-identical results.
 //
 // Classical Gram-Schmidt runs as two fused passes over the basis:
-//   "dot"     h = V^H w and ||w||^2                 (k_mdot_norm, 8 basis vectors per block row)
+//   "dot"     h = V^H w and ||w||^2                 (k_mdot_norm, at most 8 basis vectors per block row)
 //   "update"  w <- w - V h and ||w'||^2, same sweep (k_update_norm)
 // followed by the DGKS test on the device (k_reduce_decide); the optional second pass reuses
 // the same kernels, gated by the device flag, so the host never waits for the decision.
@@ -44,34 +44,108 @@ __device__ __forceinline__ void block_sum(double2 (&v)[NV], double2 *out_shared)
     }
 }
 
-// Pass "dot": partials[i * G + b] = sum_q conj(V_i[q]) w[q] for the CH vectors of chunk
-// blockIdx.y (i < nv), and chunk 0 also partials[nv * G + b] = (sum |w[q]|^2, 0).
-// Grid (G, max(1, ceil(nv / CH))).  Skipped entirely when *gate == 0.
-template <int CH>
-__global__ void __launch_bounds__(NT) k_mdot_norm(size_t n, const double2 *__restrict__ V, size_t ldv, int nv,
-                                                  const double2 *__restrict__ w, double2 *__restrict__ partials,
-                                                  const int *__restrict__ gate) {
-    pdl_enter();
-    if (gate && *gate == 0) return;
-    __shared__ double2 sums[CH + 1];
-    const int i0 = blockIdx.y * CH;
-    const int cnt = min(CH, nv - i0);
-    const bool first = blockIdx.y == 0;
-    double2 acc[CH + 1];
+// Sums of N real values per thread over the warp (N a power of two, at most 32) by a transposing
+// butterfly: at offsets 16, 8, ... a lane keeps half of its values, sends the other half to the lane
+// at that offset and adds what it receives, so the values per lane halve at every level (N - 1 + the
+// plain levels additions per lane instead of 5 N; on the FP64 units, where a warp's instruction takes
+// 64 clocks of its scheduler, 5 N additions for 9 complex values cost more than the pass itself).
+// Lanes l with l % (32 / N) == 0 end with the sum of value idx in v[0].
+template <int N> __device__ __forceinline__ int warp_transpose_sum(double (&v)[N]) {
+    const int lane = threadIdx.x & 31;
+    int idx = 0;
 #pragma unroll
-    for (int t = 0; t <= CH; t++) acc[t] = make_double2(0.0, 0.0);
+    for (int o = 16, m = N; o > 0; o >>= 1) {
+        if (m > 1) {
+            const bool upper = (lane & o) != 0;
+#pragma unroll
+            for (int i = 0; i < m / 2; i++) {
+                const double keep = upper ? v[i + m / 2] : v[i], send = upper ? v[i] : v[i + m / 2];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+            if (upper) idx += m / 2;
+            m /= 2;
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+        }
+    }
+    return idx;
+}
+
+// Block-wide sum of one real value per thread, in thread 0 (fixed tree).
+__device__ __forceinline__ double block_sum_real(double v) {
+    __shared__ double red[NT / 32];
+    double a[1] = {v};
+    warp_transpose_sum<1>(a);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a[0];
+    __syncthreads();
+    double s = red[0];
+    if (threadIdx.x == 0)
+        for (int w = 1; w < NT / 32; w++) s += red[w];
+    return s;
+}
+
+// partials[b] = (sum |w[q]|^2, 0)
+__global__ void __launch_bounds__(NT) k_norm2(size_t n, const double2 *__restrict__ w, double2 *__restrict__ partials) {
+    pdl_enter();
+    double acc = 0.0;
     for (size_t q = blockIdx.x * (size_t)NT + threadIdx.x; q < n; q += (size_t)gridDim.x * NT) {
         const double2 wq = w[q];
-        if (first) acc[CH].x = fma(wq.x, wq.x, fma(wq.y, wq.y, acc[CH].x));
+        acc = fma(wq.x, wq.x, fma(wq.y, wq.y, acc));
+    }
+    acc = block_sum_real(acc);
+    if (threadIdx.x == 0) partials[blockIdx.x] = make_double2(acc, 0.0);
+}
+
+// Pass "dot": partials[i * G + b] = sum_q conj(V_i[q]) w[q] (i < nv), and partials[nv * G + b] =
+// (sum |w[q]|^2, 0).  Grid (G, chunks): block row y takes the vectors nv y / chunks ..
+// nv (y + 1) / chunks - 1, at most CH, so the rows are even.  Skipped entirely when *gate == 0.
+// Bound by the FP64 units (4 fused multiply-adds per vector and node): two blocks per SM, each thread
+// many nodes (a grid of one or two nodes per thread spent most of its time in the block sums:
+// 513^2, 13 vectors, 89 us per pass under ncu against 23 us of multiply-adds).
+template <int CH>
+__global__ void __launch_bounds__(NT, 2) k_mdot_norm(size_t n, const double2 *__restrict__ V, size_t ldv, int nv,
+                                                     const double2 *__restrict__ w, double2 *__restrict__ partials,
+                                                     const int *__restrict__ gate) {
+    pdl_enter();
+    if (gate && *gate == 0) return;
+    __shared__ double red[NT / 32][2 * CH + 1];
+    const int chunks = gridDim.y;
+    const int i0 = nv * (int)blockIdx.y / chunks;
+    const int cnt = nv * ((int)blockIdx.y + 1) / chunks - i0;
+    const bool first = blockIdx.y == 0;
+    double acc[2 * CH], nn[1] = {0.0};
+#pragma unroll
+    for (int t = 0; t < 2 * CH; t++) acc[t] = 0.0;
+    const double2 *Vc = V + (size_t)i0 * ldv;
+    for (size_t q = blockIdx.x * (size_t)NT + threadIdx.x; q < n; q += (size_t)gridDim.x * NT) {
+        const double2 wq = w[q];
+        double2 v[CH];
+        const double2 *p = Vc + q;
+#pragma unroll
+        for (int t = 0; t < CH; t++, p += ldv) v[t] = t < cnt ? *p : make_double2(0.0, 0.0);
+        if (first) nn[0] = fma(wq.x, wq.x, fma(wq.y, wq.y, nn[0]));
 #pragma unroll
         for (int t = 0; t < CH; t++)
-            if (t < cnt) acc[t] = cfmac(V[(size_t)(i0 + t) * ldv + q], wq, acc[t]);
+            if (t < cnt) {
+                acc[2 * t] = fma(v[t].x, wq.x, fma(v[t].y, wq.y, acc[2 * t]));
+                acc[2 * t + 1] = fma(v[t].x, wq.y, fma(-v[t].y, wq.x, acc[2 * t + 1]));
+            }
     }
-    block_sum<CH + 1>(acc, sums);
-    const int G = gridDim.x;
-    if constexpr (CH > 0)
-        if (threadIdx.x < CH && (int)threadIdx.x < cnt) partials[(size_t)(i0 + threadIdx.x) * G + blockIdx.x] = sums[threadIdx.x];
-    if (first && threadIdx.x == CH) partials[(size_t)nv * G + blockIdx.x] = sums[CH];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int idx = warp_transpose_sum<2 * CH>(acc);
+    if ((lane & (32 / (2 * CH) - 1)) == 0) red[warp][idx] = acc[0];
+    if (first) {
+        warp_transpose_sum<1>(nn);
+        if (lane == 0) red[warp][2 * CH] = nn[0];
+    }
+    __syncthreads();
+    const int t = threadIdx.x, G = gridDim.x;
+    if (t < 2 * cnt || (first && t == 2 * CH)) {
+        double s = red[0][t];
+        for (int x = 1; x < NT / 32; x++) s += red[x][t];
+        if (t < 2 * CH) ((double *)(partials + (size_t)(i0 + (t >> 1)) * G + blockIdx.x))[t & 1] = s;
+        else partials[(size_t)nv * G + blockIdx.x] = make_double2(s, 0.0);
+    }
 }
 
 // Pass "update": w -= sum_{i < nv} V_i h_i, then partials[b] = (sum |w|^2, 0).  Gated.
@@ -81,10 +155,9 @@ __global__ void __launch_bounds__(NT) k_update_norm(size_t n, const double2 *__r
     pdl_enter();
     if (gate && *gate == 0) return;
     __shared__ double2 hs[64];
-    __shared__ double2 sums[1];
     for (int i = threadIdx.x; i < nv; i += NT) hs[i] = h[i];
     __syncthreads();
-    double2 acc[1] = {make_double2(0.0, 0.0)};
+    double acc = 0.0;
     for (size_t q = blockIdx.x * (size_t)NT + threadIdx.x; q < n; q += (size_t)gridDim.x * NT) {
         double2 wq = w[q];
 #pragma unroll 8
@@ -95,16 +168,16 @@ __global__ void __launch_bounds__(NT) k_update_norm(size_t n, const double2 *__r
             wq.y = fma(-v.x, hh.y, fma(-v.y, hh.x, wq.y));
         }
         w[q] = wq;
-        acc[0].x = fma(wq.x, wq.x, fma(wq.y, wq.y, acc[0].x));
+        acc = fma(wq.x, wq.x, fma(wq.y, wq.y, acc));
     }
-    block_sum<1>(acc, sums);
-    if (threadIdx.x == 0) partials[blockIdx.x] = sums[0];
+    acc = block_sum_real(acc);
+    if (threadIdx.x == 0) partials[blockIdx.x] = make_double2(acc, 0.0);
 }
 
 // out[i] = sum_b partials[i * nblk + b] in a fixed order for i = blockIdx.x; mode 0 '=',
-// 1 '+=', 2 (sqrt(re), 0).  Gated.
+// 1 '+=', 2 (sqrt(re), 0).  With out2, out2[i] = the plain sum as well.  Gated.
 __global__ void k_reduce(const double2 *__restrict__ partials, int nblk, double2 *__restrict__ out, int mode,
-                         const int *__restrict__ gate, double *host_out) {
+                         const int *__restrict__ gate, double *host_out, double2 *__restrict__ out2) {
     pdl_enter();
     if (gate && *gate == 0) return;
     __shared__ double2 sums[1];
@@ -119,6 +192,7 @@ __global__ void k_reduce(const double2 *__restrict__ partials, int nblk, double2
         else if (mode == 1) r = cadd(out[i], t);
         else r = make_double2(sqrt(t.x), 0.0);
         out[i] = r;
+        if (out2) out2[i] = t;
         if (host_out) host_out[i] = r.x;
     }
 }
@@ -142,13 +216,16 @@ __global__ void k_reduce_decide(const double2 *__restrict__ partials, int nblk, 
     }
 }
 
-__global__ void k_scale_inv(size_t n, const double2 *x, const double2 *__restrict__ scale, double2 *y) {
+// y = x / scale; with b_out, its complex64 copy too (the next cycle's right-hand side)
+__global__ void k_scale_inv(size_t n, const double2 *x, const double2 *__restrict__ scale, double2 *y,
+                            float2 *__restrict__ b_out) {
     pdl_enter();
     const double s = scale[0].x;
     const double r = s != 0.0 ? 1.0 / s : 0.0;
     for (size_t q = blockIdx.x * (size_t)NT + threadIdx.x; q < n; q += (size_t)gridDim.x * NT) {
-        const double2 v = x[q];
-        y[q] = make_double2(v.x * r, v.y * r);
+        const double2 v = x[q], t = make_double2(v.x * r, v.y * r);
+        y[q] = t;
+        if (b_out) b_out[q] = to_c(t, 0.f);
     }
 }
 
@@ -205,9 +282,12 @@ __global__ void __launch_bounds__(NT) k_combine_df(size_t n, const float2 *__res
 // Complex Givens rotations G = [c s; -conj(s) c] (c real) on column j of the Hessenberg
 // matrix (column-major, leading dimension ldh); see Saad, Iterative Methods for Sparse Linear
 // Systems, Section 6.5.9 for the real case.
-// Called by one warp: the lanes stage column j of H (j + 2 entries) and the earlier rotations in
-// shared memory, lane 0 applies the rotations in order and forms the new one, the lanes write the
-// column back.  The arithmetic is that of a single thread walking the column in global memory.
+// Called by one warp.  A warp's FP64 instruction takes 64 clocks of its scheduler however few lanes
+// are live, so the chain is written for few instructions: the lanes stage column j of H (j + 2
+// entries) and the earlier rotations in shared memory; each rotation is three multiply-adds, lanes 0
+// .. 3 forming the real and imaginary parts of its two outputs; the new rotation's moduli and
+// quotients are formed side by side in different lanes; and est[j] = |g_{j+1}| / ||f|| is est[j-1]
+// times the new rotation's |s| = |b| / t.  (One lane doing all of it took 12.8 us per step at j = 13.)
 // est_host (may be null): pinned host memory, where est[j] is also stored, so that the host reads
 // the estimate once the step's event has fired, with no copy in the step (a device-to-host copy
 // node cost about 7 us per step at the end of every replayed step graph).
@@ -218,45 +298,65 @@ __device__ __forceinline__ void givens_body(double2 *H, int ldh, int j, double *
     __shared__ double2 colS[66], snS[64];
     __shared__ double csS[64];
     const int lane = threadIdx.x & 31;
+    constexpr unsigned all = 0xffffffffu;
     double2 *col = H + (size_t)ldh * j;
     for (int i = lane; i <= j + 1; i += 32) colS[i] = col[i];
     for (int i = lane; i < j; i += 32) {
         csS[i] = cs[i];
         snS[i] = sn[i];
     }
+    const double2 gj = g[j];
+    const double fnorm = fnorm_dev->x, before = j > 0 ? est[j - 1] : 0.0;
     __syncwarp();
+    double2 a = colS[0];
+    for (int i = 0; i < j; i++) {
+        const double2 b = colS[i + 1], s = snS[i];
+        const double c = csS[i];
+        // lanes 0, 1: c a + s b;  lanes 2, 3: c b - conj(s) a  (real, imaginary)
+        const bool im = lane & 1, second = lane & 2;
+        const double2 u = second ? b : a, v = second ? make_double2(-a.x, -a.y) : b;
+        const double p = im ? u.y : u.x, q = im ? v.y : v.x;
+        double r = im ? v.x : -v.y;
+        if (second) r = -r;
+        const double o = fma(c, p, fma(s.x, q, s.y * r));
+        if (lane < 2) ((double *)&colS[i])[lane] = o;
+        a = make_double2(__shfl_sync(all, o, 2), __shfl_sync(all, o, 3));
+    }
+    const double2 b = colS[j + 1];
+    __syncwarp();
+    // lane 0: |a|, lane 1: |b|
+    const double m = lane == 0 ? hypot(a.x, a.y) : hypot(b.x, b.y);
+    const double na = __shfl_sync(all, m, 0), nb = __shfl_sync(all, m, 1);
+    const double t = hypot(na, nb);
+    // lanes 0 .. 4: c = |a| / t, a / |a|, 1 / t, |s| = |b| / t;  lane 5 (j = 0): |g_0| / ||f||
+    const double num = lane == 0 ? na : lane == 1 ? a.x : lane == 2 ? a.y : lane == 3 ? 1.0 : lane == 4 ? nb : fabs(gj.x);
+    const double den = lane == 1 || lane == 2 ? na : lane == 5 ? fnorm : t;
+    const double quo = num / den;
+    double c = __shfl_sync(all, quo, 0);
+    const double2 ua = make_double2(__shfl_sync(all, quo, 1), __shfl_sync(all, quo, 2));
+    const double rt = __shfl_sync(all, quo, 3);
+    double sm = __shfl_sync(all, quo, 4);
+    const double e0 = __shfl_sync(all, quo, 5);
+    double2 s;
+    if (na == 0.0) {
+        c = 0.0;
+        s = make_double2(1.0, 0.0);
+        sm = 1.0;
+    } else {
+        s = cscale(cmul(ua, make_double2(b.x, -b.y)), rt);
+    }
     if (lane == 0) {
-        const double fnorm = fnorm_dev->x;
-        for (int i = 0; i < j; i++) {
-            const double2 a = colS[i], b = colS[i + 1];
-            const double c = csS[i];
-            const double2 s = snS[i];
-            colS[i] = cadd(cscale(a, c), cmul(s, b));
-            colS[i + 1] = csub(cscale(b, c), cmul(make_double2(s.x, -s.y), a));
-        }
-        const double2 a = colS[j], b = colS[j + 1];
-        const double na = hypot(a.x, a.y);
-        const double t = hypot(na, hypot(b.x, b.y));
-        double c;
-        double2 s;
-        if (na == 0.0) {
-            c = 0.0;
-            s = make_double2(1.0, 0.0);
-        } else {
-            c = na / t;
-            const double2 ua = make_double2(a.x / na, a.y / na);
-            s = cscale(cmul(ua, make_double2(b.x, -b.y)), 1.0 / t);
-        }
         cs[j] = c;
         sn[j] = s;
         colS[j] = cadd(cscale(a, c), cmul(s, b));
         colS[j + 1] = make_double2(0.0, 0.0);
-        const double2 gj = g[j];
-        g[j + 1] = cscale(cmul(make_double2(-s.x, s.y), gj), 1.0);
+        g[j + 1] = cmul(make_double2(-s.x, s.y), gj);
         g[j] = cscale(gj, c);
-        est[j] = hypot(g[j + 1].x, g[j + 1].y) / fnorm;
-        if (est_host) est_host[j] = est[j];
-        if (stop && !(est[j] > *tol)) *stop = 1;
+        // g_0 = (||r0||, 0)
+        const double e = (j > 0 ? before : e0) * sm;
+        est[j] = e;
+        if (est_host) est_host[j] = e;
+        if (stop && !(e > *tol)) *stop = 1;
     }
     __syncwarp();
     for (int i = lane; i <= j + 1; i += 32) col[i] = colS[i];
@@ -369,9 +469,7 @@ __global__ void __launch_bounds__(NT) k_backsolve(const double2 *H, int ldh, int
 
 // Bi-CGSTAB scalar block (device): 0 rho, 1 rho_old, 2 alpha, 3 omega, 4 beta, 5 <rh,v>,
 // 6 <t,s>, 7 <t,t>, 8 -alpha, 9 -omega, 10 one, 11 flags (x: breakdown)
-__global__ void k_bicg_scalars(int stage, double2 *sc) {
-    pdl_enter();
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__device__ __forceinline__ void bicg_stage(int stage, double2 *sc) {
     const double2 zero = make_double2(0.0, 0.0);
     auto isz = [](double2 v) { return v.x == 0.0 && v.y == 0.0; };
     if (stage == 0) {            // beta = (rho / rho_old) (alpha / omega)
@@ -392,23 +490,126 @@ __global__ void k_bicg_scalars(int stage, double2 *sc) {
         sc[11] = zero;
     }
 }
+__global__ void k_bicg_scalars(int stage, double2 *sc) {
+    pdl_enter();
+    if (threadIdx.x == 0 && blockIdx.x == 0) bicg_stage(stage, sc);
+}
 
+// The vector passes of an iteration, each one launch that also forms the inner products of what it
+// writes; the last block to finish sums the blocks' partials in a fixed order and takes the scalar
+// step (a dot, its reduction, the scalar kernel, the copy and the update as launches of their own
+// took 39 + 5 + 3 + 5 us of a 385^2 iteration's four dots; now five passes an iteration, the two
+// norms the host reads stored in pinned memory by the pass that forms them).
+
+// v[0 .. N) summed over the grid into sum[0 .. N) (shared memory) of the last block, which returns
+// true; partials: N x gridDim.x doubles.
+template <int N>
+__device__ __forceinline__ bool grid_sums(double (&v)[N], double *partials, unsigned *ticket, double (&sum)[N]) {
+    __shared__ double red[NT / 32][N];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = gridDim.x;
+    auto block = [&](double (&x)[N]) {
+        const int idx = warp_transpose_sum<N>(x);
+        if ((lane & (32 / N - 1)) == 0) red[warp][idx] = x[0];
+        __syncthreads();
+        double s = 0.0;
+        if (threadIdx.x < N)
+            for (int w = 0; w < NT / 32; w++) s += red[w][threadIdx.x];
+        __syncthreads();
+        return s;
+    };
+    const double s = block(v);
+    if (threadIdx.x < N) partials[(size_t)threadIdx.x * G + blockIdx.x] = s;
+    if (!last_block(ticket, G)) return false;
+    double t[N];
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+        t[k] = 0.0;
+        for (int b = threadIdx.x; b < G; b += NT) t[k] += __ldcg(&partials[(size_t)k * G + b]);
+    }
+    const double f = block(t);
+    if (threadIdx.x < N) sum[threadIdx.x] = f;
+    if (threadIdx.x == 0) *ticket = 0u;
+    __syncthreads();
+    return true;
+}
+
+// STAGE 1: <a, b> = <rh, v>, then alpha.  STAGE 2: <a, b> = <t, s> and <t, t>, then omega.
+template <int STAGE>
+__global__ void __launch_bounds__(NT) k_bicg_dots(size_t n, const double2 *__restrict__ a, const double2 *__restrict__ b,
+                                                  double2 *sc, double *partials, unsigned *ticket) {
+    pdl_enter();
+    constexpr int N = STAGE == 1 ? 2 : 4;
+    __shared__ double sum[N];
+    double v[N];
+#pragma unroll
+    for (int k = 0; k < N; k++) v[k] = 0.0;
+    for (size_t q = blockIdx.x * (size_t)NT + threadIdx.x; q < n; q += (size_t)gridDim.x * NT) {
+        const double2 x = a[q], y = b[q];
+        v[0] = fma(x.x, y.x, fma(x.y, y.y, v[0]));
+        v[1] = fma(x.x, y.y, fma(-x.y, y.x, v[1]));
+        if constexpr (STAGE == 2) v[2] = fma(x.x, x.x, fma(x.y, x.y, v[2]));
+    }
+    if (!grid_sums<N>(v, partials, ticket, sum) || threadIdx.x != 0) return;
+    sc[STAGE == 1 ? 5 : 6] = make_double2(sum[0], sum[1]);
+    if constexpr (STAGE == 2) sc[7] = make_double2(sum[2], 0.0);
+    bicg_stage(STAGE, sc);
+}
+
+// p = r + beta (p - omega v); with b_out, its complex64 copy (the next cycle's right-hand side)
 __global__ void k_bicg_p(size_t n, const double2 *__restrict__ r, const double2 *__restrict__ v,
-                         const double2 *__restrict__ sc, double2 *__restrict__ p) {
+                         const double2 *__restrict__ sc, double2 *__restrict__ p, float2 *__restrict__ b_out) {
     pdl_enter();
     const double2 beta = sc[4], om = sc[3];
     for (size_t q = blockIdx.x * (size_t)NT + threadIdx.x; q < n; q += (size_t)gridDim.x * NT) {
-        const double2 t = csub(p[q], cmul(om, v[q]));
-        p[q] = cfma(beta, t, r[q]);
+        const double2 t = cfma(beta, csub(p[q], cmul(om, v[q])), r[q]);
+        p[q] = t;
+        if (b_out) b_out[q] = to_c(t, 0.f);
     }
 }
 
-__global__ void k_axpby(size_t n, const double2 *__restrict__ a, const double2 *__restrict__ x,
-                        const double2 *__restrict__ b, double2 *__restrict__ y) {
+// s = r - alpha v and ||s||; host[0] = ||s||, host[1] = the breakdown flag (pinned)
+__global__ void __launch_bounds__(NT) k_bicg_s(size_t n, const double2 *__restrict__ r, const double2 *__restrict__ v,
+                                               double2 *sc, double2 *__restrict__ so, float2 *__restrict__ b_out,
+                                               double *partials, unsigned *ticket, double *host) {
     pdl_enter();
-    const double2 av = a[0], bv = b[0];
-    for (size_t q = blockIdx.x * (size_t)NT + threadIdx.x; q < n; q += (size_t)gridDim.x * NT)
-        y[q] = cfma(av, x[q], cmul(bv, y[q]));
+    __shared__ double sum[1];
+    const double2 na = sc[8];
+    double acc[1] = {0.0};
+    for (size_t q = blockIdx.x * (size_t)NT + threadIdx.x; q < n; q += (size_t)gridDim.x * NT) {
+        const double2 t = cfma(na, v[q], r[q]);
+        so[q] = t;
+        if (b_out) b_out[q] = to_c(t, 0.f);
+        acc[0] = fma(t.x, t.x, fma(t.y, t.y, acc[0]));
+    }
+    if (!grid_sums<1>(acc, partials, ticket, sum) || threadIdx.x != 0) return;
+    host[0] = sqrt(sum[0]);
+    host[1] = sc[11].x;
+}
+
+// x += alpha y + omega z; r = s - omega t; ||r||, <rh, r> -> the next iteration's rho and beta;
+// host[0] = ||r||, host[1] = the breakdown flag before that step (pinned)
+template <typename CY>
+__global__ void __launch_bounds__(NT) k_bicg_xr(size_t n, const CY *__restrict__ y, const CY *__restrict__ z,
+                                                const double2 *__restrict__ s, const double2 *__restrict__ t,
+                                                const double2 *__restrict__ rh, double2 *sc, double2 *__restrict__ x,
+                                                double2 *__restrict__ r, double *partials, unsigned *ticket, double *host) {
+    pdl_enter();
+    __shared__ double sum[4];
+    const double2 al = sc[2], om = sc[3], no = sc[9];
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    for (size_t q = blockIdx.x * (size_t)NT + threadIdx.x; q < n; q += (size_t)gridDim.x * NT) {
+        x[q] = cfma(om, to_c(z[q], 0.0), cfma(al, to_c(y[q], 0.0), x[q]));
+        const double2 rq = cfma(no, t[q], s[q]), h = rh[q];
+        r[q] = rq;
+        v[0] = fma(h.x, rq.x, fma(h.y, rq.y, v[0]));
+        v[1] = fma(h.x, rq.y, fma(-h.y, rq.x, v[1]));
+        v[2] = fma(rq.x, rq.x, fma(rq.y, rq.y, v[2]));
+    }
+    if (!grid_sums<4>(v, partials, ticket, sum) || threadIdx.x != 0) return;
+    host[0] = sqrt(sum[2]);
+    host[1] = sc[11].x;
+    sc[0] = make_double2(sum[0], sum[1]);
+    bicg_stage(0, sc);
 }
 
 template <typename CY>
@@ -483,16 +684,25 @@ unsigned stream_grid(size_t n) { return (unsigned)std::min<size_t>(cdiv(n, NT), 
 
 int blas_nblocks(size_t n) { return (int)std::min<size_t>(cdiv(n, NT), (size_t)MAXBLK); }
 
+// Two blocks per SM over all block rows.
+int mdot_nblocks(size_t n, int nv) {
+    if (nv <= 0) return blas_nblocks(n);
+    return (int)std::min<size_t>(cdiv(n, NT), (size_t)std::max(1, 2 * 152 / ((nv + 7) / 8)));
+}
+
 cudaError_t launch_mdot_norm(size_t n, const double2 *V, size_t ldv, int nv, const double2 *w, double2 *partials,
                              const int *gate, cudaStream_t s) {
-    if (nv < 0 || nv > 64) return cudaErrorInvalidValue;
-    if (nv == 0) {  // the norm alone: one value per block to reduce, not CH + 1
-        launch_pdl(k_mdot_norm<0>, dim3(blas_nblocks(n), 1), NT, 0, s, n, V, ldv, nv, w, partials, gate);
+    if (nv < 0 || nv > 64 || (nv == 0 && gate)) return cudaErrorInvalidValue;
+    const int G = mdot_nblocks(n, nv);
+    if (nv == 0) {  // the norm alone
+        launch_pdl(k_norm2, G, NT, 0, s, n, w, partials);
         return cudaGetLastError();
     }
-    constexpr int CH = 8;
-    dim3 g(blas_nblocks(n), std::max(1, (nv + CH - 1) / CH));
-    launch_pdl(k_mdot_norm<CH>, g, NT, 0, s, n, V, ldv, nv, w, partials, gate);
+    const int chunks = (nv + 7) / 8, most = (nv + chunks - 1) / chunks;
+    const dim3 g(G, chunks);
+    if (most <= 2) launch_pdl(k_mdot_norm<2>, g, NT, 0, s, n, V, ldv, nv, w, partials, gate);
+    else if (most <= 4) launch_pdl(k_mdot_norm<4>, g, NT, 0, s, n, V, ldv, nv, w, partials, gate);
+    else launch_pdl(k_mdot_norm<8>, g, NT, 0, s, n, V, ldv, nv, w, partials, gate);
     return cudaGetLastError();
 }
 
@@ -504,8 +714,8 @@ cudaError_t launch_update_norm(size_t n, const double2 *V, size_t ldv, int nv, c
 }
 
 cudaError_t launch_reduce(const double2 *partials, int nblk, int nv, double2 *out, int mode, const int *gate,
-                          cudaStream_t s, double *host_out) {
-    launch_pdl(k_reduce, nv, NT, 0, s, partials, nblk, out, mode, gate, host_out);
+                          cudaStream_t s, double *host_out, double2 *out2) {
+    launch_pdl(k_reduce, nv, NT, 0, s, partials, nblk, out, mode, gate, host_out, out2);
     return cudaGetLastError();
 }
 
@@ -515,8 +725,9 @@ cudaError_t launch_reduce_decide(const double2 *partials, int nblk, double2 *hno
     return cudaGetLastError();
 }
 
-cudaError_t launch_scale_inv(size_t n, const double2 *x, const double2 *scale, double2 *y, cudaStream_t s) {
-    launch_pdl(k_scale_inv, stream_grid(n), NT, 0, s, n, x, scale, y);
+cudaError_t launch_scale_inv(size_t n, const double2 *x, const double2 *scale, double2 *y, float2 *b_out,
+                             cudaStream_t s) {
+    launch_pdl(k_scale_inv, stream_grid(n), NT, 0, s, n, x, scale, y, b_out);
     return cudaGetLastError();
 }
 
@@ -598,17 +809,39 @@ cudaError_t launch_bicg_scalars(int stage, double2 *sc, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_bicg_p(size_t n, const double2 *r, const double2 *v, const double2 *sc, double2 *p,
+cudaError_t launch_bicg_p(size_t n, const double2 *r, const double2 *v, const double2 *sc, double2 *p, float2 *b_out,
                           cudaStream_t s) {
-    launch_pdl(k_bicg_p, stream_grid(n), NT, 0, s, n, r, v, sc, p);
+    launch_pdl(k_bicg_p, stream_grid(n), NT, 0, s, n, r, v, sc, p, b_out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_axpby(size_t n, const double2 *a, const double2 *x, const double2 *b, double2 *y,
-                         cudaStream_t s) {
-    launch_pdl(k_axpby, stream_grid(n), NT, 0, s, n, a, x, b, y);
+cudaError_t launch_bicg_dots(int stage, size_t n, const double2 *a, const double2 *b, double2 *sc, double2 *partials,
+                             unsigned *ticket, cudaStream_t s) {
+    double *pd = (double *)partials;
+    if (stage == 1) launch_pdl(k_bicg_dots<1>, blas_nblocks(n), NT, 0, s, n, a, b, sc, pd, ticket);
+    else launch_pdl(k_bicg_dots<2>, blas_nblocks(n), NT, 0, s, n, a, b, sc, pd, ticket);
     return cudaGetLastError();
 }
+
+cudaError_t launch_bicg_s(size_t n, const double2 *r, const double2 *v, double2 *sc, double2 *so, float2 *b_out,
+                          double2 *partials, unsigned *ticket, double *host, cudaStream_t s) {
+    launch_pdl(k_bicg_s, blas_nblocks(n), NT, 0, s, n, r, v, sc, so, b_out, (double *)partials, ticket, host);
+    return cudaGetLastError();
+}
+
+template <typename CY>
+cudaError_t launch_bicg_xr(size_t n, const CY *y, const CY *z, const double2 *so, const double2 *t, const double2 *rh,
+                           double2 *sc, double2 *x, double2 *r, double2 *partials, unsigned *ticket, double *host,
+                           cudaStream_t s) {
+    launch_pdl(k_bicg_xr<CY>, blas_nblocks(n), NT, 0, s, n, y, z, so, t, rh, sc, x, r, (double *)partials, ticket, host);
+    return cudaGetLastError();
+}
+template cudaError_t launch_bicg_xr<float2>(size_t, const float2 *, const float2 *, const double2 *, const double2 *,
+                                            const double2 *, double2 *, double2 *, double2 *, double2 *, unsigned *,
+                                            double *, cudaStream_t);
+template cudaError_t launch_bicg_xr<double2>(size_t, const double2 *, const double2 *, const double2 *, const double2 *,
+                                             const double2 *, double2 *, double2 *, double2 *, double2 *, unsigned *,
+                                             double *, cudaStream_t);
 
 template <typename CY>
 cudaError_t launch_axpy_mixed(size_t n, const double2 *a, const CY *x, double2 *y, cudaStream_t s) {

@@ -176,7 +176,7 @@ static cudaError_t dev_dot(helm_handle *h, const double2 *a, const double2 *b, d
     ProfScope ps(h, HELM_K_VECTOR, h->np * 32.0, h->np * 12.0);
     cudaError_t e = launch_mdot_norm(h->np, a, h->np, 1, b, h->partials, nullptr, h->stream);
     if (e != cudaSuccess) return e;
-    return launch_reduce(h->partials, blas_nblocks(h->np), 1, out, 0, nullptr, h->stream);
+    return launch_reduce(h->partials, mdot_nblocks(h->np, 1), 1, out, 0, nullptr, h->stream);
 }
 
 static helm_status read_scalars(helm_handle *h, const void *dev, size_t bytes, void *host) {
@@ -240,12 +240,19 @@ static cudaError_t precond_apply_level0(helm_handle *h, float2 *z, float4 *w, co
 // meets the tolerance, cleared at the start of every cycle.
 static int *stop_flag(helm_handle *h) { return h->gs_flag + 2; }
 
-// z = precondition(v) in the workspace precision; w = A z (FP64)
+// FP64 Arnoldi with a complex64 cycle: every basis vector's complex64 copy is written into level 0's
+// right-hand side by the pass that normalises it.
+static bool fp64_fold(const helm_handle *h) {
+    return h->mg.gs_arith == HELM_GS_FP64 && h->z_prec == HELM_C64 && h->mg.kind != HELM_PC_NONE;
+}
+
+// z = precondition(v) in the workspace precision (v null: complex64 of what level 0's right-hand
+// side holds); w = A z (FP64)
 static cudaError_t precond_apply(helm_handle *h, const double2 *v, void *z, double2 *w) {
     cudaError_t e;
     const double ni = interior_pts(h);
     if (h->z_prec == HELM_C64) {
-        e = precondition<float>(h, v, (float2 *)z);
+        e = v ? precondition<float>(h, v, (float2 *)z) : precondition_level0_c64(h, (float2 *)z);
         if (e != cudaSuccess) return e;
         ProfScope ps(h, HELM_K_APPLY, ni * (8 + 8 + 16), apply_flops(h));
         return launch_apply<double, float2>(h->A64, h->dim, (const float2 *)z, w, h->stream);
@@ -276,7 +283,7 @@ static cudaError_t fgmres_step(helm_handle *h, int j, int m) {
     // Gram-Schmidt passes in FP64, or in double-FP32 on float-pair basis vectors (same
     // partials layout)
     const bool df = h->mg.gs_arith == HELM_GS_DF;
-    const int gblk = df ? gs_df_nblocks(np) : blas_nblocks(np);         // blocks of the dot pass
+    const int gblk = df ? gs_df_nblocks(np) : mdot_nblocks(np, j + 1);  // blocks of the dot pass
     const int ublk = df ? gs_df_update_nblocks(np) : blas_nblocks(np);  // blocks of the update pass
     const float4 *V4 = (const float4 *)h->V;
     auto gs_dot = [&](int nv, double2 *w, const int *gate) {
@@ -289,8 +296,9 @@ static cudaError_t fgmres_step(helm_handle *h, int j, int m) {
     };
     double2 *vj = h->V + (size_t)j * np, *w = h->V + (size_t)(j + 1) * np;
     void *zj = (char *)h->Z + (size_t)j * np * zsz;
+    // the pass that normalised v_j left its complex64 copy in level 0's right-hand side
     if (df) CKE(precond_apply_pair(h, (const float4 *)vj, nullptr, zj, (float4 *)w));
-    else CKE(precond_apply(h, vj, zj, w));
+    else CKE(precond_apply(h, fp64_fold(h) ? nullptr : vj, zj, w));
     double2 *hcol = h->H + (size_t)ldh * j;
     const double nv = j + 1;
     // Classical Gram-Schmidt with the DGKS re-orthogonalisation test:
@@ -303,10 +311,12 @@ static cudaError_t fgmres_step(helm_handle *h, int j, int m) {
         CKE(gs_dot(j + 1, w, nullptr));
     }
     {
+        pdl_cycle_scope pdl;  // a few blocks, placed while the dot pass drains
         ProfScope ps(h, HELM_K_SMALL, 0, 0);
         CKE(launch_reduce(h->partials, gblk, j + 2, hcol, 0, nullptr, s));
     }
     {
+        pdl_cycle_scope pdl;  // placed while the reduction's few blocks finish
         ProfScope ps(h, HELM_K_UPDATE_NORM, np * 16.0 * (nv + 2), df ? 0.0 : np * (8.0 * nv + 4.0));
         CKE(gs_update(j + 1, hcol, w, nullptr));
     }
@@ -328,11 +338,12 @@ static cudaError_t fgmres_step(helm_handle *h, int j, int m) {
         CKE(gs_dot(j + 1, w, h->gs_flag));
     }
     {
+        pdl_cycle_scope pdl;
         ProfScope ps(h, HELM_K_SMALL, 0, 0);
-        CKE(launch_reduce(h->partials, gblk, j + 1, h->h2, 0, h->gs_flag, s));
-        CKE(launch_reduce(h->partials, gblk, j + 1, hcol, 1, h->gs_flag, s));
+        CKE(launch_reduce(h->partials, gblk, j + 1, hcol, 1, h->gs_flag, s, nullptr, h->h2));
     }
     {
+        pdl_cycle_scope pdl;
         ProfScope ps(h, HELM_K_UPDATE_NORM, pass2 * np * 16.0 * (nv + 2), df ? 0.0 : pass2 * np * (8.0 * nv + 4.0));
         CKE(gs_update(j + 1, h->h2, w, h->gs_flag));
     }
@@ -343,7 +354,7 @@ static cudaError_t fgmres_step(helm_handle *h, int j, int m) {
     {
         ProfScope ps(h, HELM_K_VECTOR, np * 32.0, df ? 0.0 : np * 2.0);
         if (df) CKE(launch_scale_inv_pair(np, (float4 *)w, hcol + j + 1, s));
-        else CKE(launch_scale_inv(np, w, hcol + j + 1, w, s));
+        else CKE(launch_scale_inv(np, w, hcol + j + 1, w, fp64_fold(h) ? level0_rhs_c64(h) : nullptr, s));
     }
     {
         ProfScope ps(h, HELM_K_SMALL, 0, 0);
@@ -623,7 +634,7 @@ helm_status fgmres_advance(FgmresRun &r, bool block) {
             r.restarts++;
             // v_0 = r0 / beta (as a float-pair vector for the double-FP32 Arnoldi)
             if (h->mg.gs_arith != HELM_GS_FP64) CKR(launch_split_scale(np, h->V, h->scal, s));
-            else CKR(launch_scale_inv(np, h->V, h->scal, h->V, s));
+            else CKR(launch_scale_inv(np, h->V, h->scal, h->V, fp64_fold(h) ? level0_rhs_c64(h) : nullptr, s));
             // g = beta e_1; the cycle's stop flag cleared and the tolerance it is tested against set
             CKR(launch_cycle_start(h->g, m + 1, h->scal, stop_flag(h), h->tol_dev, r.tol, s));
             r.jmax = std::min(m, r.maxit - r.it);
@@ -731,24 +742,23 @@ static helm_status bicgstab(helm_handle *h, const double2 *f, double2 *x, double
     int it = 0;
     helm_status status = est <= tol ? HELM_OK : HELM_ERR_NOCONV;
     const bool c64 = h->z_prec == HELM_C64;
-    while (status == HELM_ERR_NOCONV && it < maxit) {
+    // a complex64 cycle's right-hand side (p, then s) is rounded by the pass that forms the vector
+    float2 *b32 = c64 ? level0_rhs_c64(h) : nullptr;
+    double *host = h->est_host;
+    unsigned *ticket = h->tickets + 2;
+    if (status == HELM_ERR_NOCONV) {
         CKR(dev_dot(h, h->brh, h->br, sc + 0));                                   // rho
         CKR(launch_bicg_scalars(0, sc, s));                                       // beta
-        CKR(launch_bicg_p(np, h->br, h->bv, sc, h->bp, s));                       // p
-        CKR(precond_apply(h, h->bp, h->by, h->bv));                               // y = M p, v = A y
-        CKR(dev_dot(h, h->brh, h->bv, sc + 5));                                   // <rh, v>
-        CKR(launch_bicg_scalars(1, sc, s));                                       // alpha
-        CKR(cudaMemcpyAsync(h->bs, h->br, np * sizeof(double2), cudaMemcpyDeviceToDevice, s));
-        CKR(launch_axpby(np, sc + 8, h->bv, sc + 10, h->bs, s));                  // s = r - alpha v
-        CKR(dev_norm(h, h->bs, nrm));
-        double2 hs[12];
-        CKR(cudaMemcpyAsync(h->est_host, nrm, sizeof(double2), cudaMemcpyDeviceToHost, s));
-        CKR(cudaMemcpyAsync(h->est_host + 2, sc + 11, sizeof(double2), cudaMemcpyDeviceToHost, s));
+    }
+    while (status == HELM_ERR_NOCONV && it < maxit) {
+        CKR(launch_bicg_p(np, h->br, h->bv, sc, h->bp, b32, s));                  // p
+        CKR(precond_apply(h, c64 ? nullptr : h->bp, h->by, h->bv));               // y = M p, v = A y
+        CKR(launch_bicg_dots(1, np, h->brh, h->bv, sc, h->partials, ticket, s));  // <rh, v>, alpha
+        CKR(launch_bicg_s(np, h->br, h->bv, sc, h->bs, b32, h->partials, ticket, host, s));  // s = r - alpha v
         CKR(cudaStreamSynchronize(s));
-        memcpy(hs, h->est_host, 2 * sizeof(double2));
         it++;
-        if (hs[1].x != 0.0) { status = HELM_ERR_BREAKDOWN; break; }
-        est = hs[0].x / fn;
+        if (host[1] != 0.0) { status = HELM_ERR_BREAKDOWN; break; }
+        est = host[0] / fn;
         if (!std::isfinite(est)) { status = HELM_ERR_NONFINITE; break; }
         if (est <= tol) {                                                         // x += alpha y
             if (c64) CKR(launch_axpy_mixed<float2>(np, sc + 2, (const float2 *)h->by, x, s));
@@ -757,29 +767,20 @@ static helm_status bicgstab(helm_handle *h, const double2 *f, double2 *x, double
             if (st && st->history && it - 1 < st->history_len) st->history[it - 1] = est;
             break;
         }
-        CKR(precond_apply(h, h->bs, h->bz, h->bt));                               // z = M s, t = A z
-        CKR(dev_dot(h, h->bt, h->bs, sc + 6));                                    // <t, s>
-        CKR(dev_dot(h, h->bt, h->bt, sc + 7));                                    // <t, t>
-        CKR(launch_bicg_scalars(2, sc, s));                                       // omega
-        if (c64) {
-            CKR(launch_axpy_mixed<float2>(np, sc + 2, (const float2 *)h->by, x, s));
-            CKR(launch_axpy_mixed<float2>(np, sc + 3, (const float2 *)h->bz, x, s));
-        } else {
-            CKR(launch_axpy_mixed<double2>(np, sc + 2, (const double2 *)h->by, x, s));
-            CKR(launch_axpy_mixed<double2>(np, sc + 3, (const double2 *)h->bz, x, s));
-        }
-        CKR(cudaMemcpyAsync(h->br, h->bs, np * sizeof(double2), cudaMemcpyDeviceToDevice, s));
-        CKR(launch_axpby(np, sc + 9, h->bt, sc + 10, h->br, s));                  // r = s - omega t
-        CKR(dev_norm(h, h->br, nrm));
-        CKR(cudaMemcpyAsync(h->est_host, nrm, sizeof(double2), cudaMemcpyDeviceToHost, s));
-        CKR(cudaMemcpyAsync(h->est_host + 2, sc + 11, sizeof(double2), cudaMemcpyDeviceToHost, s));
+        CKR(precond_apply(h, c64 ? nullptr : h->bs, h->bz, h->bt));               // z = M s, t = A z
+        CKR(launch_bicg_dots(2, np, h->bt, h->bs, sc, h->partials, ticket, s));   // <t, s>, <t, t>, omega
+        if (c64)                                                                  // x, r = s - omega t, rho, beta
+            CKR(launch_bicg_xr<float2>(np, (const float2 *)h->by, (const float2 *)h->bz, h->bs, h->bt, h->brh, sc, x,
+                                       h->br, h->partials, ticket, host, s));
+        else
+            CKR(launch_bicg_xr<double2>(np, (const double2 *)h->by, (const double2 *)h->bz, h->bs, h->bt, h->brh, sc, x,
+                                        h->br, h->partials, ticket, host, s));
         CKR(cudaStreamSynchronize(s));
-        memcpy(hs, h->est_host, 2 * sizeof(double2));
-        est = hs[0].x / fn;
+        est = host[0] / fn;
         if (st && st->history && it - 1 < st->history_len) st->history[it - 1] = est;
         if (!std::isfinite(est)) { status = HELM_ERR_NONFINITE; break; }
         if (est <= tol) { status = HELM_OK; break; }
-        if (hs[1].x != 0.0) { status = HELM_ERR_BREAKDOWN; break; }
+        if (host[1] != 0.0) { status = HELM_ERR_BREAKDOWN; break; }
     }
     // true residual
     CKR(launch_residual<double, double2>(h->A64, h->dim, f, x, h->br, s));
