@@ -745,7 +745,9 @@ static cudaError_t cycle(helm_handle *h, int l, const typename CT<R>::T *b, type
     CKE(smooth<R>(h, l, nu1, b, &cur, &oth, zero));
     {
         ProfScope ps(h, HELM_K_RESTRICT, ni * (2 * es + rs + es / nd), 0);
-        CKE(launch_residual_restrict<R>(LvBuf<R>::op(L), h->dim, b, cur, LvBuf<R>::b(Lc), h->stream));
+        const bool red = rb && h->mg.omega == 1.0 && nu1 > 0;
+        CKE(launch_residual_restrict<R>(LvBuf<R>::op(L), h->dim, b, cur, LvBuf<R>::b(Lc), h->stream, red,
+                                        red && nu1 == 1 && zero));
     }
     CKE(coarse());
     {

@@ -47,6 +47,20 @@ __device__ __forceinline__ float2 cinv_fast(float2 a) {
     const float r = __fdividef(1.0f, fmaf(a.x, a.x, a.y * a.y));
     return make_float2(a.x * r, -a.y * r);
 }
+// True when v is +0 or -0 (an integer test: comparisons of doubles run on the FP64 units).
+__device__ __forceinline__ bool is_zero(double v) { return ((unsigned long long)__double_as_longlong(v) << 1) == 0ull; }
+__device__ __forceinline__ bool is_zero(float v) { return (__float_as_uint(v) << 1) == 0u; }
+// acc + cw xw + ce xe for one axis of the stencil.  Outside the absorbing layers the coefficients of A,
+// and of the preconditioners that do not rotate the widths, are real (REAL): half the multiply-adds.
+// A compile-time choice: as a run-time branch the compiler issues both forms.
+template <bool REAL, typename C> __device__ __forceinline__ C axis_add(C cw, C ce, C xw, C xe, C acc) {
+    if (REAL) return mk(fma(cw.x, xw.x, fma(ce.x, xe.x, acc.x)), fma(cw.x, xw.y, fma(ce.x, xe.y, acc.y)));
+    return cfma(ce, xe, cfma(cw, xw, acc));
+}
+// acc - cw xw - ce xe
+template <bool REAL, typename C> __device__ __forceinline__ C axis_sub(C cw, C ce, C xw, C xe, C acc) {
+    return axis_add<REAL>(mk(-cw.x, -cw.y), mk(-ce.x, -ce.y), xw, xe, acc);
+}
 // dst[q] = src[q] for q < n (src global and unchanged during the kernel, dst this block's
 // shared memory): each thread issues eight loads before it stores, so that a block's copy takes
 // a few memory round trips instead of one per float4 a thread moves.
@@ -181,10 +195,12 @@ cudaError_t launch_jacobi(const DevOp<R> &op, int dim, R omega, const CB *b, con
 template <typename R, typename CB>
 cudaError_t launch_rb(const DevOp<R> &op, int dim, R omega, const CB *b, typename CT<R>::T *u, int colour, int zero,
                       cudaStream_t s);
-// rc = FW(b - M u) on the coarse grid (fine nodes op.n, coarse nodes (n+1)/2).
+// rc = FW(b - M u) on the coarse grid (fine nodes op.n, coarse nodes (n+1)/2).  red: u comes from a
+// red-black sweep with omega = 1, so that the residual of the second colour is zero; first: that sweep
+// was the first from zero (3D uses both; 2D forms every residual).
 template <typename R, typename CB>
 cudaError_t launch_residual_restrict(const DevOp<R> &op, int dim, const CB *b, const typename CT<R>::T *u,
-                                     typename CT<R>::T *rc, cudaStream_t s);
+                                     typename CT<R>::T *rc, cudaStream_t s, bool red = false, bool first = false);
 // uf += P ec (fine nodes nf).
 template <typename R>
 cudaError_t launch_prolong_add(const int nf[3], int dim, const typename CT<R>::T *ec, typename CT<R>::T *uf,

@@ -180,12 +180,22 @@ template <typename C> __device__ __forceinline__ C dinv_at(const Ctx &X, const L
 }
 
 // The off-diagonal part of (M u) at node (j, q) from this block's rows of the array at offset u
-// (j - 1 and j + 1 may be halo rows).
+// (j - 1 and j + 1 may be halo rows); complex128: acc0 minus that part.
 template <typename C, int DIM>
-__device__ __forceinline__ C offdiag_at(const Ctx &X, const LV &L, unsigned u, int j, int q, int i, int y) {
+__device__ __forceinline__ C offdiag_at(const Ctx &X, const LV &L, unsigned u, int j, int q, int i, int y, C acc0) {
     const C *cx = (const C *)(X.sm + L.ocx), *cs = (const C *)(X.sm + L.ocs);
     const int li = j - L.j0;
     const C *un = lrow<C>(X, L, u, j - 1), *uc = lrow<C>(X, L, u, j), *us = lrow<C>(X, L, u, j + 1);
+    if constexpr (sizeof(acc0) == sizeof(double2)) {
+        const C w0 = cx[3 * i], e0 = cx[3 * i + 2], w2 = cs[3 * li], e2 = cs[3 * li + 2];
+        C acc = axis_sub<false>(w0, e0, uc[q - 1], uc[q + 1], acc0);
+        if constexpr (DIM == 3) {
+            const C *cy = (const C *)(X.sm + L.ocy);
+            const C w1 = cy[3 * y], e1 = cy[3 * y + 2];
+            acc = axis_sub<false>(w1, e1, uc[q - L.nx], uc[q + L.nx], acc);
+        }
+        return axis_sub<false>(w2, e2, un[q], us[q], acc);
+    }
     C acc = cmul(cx[3 * i], uc[q - 1]);
     acc = cfma(cx[3 * i + 2], uc[q + 1], acc);
     if constexpr (DIM == 3) {
@@ -202,11 +212,10 @@ __device__ __forceinline__ typename CT<R>::T relax_at(const Ctx &X, const LV &L,
                                                       R om) {
     typedef typename CT<R>::T C;
     const C b = lrow<C>(X, L, L.ob, j)[q], uc = lrow<C>(X, L, u, j)[q], di = dinv_at<C>(X, L, j, q);
-    const C off = offdiag_at<C, DIM>(X, L, u, j, q, i, y);
+    const C off = offdiag_at<C, DIM>(X, L, u, j, q, i, y, b);
     if constexpr (sizeof(R) == sizeof(double)) {
-        // (1 - omega) u + (omega / D) (b - off)
-        const C r = csub(b, off);
-        return cfma(di, r, cscale(uc, R(1) - om));
+        // (1 - omega) u + (omega / D) (b - offdiagonal part)
+        return cfma(di, off, cscale(uc, R(1) - om));
     } else {
         const C mu = cfma(diag_at<C>(X, L, j, q), uc, off);
         return cadd(uc, cscale(cmul(csub(b, mu), di), om));
@@ -273,13 +282,25 @@ template <typename C, int DIM> __device__ __forceinline__ C w121_row(const C *r,
 
 // Residual of level l (iterate u) into r, then full weighting into level l + 1's b (the fine
 // rows 2J-1 .. 2J+1 of an owned coarse row J are owned or halo rows: nested slabs).
+// first: u is one sweep from zero, so that D u = omega b (red-black: omega (b - offdiagonal part) at the
+// second colour) and complex128 needs no diagonal term.
 template <typename R, int DIM>
-__device__ __noinline__ void ph_restrict(Ctx X, const CArgs<R> *A, int l, unsigned u, unsigned r) {
+__device__ __noinline__ void ph_restrict(Ctx X, const CArgs<R> *A, int l, unsigned u, unsigned r, bool first) {
     typedef typename CT<R>::T C;
     const LV L = lv_of(X, A->lv[l]), Lc = lv_of(X, A->lv[l + 1]);
+    const R q1 = R(1) - A->omega;
+    const bool rb = A->rb != 0;
     for_owned<DIM>(X, L, [&](int j, int q, int i, int y) {
-        const C mu = cfma(diag_at<C>(X, L, j, q), lrow<C>(X, L, u, j)[q], offdiag_at<C, DIM>(X, L, u, j, q, i, y));
-        put(X, L, r, j, q, csub(lrow<C>(X, L, L.ob, j)[q], mu), X.rank);
+        const C b = lrow<C>(X, L, L.ob, j)[q];
+        C v;
+        if constexpr (sizeof(R) == sizeof(double)) {
+            if (!first) v = csub(offdiag_at<C, DIM>(X, L, u, j, q, i, y, b), cmul(diag_at<C>(X, L, j, q), lrow<C>(X, L, u, j)[q]));
+            else if (rb && ((i + y + j) & 1)) v = cscale(offdiag_at<C, DIM>(X, L, u, j, q, i, y, b), q1);
+            else v = offdiag_at<C, DIM>(X, L, u, j, q, i, y, cscale(b, q1));
+        } else {
+            v = csub(b, cfma(diag_at<C>(X, L, j, q), lrow<C>(X, L, u, j)[q], offdiag_at<C, DIM>(X, L, u, j, q, i, y, b)));
+        }
+        put(X, L, r, j, q, v, X.rank);
     });
     csync();
     for_owned<DIM>(X, Lc, [&](int J, int Q, int I, int Y) {
@@ -390,7 +411,7 @@ __device__ __noinline__ void ct_cycle(Ctx X, const CArgs<R> *A, bool zero, int g
     }
     if constexpr (LVL + 1 < MAX_CT_LEVELS) {
         uint2 co = ph_smooth<R, DIM>(X, A, LVL, A->nu1, make_uint2(L.ou, L.ot), zero);
-        ph_restrict<R, DIM>(X, A, LVL, co.x, co.y);
+        ph_restrict<R, DIM>(X, A, LVL, co.x, co.y, zero && A->nu1 == 1);
         if (LVL + 1 == A->nlev - 1) {
             ph_dense<R, DIM>(X, A, LVL + 1);
         } else {

@@ -50,24 +50,23 @@ __device__ __forceinline__ void block_sum(double2 (&v)[NV], double2 *out_shared)
 // plain levels additions per lane instead of 5 N; on the FP64 units, where a warp's instruction takes
 // 64 clocks of its scheduler, 5 N additions for 9 complex values cost more than the pass itself).
 // Lanes l with l % (32 / N) == 0 end with the sum of value idx in v[0].
-template <int N> __device__ __forceinline__ int warp_transpose_sum(double (&v)[N]) {
-    const int lane = threadIdx.x & 31;
-    int idx = 0;
+template <int M, int O, int N> __device__ __forceinline__ void transpose_level(double (&v)[N], int lane, int &idx) {
+    if constexpr (M > 1) {
+        const bool upper = (lane & O) != 0;
 #pragma unroll
-    for (int o = 16, m = N; o > 0; o >>= 1) {
-        if (m > 1) {
-            const bool upper = (lane & o) != 0;
-#pragma unroll
-            for (int i = 0; i < m / 2; i++) {
-                const double keep = upper ? v[i + m / 2] : v[i], send = upper ? v[i] : v[i + m / 2];
-                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-            }
-            if (upper) idx += m / 2;
-            m /= 2;
-        } else {
-            v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+        for (int i = 0; i < M / 2; i++) {
+            const double keep = upper ? v[i + M / 2] : v[i], send = upper ? v[i] : v[i + M / 2];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
         }
+        if (upper) idx += M / 2;
+    } else {
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
     }
+    if constexpr (O > 1) transpose_level<(M > 1 ? M / 2 : 1), O / 2>(v, lane, idx);
+}
+template <int N> __device__ __forceinline__ int warp_transpose_sum(double (&v)[N]) {
+    int idx = 0;
+    transpose_level<N, 16>(v, threadIdx.x & 31, idx);
     return idx;
 }
 

@@ -95,37 +95,75 @@ __device__ __forceinline__ typename CT<R>::T apply_point(const OpView<R> &o, con
     const size_t sz = (size_t)(o).nx * (o).ny;                      \
     size_t p = (size_t)i + (size_t)(o).nx * ((size_t)j + (size_t)(o).ny * k0);
 
-template <typename R, int DIM, typename CX>
-__global__ void __launch_bounds__(BX *BY) k_apply(OpView<R> o, const CX *__restrict__ x, typename CT<R>::T *__restrict__ y) {
-    pdl_enter();
+// y = M x, or with RES y = b - M x; each thread marches kc planes in 3D with its x and y coefficients
+// in registers.  complex128 is bound by the FP64 units (two lanes per SM and clock): 36 operations per
+// node in 3D, but 16 where every axis is outside the layers, since those coefficients of A are real.
+// Each warp picks the form by axis (x: all its columns, y: its row, z: all its planes), once, so that
+// every form is a loop of its own.  Measured, A x in complex128 on 225 x 193 x 161 nodes: 406 us with
+// every term complex, 321 us so (543 us with the form chosen by a branch at every node).
+template <typename R, int DIM, typename CX, typename CB, bool RES, bool RX, bool RY, bool RZ>
+__device__ __forceinline__ void apply_march(const OpView<R> &o, const CB *__restrict__ b, const CX *__restrict__ x,
+                                            typename CT<R>::T *__restrict__ y, int i, int j, int k0, int k1) {
     typedef typename CT<R>::T C;
-    INTERIOR_IJ(o);
-    C xm = mk(R(0), R(0)), xc = to_c(x[p], R()), xp = mk(R(0), R(0));
+    constexpr bool RD = RX && RY && RZ;
+    const size_t sy = (size_t)o.nx, sz = sy * o.ny;
+    size_t p = (size_t)i + sy * ((size_t)j + (size_t)o.ny * k0);
+    const C cwx = __ldg(&o.cx[3 * i]), cex = __ldg(&o.cx[3 * i + 2]), cwy = __ldg(&o.cy[3 * j]), cey = __ldg(&o.cy[3 * j + 2]);
+    const C dxy = cadd(cadd(__ldg(&o.cx[3 * i + 1]), __ldg(&o.cy[3 * j + 1])), o.c);
+    C xm = mk(R(0), R(0)), xc = to_c(x[p], R()), xp = xm;
     if (DIM == 3) xm = to_c(x[p - sz], R());
     for (int k = k0; k < k1; k++, p += sz) {
         if (DIM == 3) xp = to_c(x[p + sz], R());
-        C d;
-        y[p] = stencil<R, DIM>(o, x, p, i, j, k, xm, xc, xp, d);
+        const R kq = o.k2[p];
+        C d = dxy, acc = mk(R(0), R(0));
+        if (DIM == 3) {
+            const C ccz = __ldg(&o.cz[3 * k + 1]);
+            d = RD ? mk(d.x + ccz.x, R(0)) : cadd(d, ccz);
+            acc = axis_add<RZ>(__ldg(&o.cz[3 * k]), __ldg(&o.cz[3 * k + 2]), xm, xp, acc);
+        }
+        acc = axis_add<RX>(cwx, cex, to_c(x[p - 1], R()), to_c(x[p + 1], R()), acc);
+        acc = axis_add<RY>(cwy, cey, to_c(x[p - sy], R()), to_c(x[p + sy], R()), acc);
+        d.x = fma(o.bk.x, kq, d.x);
+        if (RD) {
+            acc = mk(fma(d.x, xc.x, acc.x), fma(d.x, xc.y, acc.y));
+        } else {
+            d.y = fma(o.bk.y, kq, d.y);
+            acc = cfma(d, xc, acc);
+        }
+        y[p] = RES ? csub(to_c(b[p], R()), acc) : acc;
         if (DIM == 3) { xm = xc; xc = xp; }
     }
 }
 
-template <typename R, int DIM, typename CB>
-__global__ void __launch_bounds__(BX *BY) k_residual(OpView<R> o, const CB *__restrict__ b, const typename CT<R>::T *__restrict__ u,
-                                                     typename CT<R>::T *__restrict__ r) {
+template <typename R, int DIM, typename CX, typename CB, bool RES>
+__global__ void __launch_bounds__(BX *BY) k_apply(OpView<R> o, const CB *__restrict__ b, const CX *__restrict__ x,
+                                                  typename CT<R>::T *__restrict__ y, int kc) {
     pdl_enter();
-    if (o.gate && *o.gate) return;
-    typedef typename CT<R>::T C;
-    INTERIOR_IJ(o);
-    C xm = mk(R(0), R(0)), xc = u[p], xp = mk(R(0), R(0));
-    if (DIM == 3) xm = u[p - sz];
-    for (int k = k0; k < k1; k++, p += sz) {
-        if (DIM == 3) xp = u[p + sz];
-        C d;
-        C mu = stencil<R, DIM>(o, u, p, i, j, k, xm, xc, xp, d);
-        r[p] = csub(to_c(b[p], R()), mu);
-        if (DIM == 3) { xm = xc; xc = xp; }
+    if (RES && o.gate && *o.gate) return;
+    const int i = blockIdx.x * BX + threadIdx.x + 1;
+    const int j = blockIdx.y * BY + threadIdx.y + 1;
+    if (i > o.nx - 2 || j > o.ny - 2) return;
+    int k0 = 0, k1 = 1;
+    if (DIM == 3) {
+        k0 = blockIdx.z * kc + 1;
+        k1 = min(k0 + kc, o.nz - 1);
     }
+    if constexpr (sizeof(R) == sizeof(double)) {
+        auto real3 = [](const double2 *t) {
+            return is_zero(__ldg(&t[0].y)) && is_zero(__ldg(&t[1].y)) && is_zero(__ldg(&t[2].y));
+        };
+        if (is_zero(o.bk.y) && is_zero(o.c.y)) {
+            const bool rx = __all_sync(__activemask(), real3(o.cx + 3 * i)), ry = real3(o.cy + 3 * j);
+            bool rz = true;
+            if (DIM == 3)
+                for (int k = k0; k < k1; k++) rz = rz && real3(o.cz + 3 * k);
+            if (rx && ry && rz) return apply_march<R, DIM, CX, CB, RES, true, true, true>(o, b, x, y, i, j, k0, k1);
+            if (rx && ry) return apply_march<R, DIM, CX, CB, RES, true, true, false>(o, b, x, y, i, j, k0, k1);
+            if (rx && rz) return apply_march<R, DIM, CX, CB, RES, true, false, true>(o, b, x, y, i, j, k0, k1);
+            if (ry && rz) return apply_march<R, DIM, CX, CB, RES, false, true, true>(o, b, x, y, i, j, k0, k1);
+        }
+    }
+    apply_march<R, DIM, CX, CB, RES, false, false, false>(o, b, x, y, i, j, k0, k1);
 }
 
 // omega-Jacobi: every unknown from the previous iterate (ping-pong buffers).
@@ -484,6 +522,78 @@ __global__ void __launch_bounds__(R3_NT, sizeof(R) == sizeof(float) ? 2 : 1)
                 acc = v;
             } else {
                 acc = cadd(acc, cscale(v, R(2)));
+            }
+        }
+    }
+}
+
+// 3D residual + full weighting after a red-black sweep with omega = 1, whose second colour (odd
+// i + j + k) ends with zero residuals: only the first colour's residuals are formed, one thread per
+// red node of a plane of the region (the same tiles as k_resrestrict3), and the weights take only
+// them.  first: the sweep was the first from zero, so D u = b at the red nodes and their residual is
+// minus the off-diagonal part.  Bound by the FP64 units in complex128: 28 (first) or 36 operations for
+// half of the nodes.
+// Measured, 193 x 129 x 97 complex128 V(1,1) cycle: 719 us with every residual formed (277 us of it on
+// the finest level), 505 us so.
+constexpr int R3R_HW = R3_TX + 1, R3R_NT = ((R3R_HW * R3_FH + 31) / 32) * 32;
+template <typename R, typename CB>
+__global__ void __launch_bounds__(R3R_NT, 2)
+    k_resrestrict3_red(OpView<R> o, const CB *__restrict__ b, const typename CT<R>::T *__restrict__ u,
+                       typename CT<R>::T *__restrict__ rc, int ncx, int ncy, int ncz, int kc, int first) {
+    pdl_enter();
+    if (o.gate && *o.gate) return;
+    typedef typename CT<R>::T C;
+    extern __shared__ __align__(16) unsigned char r3_smem[];
+    C(*rbuf)[R3_FH][R3_FW] = reinterpret_cast<C(*)[R3_FH][R3_FW]>(r3_smem);
+    const int I0 = 1 + blockIdx.x * R3_TX, J0 = 1 + blockIdx.y * R3_TY;
+    const int K0 = 1 + blockIdx.z * kc, K1 = min(K0 + kc, ncz - 1);
+    const int t = threadIdx.x, X0 = 2 * I0 - 1, ly = t / R3R_HW, y = 2 * J0 - 1 + ly;
+    const size_t sy = (size_t)o.nx, sz = sy * o.ny;
+    const int zs = 2 * K0 - 1, ze = 2 * K1 - 1;
+    // a buffer holds planes of one parity, so its red nodes are the same in every plane: the rest
+    // (black, or outside the interior) stays zero
+    for (int q = t; q < 2 * R3_FH * R3_FW; q += R3R_NT) (&rbuf[0][0][0])[q] = mk(R(0), R(0));
+    __syncthreads();
+    const bool row = t < R3R_HW * R3_FH && y <= o.ny - 2;
+    C cwy = mk(R(0), R(0)), ccy = cwy, cey = cwy;
+    if (row) { cwy = __ldg(&o.cy[3 * y]); ccy = __ldg(&o.cy[3 * y + 1]); cey = __ldg(&o.cy[3 * y + 2]); }
+    const int cx = t % R3_TX, cy = t / R3_TX, I = I0 + cx, J = J0 + cy;
+    const bool own = t < R3_TX * R3_TY && I <= ncx - 2 && J <= ncy - 2;
+    C acc = mk(R(0), R(0));
+    for (int z = zs; z <= ze; z++) {
+        const int lx = 2 * (t - ly * R3R_HW) + ((X0 + y + z) & 1), x = X0 + lx;
+        if (row && lx < R3_FW && x <= o.nx - 2) {
+            const size_t p = (size_t)x + sy * y + sz * z;
+            C a2 = cmul(__ldg(&o.cx[3 * x]), u[p - 1]);
+            a2 = cfma(__ldg(&o.cx[3 * x + 2]), u[p + 1], a2);
+            a2 = cfma(cwy, u[p - sy], a2);
+            a2 = cfma(cey, u[p + sy], a2);
+            a2 = cfma(__ldg(&o.cz[3 * z]), u[p - sz], a2);
+            a2 = cfma(__ldg(&o.cz[3 * z + 2]), u[p + sz], a2);
+            if (first) {
+                a2 = mk(-a2.x, -a2.y);
+            } else {
+                C d = cadd(cadd(__ldg(&o.cx[3 * x + 1]), ccy), __ldg(&o.cz[3 * z + 1]));
+                d = cadd(d, cadd(cscale(o.bk, o.k2[p]), o.c));
+                a2 = csub(to_c(b[p], R()), cfma(d, u[p], a2));
+            }
+            rbuf[z & 1][ly][lx] = a2;
+        }
+        __syncthreads();
+        if (own) {
+            const C(*rr)[R3_FW] = rbuf[z & 1];
+            const int fx = 2 * cx + 1, fy = 2 * cy + 1;  // region position of fine node (2I, 2J)
+            if (z & 1) {
+                // odd plane: the red nodes are the four side neighbours (weight 2)
+                const C v = cscale(cadd(cadd(rr[fy][fx - 1], rr[fy][fx + 1]), cadd(rr[fy - 1][fx], rr[fy + 1][fx])), R(2));
+                const int K = (z - 1) >> 1;
+                if (K >= K0) rc[(size_t)I + (size_t)ncx * ((size_t)J + (size_t)ncy * K)] = cscale(cadd(acc, v), R(1.0 / 64.0));
+                acc = v;
+            } else {
+                // even plane: the centre (weight 4) and the four corners, doubled along z
+                const C v = cadd(cadd(rr[fy - 1][fx - 1], rr[fy - 1][fx + 1]), cadd(rr[fy + 1][fx - 1], rr[fy + 1][fx + 1]));
+                const C c = rr[fy][fx];
+                acc = mk(fma(R(2), fma(R(4), c.x, v.x), acc.x), fma(R(2), fma(R(4), c.y, v.y), acc.y));
             }
         }
     }
@@ -861,17 +971,23 @@ dim3 grid_for(const int n[3], int dim) {
 template <typename R, typename CX>
 cudaError_t launch_apply(const DevOp<R> &op, int dim, const CX *x, typename CT<R>::T *y, cudaStream_t s) {
     dim3 g = grid_for(op.n, dim), b(BX, BY);
-    if (dim == 3) launch_pdl(k_apply<R, 3, CX>, g, b, 0, s, view(op), x, y);
-    else launch_pdl(k_apply<R, 2, CX>, g, b, 0, s, view(op), x, y);
+    const int kc = dim == 3 ? z_chunk((size_t)g.x * g.y, op.n[2] - 2, KCHUNK, 152 * 10) : 1;
+    if (dim == 3) g.z = cdiv(op.n[2] - 2, kc);
+    const CX *none = nullptr;
+    if (dim == 3) launch_pdl(k_apply<R, 3, CX, CX, false>, g, b, 0, s, view(op), none, x, y, kc);
+    else launch_pdl(k_apply<R, 2, CX, CX, false>, g, b, 0, s, view(op), none, x, y, kc);
     return cudaGetLastError();
 }
 
 template <typename R, typename CB>
 cudaError_t launch_residual(const DevOp<R> &op, int dim, const CB *bb, const typename CT<R>::T *u,
                             typename CT<R>::T *r, cudaStream_t s) {
+    typedef typename CT<R>::T C;
     dim3 g = grid_for(op.n, dim), b(BX, BY);
-    if (dim == 3) launch_pdl(k_residual<R, 3, CB>, g, b, 0, s, view(op), bb, u, r);
-    else launch_pdl(k_residual<R, 2, CB>, g, b, 0, s, view(op), bb, u, r);
+    const int kc = dim == 3 ? z_chunk((size_t)g.x * g.y, op.n[2] - 2, KCHUNK, 152 * 10) : 1;
+    if (dim == 3) g.z = cdiv(op.n[2] - 2, kc);
+    if (dim == 3) launch_pdl(k_apply<R, 3, C, CB, true>, g, b, 0, s, view(op), bb, u, r, kc);
+    else launch_pdl(k_apply<R, 2, C, CB, true>, g, b, 0, s, view(op), bb, u, r, kc);
     return cudaGetLastError();
 }
 
@@ -927,8 +1043,16 @@ cudaError_t launch_rb(const DevOp<R> &op, int dim, R omega, const CB *bb, typena
 
 template <typename R, typename CB>
 cudaError_t launch_residual_restrict(const DevOp<R> &op, int dim, const CB *bb, const typename CT<R>::T *u,
-                                     typename CT<R>::T *rc, cudaStream_t s) {
+                                     typename CT<R>::T *rc, cudaStream_t s, bool red, bool first) {
     int nc[3] = {(op.n[0] + 1) / 2, (op.n[1] + 1) / 2, dim == 3 ? (op.n[2] + 1) / 2 : 1};
+    if (red && dim == 3) {
+        dim3 g(cdiv(nc[0] - 2, R3_TX), cdiv(nc[1] - 2, R3_TY), 1);
+        const int kc = z_chunk((size_t)g.x * g.y, nc[2] - 2, R3_KC, 152 * 4);
+        g.z = cdiv(nc[2] - 2, kc);
+        launch_pdl(k_resrestrict3_red<R, CB>, g, R3R_NT, r3_smem_bytes<R>(), s, view(op), bb, u, rc, nc[0], nc[1], nc[2],
+                   kc, first ? 1 : 0);
+        return cudaGetLastError();
+    }
     if (dim == 3 && (size_t)op.n[0] * op.n[1] < ((size_t)1 << 31)) {  // 32-bit in-plane offsets
         constexpr size_t smem = r3_smem_bytes<R>();
         static bool attr = false;
@@ -1117,7 +1241,8 @@ template <typename C> cudaError_t launch_zero(size_t n, C *x, cudaStream_t s) {
     template cudaError_t launch_rb<R, CT<R>::T>(const DevOp<R> &, int, R, const CT<R>::T *, CT<R>::T *, int,     \
                                                  int, cudaStream_t);                                            \
     template cudaError_t launch_residual_restrict<R, CT<R>::T>(const DevOp<R> &, int, const CT<R>::T *,          \
-                                                                const CT<R>::T *, CT<R>::T *, cudaStream_t);    \
+                                                                const CT<R>::T *, CT<R>::T *, cudaStream_t, bool, \
+                                                                bool);                                          \
     template cudaError_t launch_prolong_add<R>(const int *, int, const CT<R>::T *, CT<R>::T *, cudaStream_t,      \
                                                const int *);                                                   \
     template cudaError_t launch_dense_solve<R>(const int *, int, int, const CT<R>::T *, const CT<R>::T *,        \

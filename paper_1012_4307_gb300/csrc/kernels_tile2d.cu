@@ -21,7 +21,8 @@
 // live one); a red-black half-sweep takes only its own colour's nodes.  Sizes are launch arguments:
 // the code is the same for every tile.
 // Measured on GB300: 641^2 complex128 F cycle with one sweep each way 755 -> 599 us, Bi-CGSTAB on 385^2
-// (two such cycles an iteration) 57.5 -> 42.0 ms.
+// (two such cycles an iteration) 57.5 -> 42.0 ms; with the residual after one sweep from zero formed
+// without the diagonal and real coefficients taken as real (block-uniform), 599 -> 538 us.
 #include <algorithm>
 
 #include "helm_internal.h"
@@ -78,38 +79,41 @@ template <typename R> struct Region {
     const T2<R> &A;
     int X0, Y0, W, H;
     C *cx, *cy, *ua, *ub;
+    bool real;  // complex128: the off-diagonal coefficients of every column and row of the region are real
     __device__ __forceinline__ int at(int x, int y) const { return (x - X0) + W * (y - Y0); }
     // [x0 - e, x1 + e] x [y0 - e, y1 + e] inside the grid's interior
     __device__ __forceinline__ Range grow(const Range &r, int e) const {
         return Range{max(r.x0 - e, 1), min(r.x1 + e, A.nx - 2), max(r.y0 - e, 1), min(r.y1 + e, A.ny - 2)};
     }
-    __device__ void stage() const {
+    // coefficients and a zero iterate; ends with a block barrier
+    __device__ __forceinline__ void stage() {
+        int im = sizeof(R) == sizeof(float);
         for (int q = threadIdx.x; q < 3 * W; q += blockDim.x) {
             const int x = X0 + q / 3;
             cx[q] = (x >= 1 && x <= A.nx - 2) ? __ldg(&A.cx[3 * X0 + q]) : mk(R(0), R(0));
+            im |= q % 3 != 1 && !is_zero(cx[q].y);
         }
         for (int q = threadIdx.x; q < 3 * H; q += blockDim.x) {
             const int y = Y0 + q / 3;
             cy[q] = (y >= 1 && y <= A.ny - 2) ? __ldg(&A.cy[3 * Y0 + q]) : mk(R(0), R(0));
+            im |= q % 3 != 1 && !is_zero(cy[q].y);
         }
         for (int q = threadIdx.x; q < 2 * W * H; q += blockDim.x) ua[q] = mk(R(0), R(0));  // ua, then ub
+        real = !__syncthreads_or(im);
     }
     // b minus the off-diagonal part of M u at (x, y)
-    __device__ __forceinline__ C rhs_off(const C *u, C b, int x, int y) const {
+    template <bool REAL> __device__ __forceinline__ C rhs_off(const C *u, C b, int x, int y) const {
         const int p = at(x, y), ix = 3 * (x - X0), iy = 3 * (y - Y0);
-        C acc = cmul(cx[ix], u[p - 1]);
-        acc = cfma(cx[ix + 2], u[p + 1], acc);
-        acc = cfma(cy[iy], u[p - W], acc);
-        acc = cfma(cy[iy + 2], u[p + W], acc);
-        return csub(b, acc);
+        return axis_sub<REAL>(cy[iy], cy[iy + 2], u[p - W], u[p + W],
+                              axis_sub<REAL>(cx[ix], cx[ix + 2], u[p - 1], u[p + 1], b));
     }
     // one relaxed update: (1 - omega) u + (omega / D) (b - off)
-    __device__ __forceinline__ C relax(const C *u, int x, int y) const {
+    template <bool REAL> __device__ __forceinline__ C relax(const C *u, int x, int y) const {
         const size_t g = (size_t)x + (size_t)A.nx * y;
         const C b = __ldg(&A.b[g]);
         C w = __ldg(&A.di[g]);
         if constexpr (sizeof(R) == sizeof(float)) w = cscale(w, A.omega);
-        return cfma(w, rhs_off(u, b, x, y), cscale(u[at(x, y)], R(1) - A.omega));
+        return cfma(w, rhs_off<REAL>(u, b, x, y), cscale(u[at(x, y)], R(1) - A.omega));
     }
     __device__ __forceinline__ C relax_zero(int x, int y) const {
         const size_t g = (size_t)x + (size_t)A.nx * y;
@@ -121,7 +125,7 @@ template <typename R> struct Region {
 template <typename R>
 __device__ __forceinline__ Region<R> region(const T2<R> &A, unsigned char *smem, int X0, int Y0, int W, int H) {
     typedef typename CT<R>::T C;
-    Region<R> G{A, X0, Y0, W, H, nullptr, nullptr, nullptr, nullptr};
+    Region<R> G{A, X0, Y0, W, H, nullptr, nullptr, nullptr, nullptr, false};
     C *p = (C *)smem;
     G.ua = p; p += W * H;
     G.ub = p; p += W * H;
@@ -130,19 +134,9 @@ __device__ __forceinline__ Region<R> region(const T2<R> &A, unsigned char *smem,
     return G;
 }
 
-template <typename R, bool RB>
-__global__ void __launch_bounds__(512) k_tile_pre(const __grid_constant__ T2<R> A) {
+template <typename R, bool RB, bool REAL> __device__ __forceinline__ void tile_pre(const T2<R> &A, const Region<R> &G, const Range &res) {
     typedef typename CT<R>::T C;
-    pdl_enter();
-    if (A.gate && *A.gate) return;
-    extern __shared__ __align__(16) unsigned char t2_smem[];
-    const int I0 = 1 + blockIdx.x * A.tcx, J0 = 1 + blockIdx.y * A.tcy;
-    // residuals of the coarse nodes' neighbourhoods: owned fine nodes and one more row and column
-    const Range res{2 * I0 - 1, 2 * I0 + 2 * A.tcx - 1, 2 * J0 - 1, 2 * J0 + 2 * A.tcy - 1};
-    const int e = 1 + A.s;
-    const Region<R> G = region<R>(A, t2_smem, res.x0 - e, res.y0 - e, 2 * A.tcx + 1 + 2 * e, 2 * A.tcy + 1 + 2 * e);
-    G.stage();
-    __syncthreads();
+    const int I0 = 1 + blockIdx.x * A.tcx, J0 = 1 + blockIdx.y * A.tcy, e = 1 + A.s;
     C *cur = G.ua, *oth = G.ub;
     int left = e;  // the iterate is right on grow(res, left)
     if (!A.zero) {
@@ -157,7 +151,7 @@ __global__ void __launch_bounds__(512) k_tile_pre(const __grid_constant__ T2<R> 
                     over_colour(G.grow(res, left), 0, [&](int x, int y) { cur[G.at(x, y)] = G.relax_zero(x, y); });
                 } else {
                     left--;
-                    over_colour(G.grow(res, left), colour, [&](int x, int y) { cur[G.at(x, y)] = G.relax(cur, x, y); });
+                    over_colour(G.grow(res, left), colour, [&](int x, int y) { cur[G.at(x, y)] = G.template relax<REAL>(cur, x, y); });
                 }
                 __syncthreads();
             }
@@ -166,7 +160,7 @@ __global__ void __launch_bounds__(512) k_tile_pre(const __grid_constant__ T2<R> 
             __syncthreads();
         } else {
             left--;
-            over(G.grow(res, left), [&](int x, int y) { oth[G.at(x, y)] = G.relax(cur, x, y); });
+            over(G.grow(res, left), [&](int x, int y) { oth[G.at(x, y)] = G.template relax<REAL>(cur, x, y); });
             __syncthreads();
             C *t = cur;
             cur = oth;
@@ -181,9 +175,18 @@ __global__ void __launch_bounds__(512) k_tile_pre(const __grid_constant__ T2<R> 
             const size_t g = (size_t)x + (size_t)A.nx * y;
             const int p = G.at(x, y);
             const C uc = cur[p];
-            const C d = cadd(cadd(G.cx[3 * (x - G.X0) + 1], G.cy[3 * (y - G.Y0) + 1]),
-                             cadd(cscale(A.bk, __ldg(&A.k2[g])), A.c));
-            r = csub(G.rhs_off(cur, __ldg(&A.b[g]), x, y), cmul(d, uc));
+            if (A.zero && A.nu == 1) {
+                // after one sweep from zero D u = omega b (red-black: omega (b - off) at the second
+                // colour), so no diagonal is formed: r = (1 - omega) b - off, or (1 - omega) (b - off)
+                const C bv = __ldg(&A.b[g]);
+                const R q1 = R(1) - A.omega;
+                if (RB && ((x + y) & 1)) r = cscale(G.template rhs_off<REAL>(cur, bv, x, y), q1);
+                else r = G.template rhs_off<REAL>(cur, cscale(bv, q1), x, y);
+            } else {
+                const C d = cadd(cadd(G.cx[3 * (x - G.X0) + 1], G.cy[3 * (y - G.Y0) + 1]),
+                                 cadd(cscale(A.bk, __ldg(&A.k2[g])), A.c));
+                r = csub(G.template rhs_off<REAL>(cur, __ldg(&A.b[g]), x, y), cmul(d, uc));
+            }
             if (x < res.x1 && y < res.y1) A.u_out[g] = uc;
         }
         oth[G.at(x, y)] = r;
@@ -202,17 +205,28 @@ __global__ void __launch_bounds__(512) k_tile_pre(const __grid_constant__ T2<R> 
 }
 
 template <typename R, bool RB>
-__global__ void __launch_bounds__(512) k_tile_post(const __grid_constant__ T2<R> A) {
-    typedef typename CT<R>::T C;
+__global__ void __launch_bounds__(512) k_tile_pre(const __grid_constant__ T2<R> A) {
     pdl_enter();
     if (A.gate && *A.gate) return;
     extern __shared__ __align__(16) unsigned char t2_smem[];
     const int I0 = 1 + blockIdx.x * A.tcx, J0 = 1 + blockIdx.y * A.tcy;
-    const Range own{2 * I0 - 1, 2 * I0 + 2 * A.tcx - 2, 2 * J0 - 1, 2 * J0 + 2 * A.tcy - 2};
-    const int e = A.s;
-    const Region<R> G = region<R>(A, t2_smem, own.x0 - e, own.y0 - e, 2 * A.tcx + 2 * e, 2 * A.tcy + 2 * e);
+    // residuals of the coarse nodes' neighbourhoods: owned fine nodes and one more row and column
+    const Range res{2 * I0 - 1, 2 * I0 + 2 * A.tcx - 1, 2 * J0 - 1, 2 * J0 + 2 * A.tcy - 1};
+    const int e = 1 + A.s;
+    Region<R> G = region<R>(A, t2_smem, res.x0 - e, res.y0 - e, 2 * A.tcx + 1 + 2 * e, 2 * A.tcy + 1 + 2 * e);
     G.stage();
-    __syncthreads();
+    if constexpr (sizeof(R) == sizeof(double)) {
+        if (G.real) {
+            tile_pre<R, RB, true>(A, G, res);
+            return;
+        }
+    }
+    tile_pre<R, RB, false>(A, G, res);
+}
+
+template <typename R, bool RB, bool REAL> __device__ __forceinline__ void tile_post(const T2<R> &A, const Region<R> &G, const Range &own) {
+    typedef typename CT<R>::T C;
+    const int e = A.s;
     C *cur = G.ua, *oth = G.ub;
     int left = e;
     // u + P ec: the mean of the four coarse values at floor / ceil of x / 2 and y / 2
@@ -227,22 +241,22 @@ __global__ void __launch_bounds__(512) k_tile_post(const __grid_constant__ T2<R>
         const bool last = k + 1 == A.nu;
         if constexpr (RB) {
             left--;
-            over_colour(G.grow(own, left), 0, [&](int x, int y) { cur[G.at(x, y)] = G.relax(cur, x, y); });
+            over_colour(G.grow(own, left), 0, [&](int x, int y) { cur[G.at(x, y)] = G.template relax<REAL>(cur, x, y); });
             __syncthreads();
             left--;
             if (last) {
-                over_colour(G.grow(own, 0), 1, [&](int x, int y) { A.u_out[(size_t)x + (size_t)A.nx * y] = G.relax(cur, x, y); });
+                over_colour(G.grow(own, 0), 1, [&](int x, int y) { A.u_out[(size_t)x + (size_t)A.nx * y] = G.template relax<REAL>(cur, x, y); });
                 over_colour(G.grow(own, 0), 0, [&](int x, int y) { A.u_out[(size_t)x + (size_t)A.nx * y] = cur[G.at(x, y)]; });
             } else {
-                over_colour(G.grow(own, left), 1, [&](int x, int y) { cur[G.at(x, y)] = G.relax(cur, x, y); });
+                over_colour(G.grow(own, left), 1, [&](int x, int y) { cur[G.at(x, y)] = G.template relax<REAL>(cur, x, y); });
                 __syncthreads();
             }
         } else {
             left--;
             if (last) {
-                over(G.grow(own, 0), [&](int x, int y) { A.u_out[(size_t)x + (size_t)A.nx * y] = G.relax(cur, x, y); });
+                over(G.grow(own, 0), [&](int x, int y) { A.u_out[(size_t)x + (size_t)A.nx * y] = G.template relax<REAL>(cur, x, y); });
             } else {
-                over(G.grow(own, left), [&](int x, int y) { oth[G.at(x, y)] = G.relax(cur, x, y); });
+                over(G.grow(own, left), [&](int x, int y) { oth[G.at(x, y)] = G.template relax<REAL>(cur, x, y); });
                 __syncthreads();
                 C *t = cur;
                 cur = oth;
@@ -250,6 +264,25 @@ __global__ void __launch_bounds__(512) k_tile_post(const __grid_constant__ T2<R>
             }
         }
     }
+}
+
+template <typename R, bool RB>
+__global__ void __launch_bounds__(512) k_tile_post(const __grid_constant__ T2<R> A) {
+    pdl_enter();
+    if (A.gate && *A.gate) return;
+    extern __shared__ __align__(16) unsigned char t2_smem[];
+    const int I0 = 1 + blockIdx.x * A.tcx, J0 = 1 + blockIdx.y * A.tcy;
+    const Range own{2 * I0 - 1, 2 * I0 + 2 * A.tcx - 2, 2 * J0 - 1, 2 * J0 + 2 * A.tcy - 2};
+    const int e = A.s;
+    Region<R> G = region<R>(A, t2_smem, own.x0 - e, own.y0 - e, 2 * A.tcx + 2 * e, 2 * A.tcy + 2 * e);
+    G.stage();
+    if constexpr (sizeof(R) == sizeof(double)) {
+        if (G.real) {
+            tile_post<R, RB, true>(A, G, own);
+            return;
+        }
+    }
+    tile_post<R, RB, false>(A, G, own);
 }
 
 // Coarse nodes per tile: the shape with the least time by the model (blocks per SM, at least one) x

@@ -31,12 +31,12 @@ def problem(n, coarsest_n):
     return W.Problem("paths", dim, list(n), np.ascontiguousarray(k2), np.zeros(shape, complex), coarsest_n=coarsest_n)
 
 
-def check_cycle(helm, oracle, n, coarsest_n, prec, smoother, nu, gamma, tunings=({},)):
+def check_cycle(helm, oracle, n, coarsest_n, prec, smoother, nu, gamma, tunings=({},), omega=0.8, pc="csg"):
     P = problem(n, coarsest_n)
-    h = gpu_handle(helm, P, pc="csg", prec=prec, smoother=smoother, nu=nu, gamma=gamma)
-    A, M = oracle_pair(oracle, P)
+    h = gpu_handle(helm, P, pc=pc, prec=prec, smoother=smoother, nu=nu, gamma=gamma, omega=omega)
+    A, M = oracle_pair(oracle, P, pc=pc)
     v = W.random_field(tuple(reversed(n)), 51)
-    ref = oracle.MG(M, coarsest_n, nu[0], nu[1], 0.8, smoother).cycle(v, None, *gamma)
+    ref = oracle.MG(M, coarsest_n, nu[0], nu[1], omega, smoother).cycle(v, None, *gamma)
     dtype = torch.complex64 if prec == "c64" else torch.complex128
     for t in tunings:
         if t:
@@ -76,3 +76,27 @@ def test_3d_level_kernels(helm, oracle, n, coarsest_n, prec, smoother, nu, gamma
     """The 3D sweeps (omega / D formed once in complex128), red-black from zero and from a guess, with
     chunks of one to eight planes."""
     check_cycle(helm, oracle, n, coarsest_n, prec, smoother, nu, gamma, [dict(tail_levels=0)])
+
+
+@pytest.mark.parametrize("prec", ["c64", "c128"])
+@pytest.mark.parametrize("nu,gamma,tail", [((1, 1), (1, 1), 0), ((2, 1), (1, 2), 0), ((1, 1), (2, 2), -1)])
+@pytest.mark.parametrize("n,coarsest_n", [((33, 17, 65), 9), ((41, 73, 25), 10), ((97, 65), 17)])
+def test_red_black_with_omega_one(helm, oracle, n, coarsest_n, prec, nu, gamma, tail):
+    """omega = 1: the second colour's residuals are zero and the restriction takes only the first
+    colour's, after the first sweep from zero (no diagonal term) and after later ones."""
+    check_cycle(helm, oracle, n, coarsest_n, prec, "rb", nu, gamma, [dict(tail_levels=tail)], omega=1.0)
+
+
+@pytest.mark.parametrize("n,coarsest_n", [((65, 33), 17), ((33, 17, 25), 9)])
+@pytest.mark.parametrize("smoother", ["jacobi", "rb"])
+def test_real_coefficients_outside_the_layers(helm, oracle, n, coarsest_n, smoother):
+    """The shifted Laplacian keeps the widths, so its coefficients are real outside the layers and
+    each axis takes the short form there: levels, tail, and the operator itself."""
+    check_cycle(helm, oracle, n, coarsest_n, "c128", smoother, (1, 1), (1, 2), [dict(tail_levels=-1), dict(tail_levels=0)],
+                pc="csl")
+    P = problem(n, coarsest_n)
+    h = gpu_handle(helm, P, pc="csl", prec="c128")
+    A, M = oracle_pair(oracle, P, pc="csl")
+    x = W.random_field(tuple(reversed(n)), 52)
+    for which, op in (("A", A), ("M", M)):
+        assert rel_l2(to_np(helm.helm_apply(h, to_gpu(x), which=which)), op.apply(x)) <= 1e-14
