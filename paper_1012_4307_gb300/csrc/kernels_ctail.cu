@@ -222,48 +222,51 @@ __device__ __forceinline__ typename CT<R>::T relax_at(const Ctx &X, const LV &L,
     }
 }
 
+// The start of a visit from zero at an owned node whose right-hand side b has just been written, in the
+// same phase (the first sweep from zero is pointwise, so it needs no phase of its own): the first
+// Jacobi sweep into t, or the first colour of the first red-black sweep (the other colour 0) into u, or
+// u = 0 without pre-sweeps.
+template <typename R>
+__device__ __forceinline__ void start_zero(const Ctx &X, const LV &L, const CArgs<R> *A, int j, int q, int i, int y,
+                                           typename CT<R>::T b) {
+    typedef typename CT<R>::T C;
+    C v = mk(R(0), R(0));
+    if (A->nu1 > 0 && !(A->rb && ((i + y + j) & 1))) {
+        v = cmul(b, dinv_at<C>(X, L, j, q));
+        if constexpr (sizeof(R) == sizeof(float)) v = cscale(v, A->omega);
+    }
+    put(X, L, A->nu1 > 0 && !A->rb ? L.ot : L.ou, j, q, v, X.rank);
+}
+
 // The phases of the cycle.  Each is one out-of-line function over a level index, so that the
 // kernel's code stays small (inlining every phase at every depth multiplies it by the levels
 // and smoothing steps and runs out of the instruction cache); each ends with a cluster barrier.
 
-// nu sweeps on level l from *cur (partner *oth); zero: u = 0 on entry.  Returns the new pair.
+// nu sweeps on level l from *cur (partner *oth); started: start_zero has done the pointwise part of the
+// first one.  Returns the new pair.
 template <typename R, int DIM>
-__device__ __noinline__ uint2 ph_smooth(Ctx X, const CArgs<R> *A, int l, int nu, uint2 co, bool zero) {
-    typedef typename CT<R>::T C;
+__device__ __noinline__ uint2 ph_smooth(Ctx X, const CArgs<R> *A, int l, int nu, uint2 co, bool started) {
     const LV L = lv_of(X, A->lv[l]);
     const R om = A->omega;
-    const bool rb = A->rb != 0;
-    if (zero && (nu == 0 || rb)) {
-        const unsigned u = co.x;
-        for_owned<DIM>(X, L, [&](int j, int q, int, int) { put(X, L, u, j, q, mk(R(0), R(0)), X.rank); });
-        csync();
-    }
-    for (int s = 0; s < nu; s++) {
-        if (rb) {
-            for (int colour = 0; colour < 2; colour++) {
-                // in place: this colour's neighbours (the other colour) are not written here
-                const unsigned u = co.x;
-                for_colour<DIM>(X, L, colour, [&](int j, int q, int i, int y) {
-                    put(X, L, u, j, q, relax_at<R, DIM>(X, L, u, j, q, i, y, om), X.rank);
-                });
-                csync();
-            }
-        } else {
-            const bool z0 = zero && s == 0;
-            const unsigned src = co.x, dst = co.y;
-            for_owned<DIM>(X, L, [&](int j, int q, int i, int y) {
-                C v;
-                if (z0) {
-                    v = cmul(lrow<C>(X, L, L.ob, j)[q], dinv_at<C>(X, L, j, q));
-                    if constexpr (sizeof(R) == sizeof(float)) v = cscale(v, om);
-                } else {
-                    v = relax_at<R, DIM>(X, L, src, j, q, i, y, om);
-                }
-                put(X, L, dst, j, q, v, X.rank);
+    if (A->rb) {
+        for (int h = started ? 1 : 0; h < 2 * nu; h++) {
+            // in place: this colour's neighbours (the other colour) are not written here
+            const unsigned u = co.x;
+            for_colour<DIM>(X, L, h & 1, [&](int j, int q, int i, int y) {
+                put(X, L, u, j, q, relax_at<R, DIM>(X, L, u, j, q, i, y, om), X.rank);
             });
             csync();
-            co = make_uint2(dst, src);
         }
+        return co;
+    }
+    if (started && nu > 0) co = make_uint2(co.y, co.x);
+    for (int s = started ? 1 : 0; s < nu; s++) {
+        const unsigned src = co.x, dst = co.y;
+        for_owned<DIM>(X, L, [&](int j, int q, int i, int y) {
+            put(X, L, dst, j, q, relax_at<R, DIM>(X, L, src, j, q, i, y, om), X.rank);
+        });
+        csync();
+        co = make_uint2(dst, src);
     }
     return co;
 }
@@ -281,7 +284,8 @@ template <typename C, int DIM> __device__ __forceinline__ C w121_row(const C *r,
 }
 
 // Residual of level l (iterate u) into r, then full weighting into level l + 1's b (the fine
-// rows 2J-1 .. 2J+1 of an owned coarse row J are owned or halo rows: nested slabs).
+// rows 2J-1 .. 2J+1 of an owned coarse row J are owned or halo rows: nested slabs) and the start of
+// that level's visit from zero.
 // first: u is one sweep from zero, so that D u = omega b (red-black: omega (b - offdiagonal part) at the
 // second colour) and complex128 needs no diagonal term.
 template <typename R, int DIM>
@@ -289,7 +293,7 @@ __device__ __noinline__ void ph_restrict(Ctx X, const CArgs<R> *A, int l, unsign
     typedef typename CT<R>::T C;
     const LV L = lv_of(X, A->lv[l]), Lc = lv_of(X, A->lv[l + 1]);
     const R q1 = R(1) - A->omega;
-    const bool rb = A->rb != 0;
+    const bool rb = A->rb != 0, inner = l + 2 < A->nlev;  // the coarsest level is solved, not smoothed
     for_owned<DIM>(X, L, [&](int j, int q, int i, int y) {
         const C b = lrow<C>(X, L, L.ob, j)[q];
         C v;
@@ -307,7 +311,9 @@ __device__ __noinline__ void ph_restrict(Ctx X, const CArgs<R> *A, int l, unsign
         const C *r0 = lrow<C>(X, L, r, 2 * J - 1), *r1 = lrow<C>(X, L, r, 2 * J), *r2 = lrow<C>(X, L, r, 2 * J + 1);
         const int q = 2 * I + (DIM == 3 ? L.nx * 2 * Y : 0);
         const C a0 = w121_row<C, DIM>(r0, q, L.nx), a1 = w121_row<C, DIM>(r1, q, L.nx), a2 = w121_row<C, DIM>(r2, q, L.nx);
-        lrow<C>(X, Lc, Lc.ob, J)[Q] = cscale(cadd(cadd(a0, a2), cscale(a1, R(2))), DIM == 3 ? R(1.0 / 64.0) : R(0.0625));
+        const C b = cscale(cadd(cadd(a0, a2), cscale(a1, R(2))), DIM == 3 ? R(1.0 / 64.0) : R(0.0625));
+        lrow<C>(X, Lc, Lc.ob, J)[Q] = b;
+        if (inner) start_zero<R>(X, Lc, A, J, Q, I, Y, b);
     });
     csync();
 }
@@ -483,10 +489,12 @@ __device__ __forceinline__ void ct_run(const Ctx &X, const CArgs<R> *A) {
     pdl_wait();
     // every block's initial fill precedes any store into its halos
     csync();
-    for_owned<DIM>(X, T, [&](int j, int q, int, int) {
+    for_owned<DIM>(X, T, [&](int j, int q, int i, int y) {
         const size_t p = (size_t)q + (size_t)T.S * j;
-        lrow<C>(X, T, T.ob, j)[q] = A->b_top[p];
-        if (!A->zero) put(X, T, T.ou, j, q, A->u_top[p], X.rank);
+        const C b = A->b_top[p];
+        lrow<C>(X, T, T.ob, j)[q] = b;
+        if (A->zero) start_zero<R>(X, T, A, j, q, i, y, b);
+        else put(X, T, T.ou, j, q, A->u_top[p], X.rank);
     });
     csync();
     ct_cycle<R, DIM, 0>(X, A, A->zero != 0, A->gf, A->gc);

@@ -422,12 +422,12 @@ __global__ void __launch_bounds__(BX *BY) k_prolong_add(int nx, int ny, int nz, 
 // coarse nodes in (x, y) and kc coarse planes (at most R3_KC); one thread per fine node of the region those
 // coarse nodes weigh ((2 R3_TX + 1) x (2 R3_TY + 1)) marches the block's fine planes
 // 2 K0 - 1 .. 2 K1 - 1 like k_jacobi3 (coefficients in registers, the u column (z - 1, z, z + 1)
-// in registers, the next plane's operands loaded while this plane is computed) and stores its
-// residual in a shared plane (two buffers); after one barrier per plane the coarse nodes' threads
-// apply (1,2,1)/4 in x and y from the shared plane and accumulate (1,2,1)/4 in z in registers:
-// an odd fine plane 2K + 1 completes coarse plane K and starts K + 1.  Fine nodes outside the
-// grid's interior hold zero residuals.  Same arithmetic as k_residual_restrict, with the weights
-// applied per axis.
+// in registers, the next plane's operands loaded while this plane is computed).  Each thread weighs its
+// own residuals by (1, 2, 1) along z in registers; once per coarse plane the weighted plane goes through
+// shared memory (two buffers, one barrier) and the coarse nodes' threads apply (1, 2, 1) in x and y --
+// one exchange and one 3 x 3 sum per coarse plane instead of one per fine plane.  An odd fine plane
+// 2K + 1 completes coarse plane K and starts K + 1.  Fine nodes outside the grid's interior hold zero
+// residuals.  Same weights as k_residual_restrict, applied per axis.
 constexpr int R3_TX = 16, R3_TY = 8, R3_KC = 8;
 constexpr int R3_FW = 2 * R3_TX + 1, R3_FH = 2 * R3_TY + 1;  // fine region
 constexpr int R3_NT = ((R3_FW * R3_FH + 31) / 32) * 32;       // threads: one per region node
@@ -450,28 +450,30 @@ __global__ void __launch_bounds__(R3_NT, sizeof(R) == sizeof(float) ? 2 : 1)
     const int t = threadIdx.x, lx = t % R3_FW, ly = t / R3_FW;
     const int x = 2 * I0 - 1 + lx, y = 2 * J0 - 1 + ly;
     // region nodes inside the grid's interior compute residuals; the others hold zeros
-    const bool res = t < R3_FW * R3_FH && x <= nx - 2 && y <= ny - 2;
+    const bool region = t < R3_FW * R3_FH, res = region && x <= nx - 2 && y <= ny - 2;
     const size_t sy = (size_t)nx, sz = (size_t)nx * ny;
     const int zs = 2 * K0 - 1, ze = 2 * K1 - 1;
     const C zero = mk(R(0), R(0));
-    C cwx = zero, ccx = zero, cex = zero, cwy = zero, ccy = zero, cey = zero;
+    C cwx = zero, cex = zero, cwy = zero, cey = zero, dxy = zero;
     C xm = zero, xc = zero, xp = zero, xw = zero, xe = zero, xs = zero, xn = zero, bq = zero;
     R kq = R(0);
     size_t p = (size_t)x + sy * y + sz * zs;
     if (res) {
-        cwx = __ldg(&o.cx[3 * x]); ccx = __ldg(&o.cx[3 * x + 1]); cex = __ldg(&o.cx[3 * x + 2]);
-        cwy = __ldg(&o.cy[3 * y]); ccy = __ldg(&o.cy[3 * y + 1]); cey = __ldg(&o.cy[3 * y + 2]);
+        cwx = __ldg(&o.cx[3 * x]); cex = __ldg(&o.cx[3 * x + 2]);
+        cwy = __ldg(&o.cy[3 * y]); cey = __ldg(&o.cy[3 * y + 2]);
+        dxy = cadd(cadd(__ldg(&o.cx[3 * x + 1]), __ldg(&o.cy[3 * y + 1])), o.c);
         xm = u[p - sz]; xc = u[p]; xp = u[p + sz];
         xw = u[p - 1]; xe = u[p + 1]; xs = u[p - sy]; xn = u[p + sy];
         bq = to_c(b[p], R());
         kq = o.k2[p];
     }
     if (gv) return;  // the same value in every thread: no barrier is left waiting
-    // the coarse node of this thread (threads below R3_TX * R3_TY), and its running z sum
+    // the coarse node of this thread (threads below R3_TX * R3_TY)
     const int cx = t % R3_TX, cy = t / R3_TX, I = I0 + cx, J = J0 + cy;
     const bool own = t < R3_TX * R3_TY && I <= ncx - 2 && J <= ncy - 2;
-    C acc = zero;
+    C acc = zero;  // z sum of this fine column for the current coarse plane
     for (int z = zs; z <= ze; z++, p += sz) {
+        C r = zero;
         if (res) {
             C xw2 = xw, xe2 = xe, xs2 = xs, xn2 = xn, xp2 = xp, bn = bq;
             R kn = kq;
@@ -487,43 +489,41 @@ __global__ void __launch_bounds__(R3_NT, sizeof(R) == sizeof(float) ? 2 : 1)
             }
             C a2 = cmul(cwx, xw);
             a2 = cfma(cex, xe, a2);
-            C d = ccx;
             a2 = cfma(cwy, xs, a2);
             a2 = cfma(cey, xn, a2);
-            d = cadd(d, ccy);
-            const C czw = __ldg(&o.cz[3 * z]), czc = __ldg(&o.cz[3 * z + 1]), cze = __ldg(&o.cz[3 * z + 2]);
-            a2 = cfma(czw, xm, a2);
-            a2 = cfma(cze, xp, a2);
-            d = cadd(d, czc);
-            d = cadd(d, cadd(cscale(o.bk, kq), o.c));
-            rbuf[z & 1][ly][lx] = csub(bq, cfma(d, xc, a2));
+            a2 = cfma(__ldg(&o.cz[3 * z]), xm, a2);
+            a2 = cfma(__ldg(&o.cz[3 * z + 2]), xp, a2);
+            const C ccz = __ldg(&o.cz[3 * z + 1]);
+            const C d = mk(fma(o.bk.x, kq, dxy.x + ccz.x), fma(o.bk.y, kq, dxy.y + ccz.y));
+            r = csub(bq, cfma(d, xc, a2));
             xm = xc;
             xc = xp;
             xw = xw2; xe = xe2; xs = xs2; xn = xn2; xp = xp2; bq = bn; kq = kn;
-        } else if (t < R3_FW * R3_FH) {
-            rbuf[z & 1][ly][lx] = zero;
         }
-        __syncthreads();
-        if (own) {
-            // (1,2,1)/4 along x on the three fine rows 2J - 1 .. 2J + 1, then along y
-            const C(*rr)[R3_FW] = rbuf[z & 1];
-            const int fx = 2 * cx, fy = 2 * cy;
-            C a[3];
+        if (!(z & 1)) {
+            acc = mk(fma(R(2), r.x, acc.x), fma(R(2), r.y, acc.y));
+            continue;
+        }
+        // fine plane 2K + 1 (K = (z - 1) / 2) completes coarse plane K and starts K + 1
+        const int K = (z - 1) >> 1;
+        if (K >= K0) {
+            C(*buf)[R3_FW] = rbuf[K & 1];
+            if (region) buf[ly][lx] = cadd(acc, r);
+            __syncthreads();
+            if (own) {
+                // (1, 2, 1) along x on the three fine rows 2J - 1 .. 2J + 1, then along y
+                const int fx = 2 * cx, fy = 2 * cy;
+                C a[3];
 #pragma unroll
-            for (int dy = 0; dy < 3; dy++) {
-                const C *row = &rr[fy + dy][fx];
-                a[dy] = cadd(cadd(row[0], row[2]), cscale(row[1], R(2)));
-            }
-            const C v = cadd(cadd(a[0], a[2]), cscale(a[1], R(2)));
-            if (z & 1) {
-                // fine plane 2K + 1 (K = (z - 1) / 2) completes coarse plane K and starts K + 1
-                const int K = (z - 1) >> 1;
-                if (K >= K0) rc[(size_t)I + (size_t)ncx * ((size_t)J + (size_t)ncy * K)] = cscale(cadd(acc, v), R(1.0 / 64.0));
-                acc = v;
-            } else {
-                acc = cadd(acc, cscale(v, R(2)));
+                for (int dy = 0; dy < 3; dy++) {
+                    const C *row = &buf[fy + dy][fx];
+                    a[dy] = cadd(cadd(row[0], row[2]), cscale(row[1], R(2)));
+                }
+                rc[(size_t)I + (size_t)ncx * ((size_t)J + (size_t)ncy * K)] =
+                    cscale(cadd(cadd(a[0], a[2]), cscale(a[1], R(2))), R(1.0 / 64.0));
             }
         }
+        acc = r;
     }
 }
 
