@@ -387,7 +387,8 @@ helm_status helm_create_impl(const helm_grid *grid, double theta, const double *
         // each, on 16 blocks, or 8 where the device runs no cluster of 16
         for (int prec = 0; prec < 2; prec++) {
             const size_t es = prec == 0 ? sizeof(float2) : sizeof(double2);
-            const double most = tail_max_unknowns(dim, es);
+            const bool v22 = mg->smoother == HELM_SMOOTH_JACOBI && mg->nu1 == 2 && mg->nu2 == 2 && mg->gamma_f == 1 &&
+                             mg->gamma_c == 1;
             for (int nc = 16; nc >= 8 && h->tail_built[prec] < 0; nc -= 8) {
                 int fit = 0;
                 size_t bytes = 0;
@@ -395,7 +396,7 @@ helm_status helm_create_impl(const helm_grid *grid, double theta, const double *
                     const LevelDev &L = h->lv[nlev - nt];
                     const double ni = (double)(L.n[0] - 2) * (L.n[1] - 2) * (dim == 3 ? (double)(L.n[2] - 2) : 1.0);
                     const size_t b = tail_bytes(nt, nc, es);
-                    if (ni > most || b > CT_SMEM_BYTES) break;
+                    if (ni > tail_max_unknowns(dim, es, v22, nt == nlev) || b > CT_SMEM_BYTES) break;
                     fit = nt;
                     bytes = b;
                 }
@@ -528,9 +529,10 @@ static double interior(const LevelDev &L, int dim) {
 
 // smoothing steps on level l; *cur holds the iterate and may be swapped with *oth (Jacobi).
 // Algorithmic bytes per sweep and unknown: read u, b, k^2, write u (3 complex + 1 real).
+// v (complex64 3D from zero only): b's complex128 original, from which the first sweep forms b too.
 template <typename R>
 static cudaError_t smooth(helm_handle *h, int l, int sweeps, const typename CT<R>::T *b, typename CT<R>::T **cur,
-                          typename CT<R>::T **oth, bool zero) {
+                          typename CT<R>::T **oth, bool zero, const double2 *v = nullptr) {
     LevelDev &L = h->lv[l];
     const DevOp<R> &op = LvBuf<R>::op(L);
     const R om = (R)h->mg.omega;
@@ -554,6 +556,14 @@ static cudaError_t smooth(helm_handle *h, int l, int sweeps, const typename CT<R
     }
     for (int s = 0; s < sweeps; s++) {
         const bool z0 = zero && s == 0;
+        if constexpr (sizeof(R) == sizeof(float)) {
+            if (z0 && v) {
+                ProfScope ps(h, cls, ni * (16 + 2 * es + rs), 0);
+                CKE(launch_jacobi3_first(op, om, v, const_cast<float2 *>(b), *oth, h->stream));
+                std::swap(*cur, *oth);
+                continue;
+            }
+        }
         ProfScope ps(h, cls, ni * ((z0 ? 2 : 3) * es + rs), 0);
         CKE(launch_jacobi<R>(op, h->dim, om, b, z0 ? nullptr : *cur, *oth, h->stream));
         std::swap(*cur, *oth);
@@ -566,6 +576,19 @@ static cudaError_t coarse_solve(helm_handle *h, LevelDev &L, const typename CT<R
     const double es = sizeof(typename CT<R>::T), nu = h->nu_c;
     ProfScope ps(h, HELM_K_COARSE, nu * nu * es + 2 * nu * es, 8.0 * nu * nu);
     return launch_dense_solve<R>(L.n, h->dim, h->nu_c, LvBuf<R>::minv(h), b, u, h->stream);
+}
+
+// Where no tuning was set: large levels take the tile with the least halo, small ones the tile that
+// spreads them over the SMs.  Measured per complex64 V(2,2) cycle, all levels 32x8 / this rule: 257^2
+// 32.3 / 29.4 us, 385^2 37.6 / 33.4, 513^2 43.6 / 38.1, 641^2 52.1 / 47.1, 769^2 56.3 / 50.4, 1025^2 74.3 /
+// 68.0, 1281^2 100.8 / 96.2.
+int helm_level_tile(const helm_handle *h, int l) {
+    if (l >= HELM_MAX_LEVELS) return HELM_TILE_NONE;
+    if (h->tuned || h->dim != 2) return h->tune.level_tile[l];
+    const LevelDev &L = h->lv[l];
+    const double n = sqrt((double)L.n[0] * L.n[1]);
+    const int tile = n > 600 ? HELM_TILE_16x16 : n > 340 ? HELM_TILE_16x8 : HELM_TILE_8x8;
+    return fused_jacobi2_ok(L.n, 2, tile) ? tile : h->tune.level_tile[l];
 }
 
 // Key of a tail's image.
@@ -647,9 +670,11 @@ void helm_refresh_tails(helm_handle *h, bool build) {
 // u <- MG(l, M_l, b, u, nu1, nu2, C, gf, gc).  'zero' means u = 0 on entry (not read).
 // The result always ends in u.  Level l uses its own t buffer as the Jacobi partner; coarse
 // levels use their own b (restricted residual) and u (error) buffers.
+// v: level 0's right-hand side still in complex128, to be rounded into b by the level's first launch
+// (first_launch_rounds); null: b holds it.
 template <typename R>
 static cudaError_t cycle(helm_handle *h, int l, const typename CT<R>::T *b, typename CT<R>::T *u, bool zero, int gf,
-                         int gc) {
+                         int gc, const double2 *v = nullptr) {
     typedef typename CT<R>::T C;
     LevelDev &L = h->lv[l];
     const int last = (int)h->lv.size() - 1;
@@ -683,7 +708,7 @@ static cudaError_t cycle(helm_handle *h, int l, const typename CT<R>::T *b, type
         // temporal blocking: two pre-sweeps from zero + residual + FW in one launch (iterate to
         // this level's t), the coarse correction, then correction + two post-sweeps in one
         // launch (t -> u)
-        const int tile = l < HELM_MAX_LEVELS ? h->tune.level_tile[l] : (int)HELM_TILE_NONE;
+        const int tile = helm_level_tile(h, l);
         if (zero && h->mg.smoother == HELM_SMOOTH_JACOBI && h->mg.nu1 == 2 && h->mg.nu2 == 2 &&
             fused_jacobi2_ok(L.n, h->dim, tile)) {
             LevelDev &Lc = h->lv[l + 1];
@@ -693,7 +718,8 @@ static cudaError_t cycle(helm_handle *h, int l, const typename CT<R>::T *b, type
                 // residual with full weighting (u, b, k^2 -> coarse)
                 ProfScope ps(h, l == 0 ? HELM_K_SMOOTH_FINE : HELM_K_SMOOTH_COARSE, ni * (es + es + es + es / nd), 0,
                              ni * ((2 * es + rs) + (3 * es + rs) + (2 * es + rs + es / nd)));
-                CKE(launch_pre2_restrict(L.M32, tile, (float)h->mg.omega, b, L.t32, Lc.b32, h->stream));
+                if (v) CKE(launch_pre2_restrict_c128(L.M32, tile, (float)h->mg.omega, v, const_cast<float2 *>(b), L.t32, Lc.b32, h->stream));
+                else CKE(launch_pre2_restrict(L.M32, tile, (float)h->mg.omega, b, L.t32, Lc.b32, h->stream));
             }
             float2 *ec = Lc.u32;
             if (l + 1 == last) {
@@ -742,7 +768,7 @@ static cudaError_t cycle(helm_handle *h, int l, const typename CT<R>::T *b, type
         return launch_tile_post<R>(op, (R)h->mg.omega, nu2, rb, b, LvBuf<R>::t(L), u, ec, h->stream);
     }
     C *cur = u, *oth = LvBuf<R>::t(L);
-    CKE(smooth<R>(h, l, nu1, b, &cur, &oth, zero));
+    CKE(smooth<R>(h, l, nu1, b, &cur, &oth, zero, v));
     {
         ProfScope ps(h, HELM_K_RESTRICT, ni * (2 * es + rs + es / nd), 0);
         const bool red = rb && h->mg.omega == 1.0 && nu1 > 0;
@@ -752,11 +778,21 @@ static cudaError_t cycle(helm_handle *h, int l, const typename CT<R>::T *b, type
     CKE(coarse());
     {
         ProfScope ps(h, HELM_K_PROLONG, ni * (2 * es + es / nd), 0);
-        CKE(launch_prolong_add<R>(L.n, h->dim, ec, cur, h->stream, LvBuf<R>::op(L).gate));
+        CKE(launch_prolong_add<R>(L.n, h->dim, ec, cur, h->stream, LvBuf<R>::op(L).gate,
+                                  rb && h->mg.omega == 1.0 && nu2 > 0));
     }
     CKE(smooth<R>(h, l, nu2, b, &cur, &oth, false));
     if (cur != u) CKE(cudaMemcpyAsync(u, cur, L.np * sizeof(C), cudaMemcpyDeviceToDevice, h->stream));
     return cudaSuccess;
+}
+
+// Whether a complex64 cycle's first launch on level 0 can take the right-hand side in complex128.
+static bool first_launch_rounds(const helm_handle *h) {
+    const helm_mg_params &m = h->mg;
+    if (h->lv.size() < 2 || h->tail[0].top == 0 || m.smoother != HELM_SMOOTH_JACOBI) return false;
+    if (h->dim == 3) return m.nu1 >= 1;
+    const int tile = helm_level_tile(h, 0);
+    return m.nu1 == 2 && m.nu2 == 2 && tile != HELM_TILE_WAVE && fused_jacobi2_ok(h->n, 2, tile);
 }
 
 // z = M^{-1}-approximation of v (one cycle from zero), v in FP64, z in precision R.
@@ -770,6 +806,8 @@ cudaError_t precondition(helm_handle *h, const double2 *v, typename CT<R>::T *z)
     }
     if (sizeof(R) == sizeof(double))
         return cycle<R>(h, 0, (const typename CT<R>::T *)v, z, true, h->mg.gamma_f, h->mg.gamma_c);
+    if (first_launch_rounds(h))
+        return cycle<R>(h, 0, LvBuf<R>::b(h->lv[0]), z, true, h->mg.gamma_f, h->mg.gamma_c, v);
     {
         ProfScope ps(h, HELM_K_VECTOR, h->np * (16 + es), 0);
         CKE(launch_convert(h->np, v, LvBuf<R>::b(h->lv[0]), h->stream));

@@ -72,6 +72,7 @@ struct helm_handle {
     // its first level (-1: none) and blocks per cluster
     int tail_built[2] = {-1, -1}, tail_ctas[2] = {16, 16};
     helm_tuning tune{};                      // kernel choices (see helm_set_tuning)
+    bool tuned = false;                      // set by helm_set_tuning or helm_autotune
     int ctail_fit[2] = {0, 0};               // most coarsest levels a cluster tail of 8 / 16 blocks holds
     // the fused tail that the tuning selects, per precision (helm_refresh_tails)
     struct Tail {
@@ -186,6 +187,8 @@ cudaError_t precondition_pair(helm_handle *h, const float4 *v, const double2 *al
 // there by the delayed-CGS2 update pass), and that buffer.
 cudaError_t precondition_level0_c64(helm_handle *h, float2 *z);
 float2 *level0_rhs_c64(helm_handle *h);
+// The tile of level l: the tuning's, or without one a choice by the level's size.
+int helm_level_tile(const helm_handle *h, int l);
 // Recomputes h->tail for the handle's tuning; with build, also builds the initial shared-memory
 // images its cycles use (allocates device memory and launches on the handle's stream; outside graph
 // capture).

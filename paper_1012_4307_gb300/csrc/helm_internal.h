@@ -61,6 +61,8 @@ template <bool REAL, typename C> __device__ __forceinline__ C axis_add(C cw, C c
 template <bool REAL, typename C> __device__ __forceinline__ C axis_sub(C cw, C ce, C xw, C xe, C acc) {
     return axis_add<REAL>(mk(-cw.x, -cw.y), mk(-ce.x, -ce.y), xw, xe, acc);
 }
+// Asks for the cache line of p (an address inside an allocation) in L2.
+__device__ __forceinline__ void l2_prefetch(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 // dst[q] = src[q] for q < n (src global and unchanged during the kernel, dst this block's
 // shared memory): each thread issues eight loads before it stores, so that a block's copy takes
 // a few memory round trips instead of one per float4 a thread moves.
@@ -80,9 +82,36 @@ __device__ __forceinline__ void block_copy16(float4 *dst, const float4 *__restri
         }
     }
 }
+// (float)x and (double)x with integer instructions: a conversion between the two precisions runs on the
+// FP64 units (two lanes per SM and clock), which bound the kernels that converted whole vectors
+// (complex128 to complex64 of 257^3 nodes: 78% of that pipe, 68% of the DRAM rate).  Bit for bit the
+// conversions' results: round to nearest even; magnitudes outside the normal range of float (zero
+// excepted) take the instruction.
+__device__ __forceinline__ float to_float(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const unsigned h = (unsigned)(b >> 32), l = (unsigned)b, m = h & 0x7FFFFFFFu;
+    const unsigned t = m - (896u << 20);  // exponent rebased to float's, in bits 20 ..
+    if (t - (1u << 20) >= (253u << 20)) {
+        if ((m | l) != 0u) return (float)x;
+        return __uint_as_float(h);
+    }
+    // 24 significant bits truncated, then one unit added when the 29 bits below are above half of it, or
+    // half of it and the result odd
+    const unsigned r = __funnelshift_l(l, t, 3), rem = l << 3;  // rem: the 29 bits, left-aligned
+    const unsigned up = rem > 0x80000000u || (rem == 0x80000000u && (r & 1u));
+    return __uint_as_float((r + up) | (h & 0x80000000u));
+}
+__device__ __forceinline__ double to_double(float x) {
+    const unsigned b = __float_as_uint(x), m = b & 0x7FFFFFFFu;
+    if (m - (1u << 23) >= (254u << 23)) {  // zero, subnormal, infinite or not a number
+        if (m != 0u) return (double)x;
+        return __hiloint2double((int)b, 0);
+    }
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + (896u << 20))), (int)(b << 29));
+}
 __device__ __forceinline__ float2 to_c(float2 v, float) { return v; }
-__device__ __forceinline__ float2 to_c(double2 v, float) { return make_float2((float)v.x, (float)v.y); }
-__device__ __forceinline__ double2 to_c(float2 v, double) { return make_double2((double)v.x, (double)v.y); }
+__device__ __forceinline__ float2 to_c(double2 v, float) { return make_float2(to_float(v.x), to_float(v.y)); }
+__device__ __forceinline__ double2 to_c(float2 v, double) { return make_double2(to_double(v.x), to_double(v.y)); }
 __device__ __forceinline__ double2 to_c(double2 v, double) { return v; }
 
 // ------------------------------------------------------------------------------ operator
@@ -201,10 +230,11 @@ cudaError_t launch_rb(const DevOp<R> &op, int dim, R omega, const CB *b, typenam
 template <typename R, typename CB>
 cudaError_t launch_residual_restrict(const DevOp<R> &op, int dim, const CB *b, const typename CT<R>::T *u,
                                      typename CT<R>::T *rc, cudaStream_t s, bool red = false, bool first = false);
-// uf += P ec (fine nodes nf).
+// uf += P ec (fine nodes nf).  black: a red-black sweep with omega = 1 follows, which does not use the
+// first colour's values (3D then leaves those nodes as they are).
 template <typename R>
 cudaError_t launch_prolong_add(const int nf[3], int dim, const typename CT<R>::T *ec, typename CT<R>::T *uf,
-                               cudaStream_t s, const int *gate = nullptr);
+                               cudaStream_t s, const int *gate = nullptr, bool black = false);
 // u = Minv b on the interior unknowns of the coarsest grid (nodes n), natural order.
 template <typename R>
 cudaError_t launch_dense_solve(const int n[3], int dim, int nu, const typename CT<R>::T *minv,
@@ -241,6 +271,13 @@ cudaError_t launch_tile_post(const DevOp<R> &op, R omega, int nu, int rb, const 
                              cudaStream_t s);
 cudaError_t launch_pre2_restrict(const DevOp<float> &op, int tile, float omega, const float2 *b, float2 *u_out,
                                  float2 *rc, cudaStream_t s);
+// The first launch of a complex64 cycle on a complex128 right-hand side v: as launch_pre2_restrict (2D,
+// not the wavefront) or the first sweep from zero (3D), with v's interior rounded to complex64 written
+// to b_out on the way instead of by a conversion pass of its own.
+cudaError_t launch_pre2_restrict_c128(const DevOp<float> &op, int tile, float omega, const double2 *v, float2 *b_out,
+                                      float2 *u_out, float2 *rc, cudaStream_t s);
+cudaError_t launch_jacobi3_first(const DevOp<float> &op, float omega, const double2 *v, float2 *b_out, float2 *u_out,
+                                 cudaStream_t s);
 cudaError_t launch_prolong_post2(const DevOp<float> &op, int tile, float omega, const float2 *b, const float2 *u_in,
                                  float2 *u_out, const float2 *ec, cudaStream_t s);
 
@@ -257,7 +294,12 @@ constexpr size_t CT_SMEM_BYTES = 200 * 1024;
 // cycle on GB300 with the level above the line in / out of the tail: 2D complex64 129^2 24.7 / 27.2
 // us (V(2,2) on 129^2) but 161^2 30.3 / 27.4; 2D complex128 81^2 86 / 106 us (161^2), 129^2 does not
 // fit; 3D 21^3 43.1 / 45.9 us complex64 and 235 / 317 us complex128 (41^3), but 25^3 47.2 / 46.3.
-constexpr int tail_max_unknowns(int dim, size_t es) { return dim == 2 && es == sizeof(float2) ? 16384 : 8192; }
+// A level of a complex64 V(2,2) omega-Jacobi cycle has fast launches of its own (two per visit), so the
+// line is lower there: 193^2 with 97^2 in / out of the tail 26.5 / 28.5 us, 257^2 with 129^2 30.7 / 29.4 --
+// but a grid that fits the tail whole goes there (129^2: 24.7 us).
+constexpr int tail_max_unknowns(int dim, size_t es, bool v22, bool whole) {
+    return dim == 2 && es == sizeof(float2) ? (v22 && !whole ? 10000 : 16384) : 8192;
+}
 // Nested row slabs of the tail levels: block r owns the interior rows B[l][r] .. B[l][r+1]-1 of
 // level l (level 0 in runs of ceil((rows - 2) / nc), B[l+1][r] = (B[l][r] + 1) / 2).  False
 // unless every level but the last has an odd number of rows and the next has half of them.

@@ -13,49 +13,56 @@ namespace {
 
 constexpr int BX = 32, BY = 8, KCHUNK = 8;
 
-// acc += a * z with a = (re.hi, re.lo, im.hi, im.lo) and a float complex z.
+// acc += a * z with a = (re.hi, re.lo, im.hi, im.lo) and a float complex z.  REAL: a's imaginary part is
+// zero, and its products, which add exact zeros, are left out (the same result).
+template <bool REAL>
 __device__ __forceinline__ void cmac(float4 a, float2 z, float &sr, float &cr, float &si, float &ci) {
     const ff ar{a.x, a.y}, ai{a.z, a.w};
     float p, e;
     ff_prod_f(ar, z.x, p, e);
     ff_acc_prod(sr, cr, p, e);
-    ff_prod_f(ai, z.y, p, e);
-    ff_acc_prod(sr, cr, -p, -e);
+    if (!REAL) {
+        ff_prod_f(ai, z.y, p, e);
+        ff_acc_prod(sr, cr, -p, -e);
+    }
     ff_prod_f(ar, z.y, p, e);
     ff_acc_prod(si, ci, p, e);
-    ff_prod_f(ai, z.x, p, e);
-    ff_acc_prod(si, ci, p, e);
+    if (!REAL) {
+        ff_prod_f(ai, z.x, p, e);
+        ff_acc_prod(si, ci, p, e);
+    }
 }
 
 // The first term of the sums: (sr, cr) and (si, ci) start as its exact products (what adding
 // them to zero accumulators with TwoSum gives, up to the sign of a zero).
+template <bool REAL>
 __device__ __forceinline__ void cmac_first(float4 a, float2 z, float &sr, float &cr, float &si, float &ci) {
     const ff ar{a.x, a.y}, ai{a.z, a.w};
     float p, e;
     ff_prod_f(ar, z.x, sr, cr);
-    ff_prod_f(ai, z.y, p, e);
-    ff_acc_prod(sr, cr, -p, -e);
+    if (!REAL) {
+        ff_prod_f(ai, z.y, p, e);
+        ff_acc_prod(sr, cr, -p, -e);
+    }
     ff_prod_f(ar, z.y, si, ci);
-    ff_prod_f(ai, z.x, p, e);
-    ff_acc_prod(si, ci, p, e);
+    if (!REAL) {
+        ff_prod_f(ai, z.x, p, e);
+        ff_acc_prod(si, ci, p, e);
+    }
+}
+__device__ __forceinline__ bool real3(const float4 *t) {
+    return t[0].z == 0.f && t[0].w == 0.f && t[1].z == 0.f && t[1].w == 0.f && t[2].z == 0.f && t[2].w == 0.f;
 }
 
 // (bx, by, bz): this block's tile of interior nodes.  GATED: gv != 0 (a gate flag's value)
 // returns once the first operands have been loaded, writing nothing (the 2D form then loads a
 // node's operands before its arithmetic; without the gate they are loaded as the arithmetic
 // uses them, which keeps the batched kernel at 32 registers).
-template <int DIM, bool GATED>
-__device__ __forceinline__ void apply_A_df_tile(const DevOpDF &o, const float2 *__restrict__ z, float4 *__restrict__ y,
-                                                int bx, int by, int bz, int gv = 0) {
-    const int nx = o.n[0], ny = o.n[1], nz = o.n[2];
-    const int i = bx * BX + threadIdx.x + 1;
-    const int j = by * BY + threadIdx.y + 1;
-    if (i > nx - 2 || j > ny - 2) return;
-    int k0 = 0, k1 = 1;
-    if (DIM == 3) {
-        k0 = bz * KCHUNK + 1;
-        k1 = min(k0 + KCHUNK, nz - 1);
-    }
+template <int DIM, bool GATED, bool RX, bool RY, bool RZ>
+__device__ __forceinline__ void apply_A_df_march(const DevOpDF &o, const float2 *__restrict__ z, float4 *__restrict__ y,
+                                                 int i, int j, int k0, int k1, int gv) {
+    constexpr bool RD = RX && RY && RZ;
+    const int nx = o.n[0], ny = o.n[1];
     const size_t sy = (size_t)nx, sz = (size_t)nx * ny;
     const float4 cxw = o.coef[0][3 * i], cxc = o.coef[0][3 * i + 1], cxe = o.coef[0][3 * i + 2];
     const float4 cyw = o.coef[1][3 * j], cyc = o.coef[1][3 * j + 1], cye = o.coef[1][3 * j + 2];
@@ -80,18 +87,18 @@ __device__ __forceinline__ void apply_A_df_tile(const DevOpDF &o, const float2 *
                 kk2 = o.k2[q];
             }
             float sr, cr, si, ci;
-            cmac_first(cxw, zw, sr, cr, si, ci);
-            cmac(cxe, ze, sr, cr, si, ci);
-            cmac(cyw, zs, sr, cr, si, ci);
-            cmac(cye, zn, sr, cr, si, ci);
+            cmac_first<RX>(cxw, zw, sr, cr, si, ci);
+            cmac<RX>(cxe, ze, sr, cr, si, ci);
+            cmac<RY>(cyw, zs, sr, cr, si, ci);
+            cmac<RY>(cye, zn, sr, cr, si, ci);
             ff dr = dxy_r, di = dxy_i;
             const float4 czw = o.coef[2][3 * k], czc = o.coef[2][3 * k + 1], cze = o.coef[2][3 * k + 2];
-            cmac(czw, zm, sr, cr, si, ci);
-            cmac(cze, zp, sr, cr, si, ci);
+            cmac<RZ>(czw, zm, sr, cr, si, ci);
+            cmac<RZ>(cze, zp, sr, cr, si, ci);
             dr = ff_add(dr, ff{czc.x, czc.y});
             di = ff_add(di, ff{czc.z, czc.w});
             dr = ff_add(dr, ff{-kk.x, -kk.y});
-            cmac(make_float4(dr.hi, dr.lo, di.hi, di.lo), zc, sr, cr, si, ci);
+            cmac<RD>(make_float4(dr.hi, dr.lo, di.hi, di.lo), zc, sr, cr, si, ci);
             const ff yr = ff_norm(sr, cr), yi = ff_norm(si, ci);
             y[p] = make_float4(yr.hi, yr.lo, yi.hi, yi.lo);
             zm = zc;
@@ -109,24 +116,50 @@ __device__ __forceinline__ void apply_A_df_tile(const DevOpDF &o, const float2 *
                 const float2 kk = o.k2[p];
                 zc = z[p];
                 if (gv) return;
-                cmac_first(cxw, zw, sr, cr, si, ci);
-                cmac(cxe, ze, sr, cr, si, ci);
-                cmac(cyw, zs, sr, cr, si, ci);
-                cmac(cye, zn, sr, cr, si, ci);
+                cmac_first<RX>(cxw, zw, sr, cr, si, ci);
+                cmac<RX>(cxe, ze, sr, cr, si, ci);
+                cmac<RY>(cyw, zs, sr, cr, si, ci);
+                cmac<RY>(cye, zn, sr, cr, si, ci);
                 dr = ff_add(dr, ff{-kk.x, -kk.y});  // diagonal: sum of centre coefficients - k^2
             } else {
-                cmac_first(cxw, z[p - 1], sr, cr, si, ci);
-                cmac(cxe, z[p + 1], sr, cr, si, ci);
-                cmac(cyw, z[p - sy], sr, cr, si, ci);
-                cmac(cye, z[p + sy], sr, cr, si, ci);
+                cmac_first<RX>(cxw, z[p - 1], sr, cr, si, ci);
+                cmac<RX>(cxe, z[p + 1], sr, cr, si, ci);
+                cmac<RY>(cyw, z[p - sy], sr, cr, si, ci);
+                cmac<RY>(cye, z[p + sy], sr, cr, si, ci);
                 const float2 kk = o.k2[p];
                 dr = ff_add(dr, ff{-kk.x, -kk.y});
                 zc = z[p];
             }
-            cmac(make_float4(dr.hi, dr.lo, di.hi, di.lo), zc, sr, cr, si, ci);
+            cmac<RD>(make_float4(dr.hi, dr.lo, di.hi, di.lo), zc, sr, cr, si, ci);
             const ff yr = ff_norm(sr, cr), yi = ff_norm(si, ci);
             y[p] = make_float4(yr.hi, yr.lo, yi.hi, yi.lo);
         }
+    }
+}
+
+// In 3D each warp picks the form by axis (x: all its columns, y: its row, z: all its planes): the
+// coefficients are real outside the absorbing layers, and a real axis takes half the products.  The 2D
+// kernels keep the one form (measured: the same single-solve time, and the batched one slower for the
+// two registers more: 78.0 against 76.0 ms per 12-problem batch).
+template <int DIM, bool GATED>
+__device__ __forceinline__ void apply_A_df_tile(const DevOpDF &o, const float2 *__restrict__ z, float4 *__restrict__ y,
+                                                int bx, int by, int bz, int gv = 0) {
+    const int nx = o.n[0], ny = o.n[1], nz = o.n[2];
+    const int i = bx * BX + threadIdx.x + 1;
+    const int j = by * BY + threadIdx.y + 1;
+    if (i > nx - 2 || j > ny - 2) return;
+    if constexpr (DIM == 2) {
+        apply_A_df_march<2, GATED, false, false, false>(o, z, y, i, j, 0, 1, gv);
+    } else {
+        const int k0 = bz * KCHUNK + 1, k1 = min(k0 + KCHUNK, nz - 1);
+        const bool rx = __all_sync(__activemask(), real3(o.coef[0] + 3 * i)), ry = real3(o.coef[1] + 3 * j);
+        bool rz = true;
+        for (int k = k0; k < k1; k++) rz = rz && real3(o.coef[2] + 3 * k);
+        if (rx && ry && rz) apply_A_df_march<DIM, GATED, true, true, true>(o, z, y, i, j, k0, k1, gv);
+        else if (rx && ry) apply_A_df_march<DIM, GATED, true, true, false>(o, z, y, i, j, k0, k1, gv);
+        else if (rx && rz) apply_A_df_march<DIM, GATED, true, false, true>(o, z, y, i, j, k0, k1, gv);
+        else if (ry && rz) apply_A_df_march<DIM, GATED, false, true, true>(o, z, y, i, j, k0, k1, gv);
+        else apply_A_df_march<DIM, GATED, false, false, false>(o, z, y, i, j, k0, k1, gv);
     }
 }
 

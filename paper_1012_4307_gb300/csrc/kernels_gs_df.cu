@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(NT) k_pair_to_c128(size_t n, const float4 *__r
     const double r = block_recip(alpha);
     for (size_t q = blockIdx.x * (size_t)NT + threadIdx.x; q < n; q += (size_t)gridDim.x * NT) {
         const float4 a = v[q];
-        z[q] = make_double2(((double)a.x + (double)a.y) * r, ((double)a.z + (double)a.w) * r);
+        z[q] = make_double2((to_double(a.x) + to_double(a.y)) * r, (to_double(a.z) + to_double(a.w)) * r);
     }
 }
 

@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(NT) k_combine_df(size_t n, const float2 *__res
             ff_prod_f(yr, z.y, p, e); ff_acc_prod(si, ci, p, e);
         }
         const double2 xq = x[q];
-        x[q] = make_double2(xq.x + ((double)sr + (double)cr), xq.y + ((double)si + (double)ci));
+        x[q] = make_double2(xq.x + (to_double(sr) + to_double(cr)), xq.y + (to_double(si) + to_double(ci)));
     }
 }
 

@@ -208,11 +208,13 @@ __global__ void __launch_bounds__(BX *BY) k_jacobi(OpView<R> o, R omega, const C
 // 3D omega-Jacobi: k_jacobi's arithmetic in the same order, with the x and y coefficient
 // triples loaded once per thread, the (z - 1, z, z + 1) column in registers, and the next plane's
 // operands (four in-plane neighbours, z + 2, b, k^2) loaded while this plane is computed.
-// KC: fine planes per thread (shorter chunks on small grids give more blocks).
+// KC: fine planes per thread (shorter chunks on small grids give more blocks).  ZERO with a complex128 b
+// in a complex64 cycle: the sweep also writes b rounded to complex64 to b_out.
 template <typename R, typename CB, bool ZERO, int KC>
 __global__ void __launch_bounds__(BX *BY) k_jacobi3(OpView<R> o, R omega, const CB *__restrict__ b,
                                                     const typename CT<R>::T *__restrict__ u,
-                                                    typename CT<R>::T *__restrict__ un) {
+                                                    typename CT<R>::T *__restrict__ un,
+                                                    typename CT<R>::T *__restrict__ b_out) {
     pdl_enter();
     const int gv = gate_value(o.gate);
     typedef typename CT<R>::T C;
@@ -269,6 +271,7 @@ __global__ void __launch_bounds__(BX *BY) k_jacobi3(OpView<R> o, R omega, const 
                 kn = o.k2[p + sz];
             }
             const C d = cadd(cadd(dxy, cadd(cscale(o.bk, kq), o.c)), __ldg(&o.cz[3 * k + 1]));
+            if (sizeof(CB) != sizeof(C)) b_out[p] = bq;  // b is complex128: keep what the sweep used
             un[p] = cscale(cmul(bq, cinv(d)), omega);
             bq = bn;
             kq = kn;
@@ -289,6 +292,14 @@ __global__ void __launch_bounds__(BX *BY) k_jacobi3(OpView<R> o, R omega, const 
             xp2 = u[q + sz];
             bn = to_c(b[q], R());
             kn = o.k2[q];
+        }
+        // the lines two planes ahead into L2 (257^3: 733 us per cycle with them, 747 without; further
+        // ahead or in the residual kernel no gain)
+        if (k + 2 < k1 && (threadIdx.x & 15) == 0) {
+            const size_t q = p + 2 * sz;
+            l2_prefetch(&u[q + sz]);
+            l2_prefetch(&b[q]);
+            l2_prefetch(&o.k2[q]);
         }
         C acc = cmul(cwx, xw);
         acc = cfma(cex, xe, acc);
@@ -313,11 +324,11 @@ __global__ void __launch_bounds__(BX *BY) k_jacobi3(OpView<R> o, R omega, const 
 
 // one colour of omega-red-black Jacobi, in place: threads map to every other x node and march kc
 // planes.  FROM: the iterate on entry is given (RB_ANY), zero everywhere and not read (RB_ZERO: the
-// first colour of a sweep from zero is pointwise), or zero on this colour and not read there
-// (RB_OWN_ZERO: the second colour).  complex128 takes omega / D as formed once (see k_jacobi3).
+// first colour of a sweep from zero is pointwise), or zero on this colour, or omega = 1, and not read
+// there (RB_NO_OWN: the second colour of a sweep from zero, any colour with omega = 1).  complex128 takes omega / D as formed once (see k_jacobi3).
 // Measured, 193 x 129 x 97 complex128 V(1,1) cycle: 1318 us with the diagonal assembled and divided by
 // at every node, a zero fill before the first sweep and chunks of 8 planes on every level, 719 us so.
-enum { RB_ANY, RB_ZERO, RB_OWN_ZERO };
+enum { RB_ANY, RB_ZERO, RB_NO_OWN };
 template <typename R, int DIM, typename CB, int FROM>
 __global__ void __launch_bounds__(BX *BY) k_rb(OpView<R> o, R omega, const CB *__restrict__ b, typename CT<R>::T *u, int colour,
                                                int kc) {
@@ -424,15 +435,20 @@ __global__ void __launch_bounds__(BX *BY) k_prolong_add(int nx, int ny, int nz, 
 // 2 K0 - 1 .. 2 K1 - 1 like k_jacobi3 (coefficients in registers, the u column (z - 1, z, z + 1)
 // in registers, the next plane's operands loaded while this plane is computed).  Each thread weighs its
 // own residuals by (1, 2, 1) along z in registers; once per coarse plane the weighted plane goes through
-// shared memory (two buffers, one barrier) and the coarse nodes' threads apply (1, 2, 1) in x and y --
-// one exchange and one 3 x 3 sum per coarse plane instead of one per fine plane.  An odd fine plane
-// 2K + 1 completes coarse plane K and starts K + 1.  Fine nodes outside the grid's interior hold zero
+// shared memory and the coarse nodes' threads apply (1, 2, 1) in x and y.  The four groups of four warps
+// take turns at that sum: a group waits for the plane in its own turn only and merely arrives at the
+// barrier in the others' (four buffers, four barriers), so that the sum does not hold up the march of
+// the other warps.  A buffer is written again four coarse planes later, when every warp has since waited
+// in a turn of its own, behind the group that read it.  (257^3 complex64 finest level: 141 us per launch
+// with one barrier and the same four warps summing every fine plane, 128 us with the z sums in registers,
+// the cycle 725 -> 700 us with the turns; four lanes per coarse node in every warp instead: 141 us.)  An odd fine plane 2K + 1 completes coarse plane
+// K and starts K + 1.  Fine nodes outside the grid's interior hold zero
 // residuals.  Same weights as k_residual_restrict, applied per axis.
 constexpr int R3_TX = 16, R3_TY = 8, R3_KC = 8;
 constexpr int R3_FW = 2 * R3_TX + 1, R3_FH = 2 * R3_TY + 1;  // fine region
 constexpr int R3_NT = ((R3_FW * R3_FH + 31) / 32) * 32;       // threads: one per region node
-template <typename R> constexpr size_t r3_smem_bytes() {
-    return (size_t)2 * R3_FW * R3_FH * sizeof(typename CT<R>::T);
+template <typename R> constexpr size_t r3_smem_bytes(int planes) {
+    return (size_t)planes * R3_FW * R3_FH * sizeof(typename CT<R>::T);
 }
 
 template <typename R, typename CB>
@@ -468,9 +484,9 @@ __global__ void __launch_bounds__(R3_NT, sizeof(R) == sizeof(float) ? 2 : 1)
         kq = o.k2[p];
     }
     if (gv) return;  // the same value in every thread: no barrier is left waiting
-    // the coarse node of this thread (threads below R3_TX * R3_TY)
-    const int cx = t % R3_TX, cy = t / R3_TX, I = I0 + cx, J = J0 + cy;
-    const bool own = t < R3_TX * R3_TY && I <= ncx - 2 && J <= ncy - 2;
+    // the coarse node this thread sums in its warp group's turns (warps 0 .. 15)
+    const int group = (t >> 7) & 3, cn = t & 127, cx = cn % R3_TX, cy = cn / R3_TX, I = I0 + cx, J = J0 + cy;
+    const bool own = t < 512 && I <= ncx - 2 && J <= ncy - 2;
     C acc = zero;  // z sum of this fine column for the current coarse plane
     for (int z = zs; z <= ze; z++, p += sz) {
         C r = zero;
@@ -507,20 +523,24 @@ __global__ void __launch_bounds__(R3_NT, sizeof(R) == sizeof(float) ? 2 : 1)
         // fine plane 2K + 1 (K = (z - 1) / 2) completes coarse plane K and starts K + 1
         const int K = (z - 1) >> 1;
         if (K >= K0) {
-            C(*buf)[R3_FW] = rbuf[K & 1];
+            const int turn = (K - K0) & 3;
+            C(*buf)[R3_FW] = rbuf[turn];
             if (region) buf[ly][lx] = cadd(acc, r);
-            __syncthreads();
-            if (own) {
-                // (1, 2, 1) along x on the three fine rows 2J - 1 .. 2J + 1, then along y
-                const int fx = 2 * cx, fy = 2 * cy;
-                C a[3];
+            if (turn != group) {
+                asm volatile("bar.arrive %0, %1;" ::"r"(1 + turn), "n"(R3_NT) : "memory");
+            } else {
+                asm volatile("bar.sync %0, %1;" ::"r"(1 + turn), "n"(R3_NT) : "memory");
+                if (own) {
+                    // (1, 2, 1) along x on the three fine rows 2J - 1 .. 2J + 1, then along y
+                    C a[3];
 #pragma unroll
-                for (int dy = 0; dy < 3; dy++) {
-                    const C *row = &buf[fy + dy][fx];
-                    a[dy] = cadd(cadd(row[0], row[2]), cscale(row[1], R(2)));
+                    for (int dy = 0; dy < 3; dy++) {
+                        const C *row = &buf[2 * cy + dy][2 * cx];
+                        a[dy] = cadd(cadd(row[0], row[2]), cscale(row[1], R(2)));
+                    }
+                    rc[(size_t)I + (size_t)ncx * ((size_t)J + (size_t)ncy * K)] =
+                        cscale(cadd(cadd(a[0], a[2]), cscale(a[1], R(2))), R(1.0 / 64.0));
                 }
-                rc[(size_t)I + (size_t)ncx * ((size_t)J + (size_t)ncy * K)] =
-                    cscale(cadd(cadd(a[0], a[2]), cscale(a[1], R(2))), R(1.0 / 64.0));
             }
         }
         acc = r;
@@ -602,6 +622,37 @@ __global__ void __launch_bounds__(R3R_NT, 2)
 // 3D prolongation + correction in closed form: uf[p] += 1/8 of the sum of ec at the eight corners
 // (floor / ceil of i/2, j/2, k/2), coincident corners repeated, i.e. the average over the distinct
 // coarse nodes of k_prolong_add.  Each thread marches kc fine planes.
+// The same for the nodes with odd i + j + k only (threads map to every other x node): before a red-black sweep
+// with omega = 1, whose first colour does not use its old values.
+template <typename R>
+__global__ void __launch_bounds__(BX *BY) k_prolong3_black(int nx, int ny, int nz, const typename CT<R>::T *__restrict__ ec,
+                                                           typename CT<R>::T *__restrict__ uf, int kc,
+                                                           const int *__restrict__ gate) {
+    pdl_enter();
+    if (gate && *gate) return;
+    typedef typename CT<R>::T C;
+    const int t = blockIdx.x * BX + threadIdx.x;
+    const int j = blockIdx.y * BY + threadIdx.y + 1;
+    if (j > ny - 2) return;
+    const int ncx = (nx + 1) / 2, ncy = (ny + 1) / 2;
+    const int k0 = blockIdx.z * kc + 1, k1 = min(k0 + kc, nz - 1);
+    const size_t csy = (size_t)ncx, csz = (size_t)ncx * ncy, ja = csy * (j >> 1), jb = csy * ((j + 1) >> 1);
+#pragma unroll 2
+    for (int k = k0; k < k1; k++) {
+        const int i = 2 * t + 1 + ((j + k) & 1);
+        if (i > nx - 2) continue;
+        const size_t p = (size_t)i + (size_t)nx * ((size_t)j + (size_t)ny * k);
+        const int ia = i >> 1, ib = (i + 1) >> 1;
+        auto corner_sum = [&](int c) {
+            const C *e = ec + csz * c;
+            return cadd(cadd(e[ja + ia], e[ja + ib]), cadd(e[jb + ia], e[jb + ib]));
+        };
+        const C uq = uf[p], sa = corner_sum(k >> 1);
+        if (k & 1) uf[p] = cadd(uq, cscale(cadd(sa, corner_sum((k + 1) >> 1)), R(0.125)));
+        else uf[p] = cadd(uq, cscale(sa, R(0.25)));
+    }
+}
+
 template <typename R>
 __global__ void __launch_bounds__(BX *BY) k_prolong3(int nx, int ny, int nz, const typename CT<R>::T *__restrict__ ec,
                                                      typename CT<R>::T *__restrict__ uf, int kc,
@@ -788,10 +839,12 @@ __device__ __forceinline__ float2 tile_diag(const TC &tc, int sx, int sy, float 
 // rc = FW(b - M u) on the owned coarse nodes.  Blocks whose region lies inside the grid's
 // interior skip the per-node boundary tests.
 // (bx, by): the tile of coarse nodes this block owns.
-template <int TCX, int TCY>
-__device__ __forceinline__ void pre2_restrict_tile(const OpView<float> &o, float omega, const float2 *__restrict__ b,
+// CB double2: b is a complex128 vector; its owned nodes rounded to complex64 go to b_out too.
+template <int TCX, int TCY, typename CB>
+__device__ __forceinline__ void pre2_restrict_tile(const OpView<float> &o, float omega, const CB *__restrict__ b,
                                                    float2 *__restrict__ u, float2 *__restrict__ rc, int ncx, int ncy,
-                                                   int bx, int by, const int *gate = nullptr) {
+                                                   int bx, int by, const int *gate = nullptr,
+                                                   float2 *__restrict__ b_out = nullptr) {
     typedef Tile<TCX, TCY> TL;
     constexpr int RW = TL::RW, RH = TL::RH;
     extern __shared__ __align__(16) unsigned char pre_smem[];
@@ -812,7 +865,7 @@ __device__ __forceinline__ void pre2_restrict_tile(const OpView<float> &o, float
         float2 bv = make_float2(0.f, 0.f), dv = make_float2(0.f, 0.f);
         if (inside(x, y)) {
             const size_t p = (size_t)x + (size_t)nx * y;
-            bv = b[p];
+            bv = to_c(b[p], 0.f);
             dv = o.dinv[p];
         }
         T.b[sy][sx] = bv;
@@ -833,7 +886,10 @@ __device__ __forceinline__ void pre2_restrict_tile(const OpView<float> &o, float
     for_region<RW, RH, TL::NT>([&](int sx, int sy) {
         const int x = X0 + sx, y = Y0 + sy;
         const bool in = inside(x, y);
-        if (in && sx >= 2 && sx < 2 + 2 * TCX && sy >= 2 && sy < 2 + 2 * TCY) u[(size_t)x + (size_t)nx * y] = T.u2[sy][sx];
+        if (in && sx >= 2 && sx < 2 + 2 * TCX && sy >= 2 && sy < 2 + 2 * TCY) {
+            u[(size_t)x + (size_t)nx * y] = T.u2[sy][sx];
+            if (sizeof(CB) == sizeof(double2)) b_out[(size_t)x + (size_t)nx * y] = T.b[sy][sx];
+        }
         float2 r = make_float2(0.f, 0.f);
         if (in && sx >= 2 && sx < RW - 2 && sy >= 2 && sy < RH - 2) {
             const float2 d = cinv_fast(T.di[sy][sx]);
@@ -856,12 +912,12 @@ __device__ __forceinline__ void pre2_restrict_tile(const OpView<float> &o, float
     }
 }
 
-template <int TCX, int TCY>
-__global__ void __launch_bounds__(Tile<TCX, TCY>::NT, 4) k_pre2_restrict(OpView<float> o, float omega, const float2 *__restrict__ b,
+template <int TCX, int TCY, typename CB>
+__global__ void __launch_bounds__(Tile<TCX, TCY>::NT, 4) k_pre2_restrict(OpView<float> o, float omega, const CB *__restrict__ b,
                                                        float2 *__restrict__ u, float2 *__restrict__ rc, int ncx,
-                                                       int ncy) {
+                                                       int ncy, float2 *__restrict__ b_out) {
     pdl_enter();
-    pre2_restrict_tile<TCX, TCY>(o, omega, b, u, rc, ncx, ncy, blockIdx.x, blockIdx.y, o.gate);
+    pre2_restrict_tile<TCX, TCY>(o, omega, b, u, rc, ncx, ncy, blockIdx.x, blockIdx.y, o.gate, b_out);
 }
 
 // u_out <- two omega-Jacobi sweeps of (u_in + P ec), on the owned fine nodes.  u_in and u_out
@@ -998,25 +1054,44 @@ cudaError_t launch_jacobi(const DevOp<R> &op, int dim, R omega, const CB *bb, co
     if (dim == 3) {
         const int kc = z_chunk((size_t)g.x * g.y, op.n[2] - 2, KCHUNK, 152 * 10);
         g.z = cdiv(op.n[2] - 2, kc);
+        typename CT<R>::T *none = nullptr;
+        auto go = [&](auto kernel) { return launch_pdl(kernel, g, b, 0, s, view(op), omega, bb, u_in, u_out, none); };
         if (u_in == nullptr) {
             switch (kc) {
-            case 8: launch_pdl(k_jacobi3<R, CB, true, 8>, g, b, 0, s, view(op), omega, bb, u_in, u_out); break;
-            case 4: launch_pdl(k_jacobi3<R, CB, true, 4>, g, b, 0, s, view(op), omega, bb, u_in, u_out); break;
-            case 2: launch_pdl(k_jacobi3<R, CB, true, 2>, g, b, 0, s, view(op), omega, bb, u_in, u_out); break;
-            default: launch_pdl(k_jacobi3<R, CB, true, 1>, g, b, 0, s, view(op), omega, bb, u_in, u_out); break;
+            case 8: go(k_jacobi3<R, CB, true, 8>); break;
+            case 4: go(k_jacobi3<R, CB, true, 4>); break;
+            case 2: go(k_jacobi3<R, CB, true, 2>); break;
+            default: go(k_jacobi3<R, CB, true, 1>); break;
             }
         } else {
             switch (kc) {
-            case 8: launch_pdl(k_jacobi3<R, CB, false, 8>, g, b, 0, s, view(op), omega, bb, u_in, u_out); break;
-            case 4: launch_pdl(k_jacobi3<R, CB, false, 4>, g, b, 0, s, view(op), omega, bb, u_in, u_out); break;
-            case 2: launch_pdl(k_jacobi3<R, CB, false, 2>, g, b, 0, s, view(op), omega, bb, u_in, u_out); break;
-            default: launch_pdl(k_jacobi3<R, CB, false, 1>, g, b, 0, s, view(op), omega, bb, u_in, u_out); break;
+            case 8: go(k_jacobi3<R, CB, false, 8>); break;
+            case 4: go(k_jacobi3<R, CB, false, 4>); break;
+            case 2: go(k_jacobi3<R, CB, false, 2>); break;
+            default: go(k_jacobi3<R, CB, false, 1>); break;
             }
         }
     } else if (u_in == nullptr) {
         launch_pdl(k_jacobi<R, 2, CB, true>, g, b, 0, s, view(op), omega, bb, u_in, u_out);
     } else {
         launch_pdl(k_jacobi<R, 2, CB, false>, g, b, 0, s, view(op), omega, bb, u_in, u_out);
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_jacobi3_first(const DevOp<float> &op, float omega, const double2 *v, float2 *b_out, float2 *u_out,
+                                 cudaStream_t s) {
+    const int dim = 3;
+    dim3 g = grid_for(op.n, dim), b(BX, BY);
+    const int kc = z_chunk((size_t)g.x * g.y, op.n[2] - 2, KCHUNK, 152 * 10);
+    g.z = cdiv(op.n[2] - 2, kc);
+    const float2 *none = nullptr;
+    auto go = [&](auto kernel) { return launch_pdl(kernel, g, b, 0, s, view(op), omega, v, none, u_out, b_out); };
+    switch (kc) {
+    case 8: go(k_jacobi3<float, double2, true, 8>); break;
+    case 4: go(k_jacobi3<float, double2, true, 4>); break;
+    case 2: go(k_jacobi3<float, double2, true, 2>); break;
+    default: go(k_jacobi3<float, double2, true, 1>); break;
     }
     return cudaGetLastError();
 }
@@ -1029,14 +1104,15 @@ cudaError_t launch_rb(const DevOp<R> &op, int dim, R omega, const CB *bb, typena
     const int kc = dim == 3 ? z_chunk((size_t)g.x * g.y, op.n[2] - 2, KCHUNK, 152 * 10) : 1;
     if (dim == 3) g.z = cdiv(op.n[2] - 2, kc);
     auto go = [&](auto kernel) { return launch_pdl(kernel, g, b, 0, s, view(op), omega, bb, u, colour, kc); };
+    const bool no_own = zero || omega == R(1);
     if (dim == 3) {
-        if (!zero) go(k_rb<R, 3, CB, RB_ANY>);
-        else if (colour == 0) go(k_rb<R, 3, CB, RB_ZERO>);
-        else go(k_rb<R, 3, CB, RB_OWN_ZERO>);
+        if (zero && colour == 0) go(k_rb<R, 3, CB, RB_ZERO>);
+        else if (no_own) go(k_rb<R, 3, CB, RB_NO_OWN>);
+        else go(k_rb<R, 3, CB, RB_ANY>);
     } else {
-        if (!zero) go(k_rb<R, 2, CB, RB_ANY>);
-        else if (colour == 0) go(k_rb<R, 2, CB, RB_ZERO>);
-        else go(k_rb<R, 2, CB, RB_OWN_ZERO>);
+        if (zero && colour == 0) go(k_rb<R, 2, CB, RB_ZERO>);
+        else if (no_own) go(k_rb<R, 2, CB, RB_NO_OWN>);
+        else go(k_rb<R, 2, CB, RB_ANY>);
     }
     return cudaGetLastError();
 }
@@ -1049,18 +1125,13 @@ cudaError_t launch_residual_restrict(const DevOp<R> &op, int dim, const CB *bb, 
         dim3 g(cdiv(nc[0] - 2, R3_TX), cdiv(nc[1] - 2, R3_TY), 1);
         const int kc = z_chunk((size_t)g.x * g.y, nc[2] - 2, R3_KC, 152 * 4);
         g.z = cdiv(nc[2] - 2, kc);
-        launch_pdl(k_resrestrict3_red<R, CB>, g, R3R_NT, r3_smem_bytes<R>(), s, view(op), bb, u, rc, nc[0], nc[1], nc[2],
+        launch_pdl(k_resrestrict3_red<R, CB>, g, R3R_NT, r3_smem_bytes<R>(2), s, view(op), bb, u, rc, nc[0], nc[1], nc[2],
                    kc, first ? 1 : 0);
         return cudaGetLastError();
     }
     if (dim == 3 && (size_t)op.n[0] * op.n[1] < ((size_t)1 << 31)) {  // 32-bit in-plane offsets
-        constexpr size_t smem = r3_smem_bytes<R>();
-        static bool attr = false;
-        if (!attr) {
-            cudaError_t e = cudaFuncSetAttribute(k_resrestrict3<R, CB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            attr = true;
-        }
+        constexpr size_t smem = r3_smem_bytes<R>(4);
+        static_assert(smem <= 48 * 1024, "");
         dim3 g(cdiv(nc[0] - 2, R3_TX), cdiv(nc[1] - 2, R3_TY), 1);
         const int kc = z_chunk((size_t)g.x * g.y, nc[2] - 2, R3_KC, 152 * 4);
         g.z = cdiv(nc[2] - 2, kc);
@@ -1075,9 +1146,14 @@ cudaError_t launch_residual_restrict(const DevOp<R> &op, int dim, const CB *bb, 
 
 template <typename R>
 cudaError_t launch_prolong_add(const int nf[3], int dim, const typename CT<R>::T *ec, typename CT<R>::T *uf,
-                               cudaStream_t s, const int *gate) {
+                               cudaStream_t s, const int *gate, bool black) {
     dim3 g = grid_for(nf, dim), b(BX, BY);
-    if (dim == 3) {
+    if (dim == 3 && black) {
+        g.x = cdiv((nf[0] - 1) / 2, BX);
+        const int kc = z_chunk((size_t)g.x * g.y, nf[2] - 2, KCHUNK, 152 * 10);
+        g.z = cdiv(nf[2] - 2, kc);
+        launch_pdl(k_prolong3_black<R>, g, b, 0, s, nf[0], nf[1], nf[2], ec, uf, kc, gate);
+    } else if (dim == 3) {
         const int kc = z_chunk((size_t)g.x * g.y, nf[2] - 2, KCHUNK, 152 * 10);
         g.z = cdiv(nf[2] - 2, kc);
         launch_pdl(k_prolong3<R>, g, b, 0, s, nf[0], nf[1], nf[2], ec, uf, kc, gate);
@@ -1109,19 +1185,19 @@ bool fused_jacobi2_ok(const int n[3], int dim, int tile) {
     return ncx >= 3 && ncy >= 3 && (ncx - 2) % kTiles[tile][0] != 0 && (ncy - 2) % kTiles[tile][1] != 0;
 }
 
-template <int TCX, int TCY>
-static cudaError_t pre2_t(const DevOp<float> &op, float omega, const float2 *b, float2 *u_out, float2 *rc,
+template <int TCX, int TCY, typename CB>
+static cudaError_t pre2_t(const DevOp<float> &op, float omega, const CB *b, float2 *u_out, float2 *rc, float2 *b_out,
                           cudaStream_t s) {
     const int ncx = (op.n[0] + 1) / 2, ncy = (op.n[1] + 1) / 2;
     constexpr size_t smem = sizeof(typename Tile<TCX, TCY>::Pre);
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_pre2_restrict<TCX, TCY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(k_pre2_restrict<TCX, TCY, CB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         attr = true;
     }
     dim3 g(cdiv(ncx - 2, TCX), cdiv(ncy - 2, TCY));
-    launch_pdl(k_pre2_restrict<TCX, TCY>, g, Tile<TCX, TCY>::NT, smem, s, view(op), omega, b, u_out, rc, ncx, ncy);
+    launch_pdl(k_pre2_restrict<TCX, TCY, CB>, g, Tile<TCX, TCY>::NT, smem, s, view(op), omega, b, u_out, rc, ncx, ncy, b_out);
     return cudaGetLastError();
 }
 
@@ -1142,17 +1218,29 @@ static cudaError_t post2_t(const DevOp<float> &op, float omega, const float2 *b,
     return cudaGetLastError();
 }
 
+template <typename CB>
+static cudaError_t pre2_tile(const DevOp<float> &op, int tile, float omega, const CB *b, float2 *u_out, float2 *rc,
+                             float2 *b_out, cudaStream_t s) {
+    switch (tile) {
+    case 0: return pre2_t<32, 8>(op, omega, b, u_out, rc, b_out, s);
+    case 1: return pre2_t<16, 16>(op, omega, b, u_out, rc, b_out, s);
+    case 2: return pre2_t<16, 8>(op, omega, b, u_out, rc, b_out, s);
+    case HELM_TILE_8x8: return pre2_t<8, 8>(op, omega, b, u_out, rc, b_out, s);
+    default: return pre2_t<64, 4>(op, omega, b, u_out, rc, b_out, s);
+    }
+}
+
 cudaError_t launch_pre2_restrict(const DevOp<float> &op, int tile, float omega, const float2 *b, float2 *u_out,
                                  float2 *rc, cudaStream_t s) {
     if (!fused_jacobi2_ok(op.n, 2, tile) || (tile != HELM_TILE_WAVE && !op.dinv)) return cudaErrorInvalidValue;
-    switch (tile) {
-    case HELM_TILE_WAVE: return launch_pre2_wave(op, omega, b, u_out, rc, s);
-    case 0: return pre2_t<32, 8>(op, omega, b, u_out, rc, s);
-    case 1: return pre2_t<16, 16>(op, omega, b, u_out, rc, s);
-    case 2: return pre2_t<16, 8>(op, omega, b, u_out, rc, s);
-    case HELM_TILE_8x8: return pre2_t<8, 8>(op, omega, b, u_out, rc, s);
-    default: return pre2_t<64, 4>(op, omega, b, u_out, rc, s);
-    }
+    if (tile == HELM_TILE_WAVE) return launch_pre2_wave(op, omega, b, u_out, rc, s);
+    return pre2_tile(op, tile, omega, b, u_out, rc, (float2 *)nullptr, s);
+}
+
+cudaError_t launch_pre2_restrict_c128(const DevOp<float> &op, int tile, float omega, const double2 *v, float2 *b_out,
+                                      float2 *u_out, float2 *rc, cudaStream_t s) {
+    if (!fused_jacobi2_ok(op.n, 2, tile) || tile == HELM_TILE_WAVE || !op.dinv) return cudaErrorInvalidValue;
+    return pre2_tile(op, tile, omega, v, u_out, rc, b_out, s);
 }
 
 cudaError_t launch_prolong_post2(const DevOp<float> &op, int tile, float omega, const float2 *b, const float2 *u_in,
@@ -1244,7 +1332,7 @@ template <typename C> cudaError_t launch_zero(size_t n, C *x, cudaStream_t s) {
                                                                 const CT<R>::T *, CT<R>::T *, cudaStream_t, bool, \
                                                                 bool);                                          \
     template cudaError_t launch_prolong_add<R>(const int *, int, const CT<R>::T *, CT<R>::T *, cudaStream_t,      \
-                                               const int *);                                                   \
+                                               const int *, bool);                                             \
     template cudaError_t launch_dense_solve<R>(const int *, int, int, const CT<R>::T *, const CT<R>::T *,        \
                                                 CT<R>::T *, cudaStream_t);
 INST_R(float)

@@ -48,6 +48,7 @@ extern "C" helm_status helm_set_tuning(helm_handle *h, const helm_tuning *t) {
     if (!tuning_valid(*t))
         return helm_fail(HELM_ERR_ARG, "invalid tuning (tail or cluster levels, cluster blocks or halo, or a tile)");
     h->tune = *t;
+    h->tuned = true;
     helm_drop_graphs(h);
     helm_refresh_tails(h, true);
     return HELM_OK;
@@ -77,6 +78,8 @@ extern "C" helm_status helm_autotune(helm_handle *h, helm_prec prec, int reps, h
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     helm_status st = HELM_OK;
     const helm_tuning keep = h->tune;
+    const bool kept_tuned = h->tuned;
+    h->tuned = true;  // the candidates' tiles are what runs
     const bool prof = h->prof.on;
     h->prof.on = false;
     auto fail = [&](cudaError_t e, const char *what) {
@@ -224,6 +227,7 @@ extern "C" helm_status helm_autotune(helm_handle *h, helm_prec prec, int reps, h
     cudaFree(z);
     h->prof.on = prof;
     h->tune = st == HELM_OK ? cur : keep;
+    h->tuned = st == HELM_OK ? true : kept_tuned;
     helm_drop_graphs(h);
     helm_refresh_tails(h, true);
     if (st != HELM_OK) return st;
