@@ -176,7 +176,7 @@ bool plan(BatchLockstep *L, bool commit) {
     // shapes above the tail, each with one tile valid for it
     std::map<std::pair<int, int>, int> tile_of;
     for (int l = 0; l < nr - T; l++) {
-        int t = l < HELM_MAX_LEVELS ? helm_level_tile(R, l) : HELM_TILE_32x8;
+        int t = l < HELM_MAX_LEVELS ? R->tune.level_tile[l] : HELM_TILE_32x8;
         // the small tile pays off when a lone small level leaves most SMs idle; a launch over many
         // problems fills the GPU, where its larger halo share costs time
         if (t == HELM_TILE_8x8) t = HELM_TILE_16x8;

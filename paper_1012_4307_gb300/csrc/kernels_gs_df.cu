@@ -244,7 +244,10 @@ __global__ void __launch_bounds__(NT) k_update_norm_pair(size_t n, const float4 
 // bx: this block's index among the nblk blocks that cover the vector (one launch, or one
 // problem's share of a batched launch).
 // gv != 0 (a gate flag's value): stop after the first loads (the partials are then meaningless).
-template <int CH>
+// STREAM: the basis is loaded as streaming data, so that x and w, which the other block rows read too,
+// stay cached (1025^2: 21.23 -> 21.05 ms per solve; over several problems, where it does not pay, 75.0 ->
+// 77.8 ms per batch of 12, it is off).
+template <int CH, bool STREAM>
 __device__ __forceinline__ void mdot2_body(size_t n, const float4 *__restrict__ V, size_t ldv, int nv,
                                            const float4 *__restrict__ x, const float4 *__restrict__ w,
                                            double2 *__restrict__ partials, int bx, int nblk, int gv = 0) {
@@ -267,7 +270,10 @@ __device__ __forceinline__ void mdot2_body(size_t n, const float4 *__restrict__ 
         const float4 xq = x[q], wq = w[q];
         float4 vq[CH];
 #pragma unroll
-        for (int t = 0; t < CH; t++) vq[t] = t < cnt ? V[(size_t)(i0 + t) * ldv + q] : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int t = 0; t < CH; t++) {
+            const float4 *vp = V + (size_t)(i0 + t) * ldv + q;
+            vq[t] = t >= cnt ? make_float4(0.f, 0.f, 0.f, 0.f) : STREAM ? __ldcs(vp) : *vp;
+        }
         if (gv) break;
         const ff xr = ff_re(xq), xi = ff_im(xq);
 #pragma unroll
@@ -308,7 +314,7 @@ __global__ void __launch_bounds__(NT, 6) k_mdot2_pair(size_t n, const float4 *__
                                                    double2 *__restrict__ partials, const int *__restrict__ gate) {
     pdl_enter();
     const int gv = gate_value(gate);
-    mdot2_body<CH>(n, V, ldv, nv, x, w, partials, blockIdx.x, gridDim.x, gv);
+    mdot2_body<CH, true>(n, V, ldv, nv, x, w, partials, blockIdx.x, gridDim.x, gv);
 }
 
 // Index of the entry whose block range [first[e], first[e + 1]) holds block b (count entries).
@@ -334,7 +340,7 @@ __global__ void __launch_bounds__(NT, 6) k_mdot2_pair_b(const BVec *__restrict__
     if (*P.active == 0) return;
     const float4 *V = P.V;
     const float4 *x = V + (size_t)j * P.n;
-    mdot2_body<CH>(P.n, V, P.n, j + 1, x, close ? x : x + P.n, P.partials, (int)(blockIdx.x - first[e]),
+    mdot2_body<CH, false>(P.n, V, P.n, j + 1, x, close ? x : x + P.n, P.partials, (int)(blockIdx.x - first[e]),
                    (int)(first[e + 1] - first[e]));
 }
 
