@@ -419,9 +419,10 @@ int blas_nblocks(size_t n);
 int mdot_nblocks(size_t n, int nv);
 cudaError_t launch_mdot_norm(size_t n, const double2 *V, size_t ldv, int nv, const double2 *w, double2 *partials,
                              const int *gate, cudaStream_t s);
-// w -= sum_i V_i h_i, then partials[b] = (||w||^2, 0)   (h on device)
+// w -= sum_i V_i h_i, then partials[b] = (||w||^2, 0)   (h on device); wnorm (device, may be null): ||w||
+// before, with which a correction below 2^-36 of it takes the short form
 cudaError_t launch_update_norm(size_t n, const double2 *V, size_t ldv, int nv, const double2 *h, double2 *w,
-                               double2 *partials, const int *gate, cudaStream_t s);
+                               double2 *partials, const int *gate, const double2 *wnorm, cudaStream_t s);
 // out[i] (mode 0: =, 1: +=, 2: (sqrt(re), 0)) = fixed-order sum of partials of vector i; with
 // host_out (pinned host memory), host_out[i] = the real part of out[i] as well; with out2, out2[i] =
 // the plain sum too

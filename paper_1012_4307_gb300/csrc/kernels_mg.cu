@@ -98,9 +98,9 @@ __device__ __forceinline__ typename CT<R>::T apply_point(const OpView<R> &o, con
 // y = M x, or with RES y = b - M x; each thread marches kc planes in 3D with its x and y coefficients
 // in registers.  complex128 is bound by the FP64 units (two lanes per SM and clock): 36 operations per
 // node in 3D, but 16 where every axis is outside the layers, since those coefficients of A are real.
-// Each warp picks the form by axis (x: all its columns, y: its row, z: all its planes), once, so that
-// every form is a loop of its own.  Measured, A x in complex128 on 225 x 193 x 161 nodes: 406 us with
-// every term complex, 321 us so (543 us with the form chosen by a branch at every node).
+// Each warp picks the form by axis (x: all its columns, y: its row, z: runs of its planes), outside the
+// loop, so that every form is a loop of its own.  Measured, A x in complex128 on 225 x 193 x 161 nodes: 406 us with
+// every term complex, 318 us so (543 us with the form chosen by a branch at every node).
 template <typename R, int DIM, typename CX, typename CB, bool RES, bool RX, bool RY, bool RZ>
 __device__ __forceinline__ void apply_march(const OpView<R> &o, const CB *__restrict__ b, const CX *__restrict__ x,
                                             typename CT<R>::T *__restrict__ y, int i, int j, int k0, int k1) {
@@ -154,13 +154,27 @@ __global__ void __launch_bounds__(BX *BY) k_apply(OpView<R> o, const CB *__restr
         };
         if (is_zero(o.bk.y) && is_zero(o.c.y)) {
             const bool rx = __all_sync(__activemask(), real3(o.cx + 3 * i)), ry = real3(o.cy + 3 * j);
-            bool rz = true;
-            if (DIM == 3)
-                for (int k = k0; k < k1; k++) rz = rz && real3(o.cz + 3 * k);
-            if (rx && ry && rz) return apply_march<R, DIM, CX, CB, RES, true, true, true>(o, b, x, y, i, j, k0, k1);
-            if (rx && ry) return apply_march<R, DIM, CX, CB, RES, true, true, false>(o, b, x, y, i, j, k0, k1);
-            if (rx && rz) return apply_march<R, DIM, CX, CB, RES, true, false, true>(o, b, x, y, i, j, k0, k1);
-            if (ry && rz) return apply_march<R, DIM, CX, CB, RES, false, true, true>(o, b, x, y, i, j, k0, k1);
+            if constexpr (DIM == 2) {
+                if (rx && ry) return apply_march<R, DIM, CX, CB, RES, true, true, true>(o, b, x, y, i, j, 0, 1);
+                if (rx) return apply_march<R, DIM, CX, CB, RES, true, false, true>(o, b, x, y, i, j, 0, 1);
+                if (ry) return apply_march<R, DIM, CX, CB, RES, false, true, true>(o, b, x, y, i, j, 0, 1);
+            } else {
+                // runs of planes that are all real or all not
+                for (int k = k0, e; k < k1; k = e) {
+                    const bool rz = real3(o.cz + 3 * k);
+                    e = k + 1;
+                    while (e < k1 && real3(o.cz + 3 * e) == rz) e++;
+                    if (rx && ry && rz) apply_march<R, DIM, CX, CB, RES, true, true, true>(o, b, x, y, i, j, k, e);
+                    else if (rx && ry) apply_march<R, DIM, CX, CB, RES, true, true, false>(o, b, x, y, i, j, k, e);
+                    else if (rx && rz) apply_march<R, DIM, CX, CB, RES, true, false, true>(o, b, x, y, i, j, k, e);
+                    else if (ry && rz) apply_march<R, DIM, CX, CB, RES, false, true, true>(o, b, x, y, i, j, k, e);
+                    else if (rx) apply_march<R, DIM, CX, CB, RES, true, false, false>(o, b, x, y, i, j, k, e);
+                    else if (ry) apply_march<R, DIM, CX, CB, RES, false, true, false>(o, b, x, y, i, j, k, e);
+                    else if (rz) apply_march<R, DIM, CX, CB, RES, false, false, true>(o, b, x, y, i, j, k, e);
+                    else apply_march<R, DIM, CX, CB, RES, false, false, false>(o, b, x, y, i, j, k, e);
+                }
+                return;
+            }
         }
     }
     apply_march<R, DIM, CX, CB, RES, false, false, false>(o, b, x, y, i, j, k0, k1);

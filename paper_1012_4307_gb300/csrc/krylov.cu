@@ -290,9 +290,9 @@ static cudaError_t fgmres_step(helm_handle *h, int j, int m) {
         return df ? launch_mdot_norm_pair(np, V4, np, nv, (const float4 *)w, h->partials, gate, s)
                   : launch_mdot_norm(np, h->V, np, nv, w, h->partials, gate, s);
     };
-    auto gs_update = [&](int nv, const double2 *hh, double2 *w, const int *gate) {
+    auto gs_update = [&](int nv, const double2 *hh, double2 *w, const int *gate, const double2 *wnorm) {
         return df ? launch_update_norm_pair(np, V4, np, nv, hh, (float4 *)w, h->partials, gate, s)
-                  : launch_update_norm(np, h->V, np, nv, hh, w, h->partials, gate, s);
+                  : launch_update_norm(np, h->V, np, nv, hh, w, h->partials, gate, wnorm, s);
     };
     double2 *vj = h->V + (size_t)j * np, *w = h->V + (size_t)(j + 1) * np;
     void *zj = (char *)h->Z + (size_t)j * np * zsz;
@@ -318,7 +318,7 @@ static cudaError_t fgmres_step(helm_handle *h, int j, int m) {
     {
         pdl_cycle_scope pdl;  // placed while the reduction's few blocks finish
         ProfScope ps(h, HELM_K_UPDATE_NORM, np * 16.0 * (nv + 2), df ? 0.0 : np * (8.0 * nv + 4.0));
-        CKE(gs_update(j + 1, hcol, w, nullptr));
+        CKE(gs_update(j + 1, hcol, w, nullptr, nullptr));
     }
     {
         ProfScope ps(h, HELM_K_SMALL, 0, 0);
@@ -345,7 +345,7 @@ static cudaError_t fgmres_step(helm_handle *h, int j, int m) {
     {
         pdl_cycle_scope pdl;
         ProfScope ps(h, HELM_K_UPDATE_NORM, pass2 * np * 16.0 * (nv + 2), df ? 0.0 : pass2 * np * (8.0 * nv + 4.0));
-        CKE(gs_update(j + 1, h->h2, w, h->gs_flag));
+        CKE(gs_update(j + 1, h->h2, w, h->gs_flag, hcol + j + 1));
     }
     {
         ProfScope ps(h, HELM_K_SMALL, 0, 0);
