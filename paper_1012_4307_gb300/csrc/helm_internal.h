@@ -425,7 +425,7 @@ cudaError_t launch_update_norm(size_t n, const double2 *V, size_t ldv, int nv, c
                                double2 *partials, const int *gate, const double2 *wnorm, cudaStream_t s);
 // out[i] (mode 0: =, 1: +=, 2: (sqrt(re), 0)) = fixed-order sum of partials of vector i; with
 // host_out (pinned host memory), host_out[i] = the real part of out[i] as well; with out2, out2[i] =
-// the plain sum too
+// the plain sum (mode 2: its root) too
 cudaError_t launch_reduce(const double2 *partials, int nblk, int nv, double2 *out, int mode, const int *gate,
                           cudaStream_t s, double *host_out = nullptr, double2 *out2 = nullptr);
 // Same two passes in double-FP32 arithmetic on float-pair vectors (kernels_gs_df.cu): node q
@@ -470,9 +470,9 @@ cudaError_t launch_split_scale(size_t n, void *x, const double2 *beta, cudaStrea
 // float pairs / alpha->x -> complex64 / complex128 (alpha null: no scaling)
 cudaError_t launch_pair_to_c64(size_t n, const float4 *v, const double2 *alpha, float2 *z, cudaStream_t s);
 cudaError_t launch_pair_to_c128(size_t n, const float4 *v, const double2 *alpha, double2 *z, cudaStream_t s);
-// *hnorm: ||w||^2 in, ||w'|| out; *flag = (||w'|| < eta ||w||); *count += flag
+// *hnorm: ||w||^2 in, ||w'|| out; *norm = ||w'||; *flag = (||w'|| < eta ||w||); *count += flag
 cudaError_t launch_reduce_decide(const double2 *partials, int nblk, double2 *hnorm, int *flag, int *count, double eta,
-                                 cudaStream_t s);
+                                 double2 *norm, cudaStream_t s);
 // y = x * (1 / scale[0].x); with b_out, b_out = y rounded to complex64 as well
 cudaError_t launch_scale_inv(size_t n, const double2 *x, const double2 *scale, double2 *y, float2 *b_out,
                              cudaStream_t s);

@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(NT) k_update_norm(size_t n, const double2 *__r
 }
 
 // out[i] = sum_b partials[i * nblk + b] in a fixed order for i = blockIdx.x; mode 0 '=',
-// 1 '+=', 2 (sqrt(re), 0).  With out2, out2[i] = the plain sum as well.  Gated.
+// 1 '+=', 2 (sqrt(re), 0).  With out2, out2[i] = the plain sum (mode 2: its root) as well.  Gated.
 __global__ void k_reduce(const double2 *__restrict__ partials, int nblk, double2 *__restrict__ out, int mode,
                          const int *__restrict__ gate, double *host_out, double2 *__restrict__ out2) {
     pdl_enter();
@@ -227,16 +227,16 @@ __global__ void k_reduce(const double2 *__restrict__ partials, int nblk, double2
         else if (mode == 1) r = cadd(out[i], t);
         else r = make_double2(sqrt(t.x), 0.0);
         out[i] = r;
-        if (out2) out2[i] = t;
+        if (out2) out2[i] = mode == 2 ? r : t;
         if (host_out) host_out[i] = r.x;
     }
 }
 
 // DGKS test after one classical Gram-Schmidt pass: the new norm ||w'|| = sqrt(sum partials)
-// is written to *hnorm (which held ||w||^2 before the pass); re-orthogonalise (*flag = 1) when
+// is written to *hnorm (which held ||w||^2 before the pass) and to *norm; re-orthogonalise (*flag = 1) when
 // ||w'|| < eta ||w||, i.e. when the projection cancelled most of w.
 __global__ void k_reduce_decide(const double2 *__restrict__ partials, int nblk, double2 *hnorm, int *flag, int *count,
-                                double eta) {
+                                double eta, double2 *norm) {
     pdl_enter();
     __shared__ double2 sums[1];
     double2 s[1] = {make_double2(0.0, 0.0)};
@@ -248,6 +248,7 @@ __global__ void k_reduce_decide(const double2 *__restrict__ partials, int nblk, 
         *flag = redo;
         if (redo) *count += 1;
         *hnorm = make_double2(after, 0.0);
+        *norm = make_double2(after, 0.0);
     }
 }
 
@@ -755,8 +756,8 @@ cudaError_t launch_reduce(const double2 *partials, int nblk, int nv, double2 *ou
 }
 
 cudaError_t launch_reduce_decide(const double2 *partials, int nblk, double2 *hnorm, int *flag, int *count, double eta,
-                                 cudaStream_t s) {
-    launch_pdl(k_reduce_decide, 1, NT, 0, s, partials, nblk, hnorm, flag, count, eta);
+                                 double2 *norm, cudaStream_t s) {
+    launch_pdl(k_reduce_decide, 1, NT, 0, s, partials, nblk, hnorm, flag, count, eta, norm);
     return cudaGetLastError();
 }
 

@@ -322,7 +322,7 @@ static cudaError_t fgmres_step(helm_handle *h, int j, int m) {
     }
     {
         ProfScope ps(h, HELM_K_SMALL, 0, 0);
-        CKE(launch_reduce_decide(h->partials, ublk, hcol + j + 1, h->gs_flag, h->gs_count, kDGKSEta, s));
+        CKE(launch_reduce_decide(h->partials, ublk, hcol + j + 1, h->gs_flag, h->gs_count, kDGKSEta, h->scal + 20, s));
     }
     // Under launch timing (eager steps, never captured) the host reads the decision, so that
     // the gated pass's bytes are attributed exactly when it runs.
@@ -349,17 +349,28 @@ static cudaError_t fgmres_step(helm_handle *h, int j, int m) {
     }
     {
         ProfScope ps(h, HELM_K_SMALL, 0, 0);
-        CKE(launch_reduce(h->partials, ublk, 1, hcol + j + 1, 2, h->gs_flag, s));
+        CKE(launch_reduce(h->partials, ublk, 1, hcol + j + 1, 2, h->gs_flag, s, nullptr, h->scal + 20));
     }
-    {
-        ProfScope ps(h, HELM_K_VECTOR, np * 32.0, df ? 0.0 : np * 2.0);
-        if (df) CKE(launch_scale_inv_pair(np, (float4 *)w, hcol + j + 1, s));
-        else CKE(launch_scale_inv(np, w, hcol + j + 1, w, fp64_fold(h) ? level0_rhs_c64(h) : nullptr, s));
+    // the rotation of column j on the side stream beside the normalisation (inline while timing
+    // launches): it is one warp's serial FP64 chain
+    const bool fork = !h->prof.on;
+    if (fork) {
+        CKE(cudaEventRecord(h->ev_fork, s));
+        CKE(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
     }
     {
         ProfScope ps(h, HELM_K_SMALL, 0, 0);
-        CKE(launch_givens(h->H, ldh, j, h->cs, h->sn, h->g, h->fnorm_dev, h->est_dev, h->est_host, nullptr, nullptr, s));
+        CKE(launch_givens(h->H, ldh, j, h->cs, h->sn, h->g, h->fnorm_dev, h->est_dev, h->est_host, nullptr, nullptr,
+                          fork ? h->side : s));
     }
+    if (fork) CKE(cudaEventRecord(h->ev_join, h->side));
+    {
+        ProfScope ps(h, HELM_K_VECTOR, np * 32.0, df ? 0.0 : np * 2.0);
+        const double2 *norm = h->scal + 20;  // ||w||, kept for this pass: the rotation replaces it in H
+        if (df) CKE(launch_scale_inv_pair(np, (float4 *)w, norm, s));
+        else CKE(launch_scale_inv(np, w, norm, w, fp64_fold(h) ? level0_rhs_c64(h) : nullptr, s));
+    }
+    if (fork) CKE(cudaStreamWaitEvent(s, h->ev_join, 0));
     // inside a capture the record must become an event node of the graph (external), so that
     // the host can wait on the event after every replay
     return h->capturing ? cudaEventRecordWithFlags(h->step_ev[j], s, cudaEventRecordExternal)
