@@ -222,7 +222,8 @@ __global__ void __launch_bounds__(BX *BY) k_jacobi(OpView<R> o, R omega, const C
 // 3D omega-Jacobi: k_jacobi's arithmetic in the same order, with the x and y coefficient
 // triples loaded once per thread, the (z - 1, z, z + 1) column in registers, and the next plane's
 // operands (four in-plane neighbours, z + 2, b, k^2) loaded while this plane is computed.
-// KC: fine planes per thread (shorter chunks on small grids give more blocks).  ZERO with a complex128 b
+// KC: fine planes per thread (shorter chunks on small grids give more blocks; 16 against 8 on 257^3: 695
+// against 700 us per cycle).  ZERO with a complex128 b
 // in a complex64 cycle: the sweep also writes b rounded to complex64 to b_out.
 template <typename R, typename CB, bool ZERO, int KC>
 __global__ void __launch_bounds__(BX *BY) k_jacobi3(OpView<R> o, R omega, const CB *__restrict__ b,
@@ -697,6 +698,7 @@ __global__ void __launch_bounds__(BX *BY) k_prolong3(int nx, int ny, int nz, con
         C sn = sb, un = uq;
         if (k + 1 < k1) {
             un = uf[p + (size_t)nx * ny];
+            if (k + 3 < k1 && (threadIdx.x & 15) == 0) l2_prefetch(&uf[p + 3 * (size_t)nx * ny]);
             if (((k + 2) >> 1) != ((k + 1) >> 1)) sn = corner_sum((k + 2) >> 1);
         }
         uf[p] = cadd(uq, cscale(cadd(sa, sb), R(0.125)));
@@ -765,6 +767,7 @@ constexpr int tile_threads(int n) { return ((n + (n + 511) / 512 - 1) / ((n + 51
 template <int TCX, int TCY> struct Tile {
     static constexpr int RW = 2 * TCX + 5, RH = 2 * TCY + 5;  // R3 extent
     static constexpr int NT = tile_threads(RW * RH);           // threads per block
+    static constexpr int NP = (RW * RH + NT - 1) / NT;          // passes of a phase
     struct Coef {
         float2 x[RW][3], y[RH][3];
     };
@@ -783,6 +786,26 @@ template <int TCX, int TCY> struct Tile {
         float2 u4[RH][RW];
     };
 };
+
+// 1 / D at the region nodes of this thread, node k of for_region_k in dv[k] (0 off the interior).
+template <int RW, int RH, int ST, int NP>
+__device__ __forceinline__ void tile_dinv(const OpView<float> &o, int X0, int Y0, float2 (&dv)[NP]) {
+#pragma unroll
+    for (int k = 0; k < NP; k++) {
+        const int q = threadIdx.x + ST * k, sy = q / RW, x = X0 + q - sy * RW, y = Y0 + sy;
+        dv[k] = (q < RW * RH && x >= 1 && x <= o.nx - 2 && y >= 1 && y <= o.ny - 2) ? __ldg(&o.dinv[(size_t)x + (size_t)o.nx * y])
+                                                                                : make_float2(0.f, 0.f);
+    }
+}
+// f(sx, sy, k) for every node of an RW x RH region, ST threads, node q = tid + ST k in row-major order.
+template <int RW, int RH, int ST, int NP, typename F>
+__device__ __forceinline__ void for_region_k(F f) {
+#pragma unroll
+    for (int k = 0; k < NP; k++) {
+        const int q = threadIdx.x + ST * k, sy = q / RW;
+        if (q < RW * RH) f(q - sy * RW, sy, k);
+    }
+}
 
 // Loads the operator's coefficient triples of the region's columns and rows.
 template <int RW, int RH, typename TC>
@@ -854,7 +877,11 @@ __device__ __forceinline__ float2 tile_diag(const TC &tc, int sx, int sy, float 
 // interior skip the per-node boundary tests.
 // (bx, by): the tile of coarse nodes this block owns.
 // CB double2: b is a complex128 vector; its owned nodes rounded to complex64 go to b_out too.
-template <int TCX, int TCY, typename CB>
+// EARLY: the caller has not yet waited for the kernel before it in the stream: the operator's data
+// (coefficients and 1 / D, which no kernel writes) is loaded before the wait (1025^2 complex64 cycle, eager:
+// 74.3 -> 69.4 us; its FGMRES solve in replayed graphs 21.05 -> 20.84 ms).  The batched kernels fill the
+// chip and keep the plain order.
+template <int TCX, int TCY, bool EARLY, typename CB>
 __device__ __forceinline__ void pre2_restrict_tile(const OpView<float> &o, float omega, const CB *__restrict__ b,
                                                    float2 *__restrict__ u, float2 *__restrict__ rc, int ncx, int ncy,
                                                    int bx, int by, const int *gate = nullptr,
@@ -863,7 +890,6 @@ __device__ __forceinline__ void pre2_restrict_tile(const OpView<float> &o, float
     constexpr int RW = TL::RW, RH = TL::RH;
     extern __shared__ __align__(16) unsigned char pre_smem[];
     __shared__ int gate_s;  // the gate flag, published by the first block barrier
-    if (threadIdx.x == 0) gate_s = gate_value(gate);
     typename TL::Pre &T = *reinterpret_cast<typename TL::Pre *>(pre_smem);
     const int I0 = 1 + bx * TCX, J0 = 1 + by * TCY;
     const int X0 = 2 * I0 - 3, Y0 = 2 * J0 - 3;
@@ -873,18 +899,24 @@ __device__ __forceinline__ void pre2_restrict_tile(const OpView<float> &o, float
     // the coefficients are first used by the second sweep: one barrier publishes them with b,
     // 1 / D and the first sweep
     tile_coef<RW, RH>(o, X0, Y0, T.tc);
-    // load b and 1 / D; sweep 1 from zero (pointwise): u1 = omega b / D
-    for_region<RW, RH, TL::NT>([&](int sx, int sy) {
+    float2 dv[TL::NP];
+    if (EARLY) {
+        tile_dinv<RW, RH, TL::NT>(o, X0, Y0, dv);
+        pdl_enter();
+    }
+    if (threadIdx.x == 0) gate_s = gate_value(gate);
+    // load b; sweep 1 from zero (pointwise): u1 = omega b / D
+    for_region_k<RW, RH, TL::NT, TL::NP>([&](int sx, int sy, int k) {
         const int x = X0 + sx, y = Y0 + sy;
-        float2 bv = make_float2(0.f, 0.f), dv = make_float2(0.f, 0.f);
+        float2 bv = make_float2(0.f, 0.f), di = EARLY ? dv[k] : make_float2(0.f, 0.f);
         if (inside(x, y)) {
             const size_t p = (size_t)x + (size_t)nx * y;
             bv = to_c(b[p], 0.f);
-            dv = o.dinv[p];
+            if (!EARLY) di = o.dinv[p];
         }
         T.b[sy][sx] = bv;
-        T.di[sy][sx] = dv;
-        T.u1[sy][sx] = cscale(cmul(bv, dv), omega);
+        T.di[sy][sx] = di;
+        T.u1[sy][sx] = cscale(cmul(bv, di), omega);
     });
     __syncthreads();
     if (gate_s) return;
@@ -930,15 +962,14 @@ template <int TCX, int TCY, typename CB>
 __global__ void __launch_bounds__(Tile<TCX, TCY>::NT, 4) k_pre2_restrict(OpView<float> o, float omega, const CB *__restrict__ b,
                                                        float2 *__restrict__ u, float2 *__restrict__ rc, int ncx,
                                                        int ncy, float2 *__restrict__ b_out) {
-    pdl_enter();
-    pre2_restrict_tile<TCX, TCY>(o, omega, b, u, rc, ncx, ncy, blockIdx.x, blockIdx.y, o.gate, b_out);
+    pre2_restrict_tile<TCX, TCY, true>(o, omega, b, u, rc, ncx, ncy, blockIdx.x, blockIdx.y, o.gate, b_out);
 }
 
 // u_out <- two omega-Jacobi sweeps of (u_in + P ec), on the owned fine nodes.  u_in and u_out
 // are different arrays: blocks read their halo of u_in while other blocks write u_out.
 // Bilinear interpolation in closed form: P ec at fine node (x, y) is the mean of the four
 // coarse values at (floor/ceil(x/2), floor/ceil(y/2)), coincident ones repeated.
-template <int TCX, int TCY>
+template <int TCX, int TCY, bool EARLY>
 __device__ __forceinline__ void prolong_post2_tile(const OpView<float> &o, float omega, const float2 *__restrict__ b,
                                                    const float2 *__restrict__ u_in, float2 *__restrict__ u,
                                                    const float2 *__restrict__ ec, int ncx, int ncy, int bx, int by,
@@ -947,7 +978,6 @@ __device__ __forceinline__ void prolong_post2_tile(const OpView<float> &o, float
     constexpr int RW = TL::RW, RH = TL::RH;
     extern __shared__ __align__(16) unsigned char post_smem[];
     __shared__ int gate_s;  // the gate flag, published by the first block barrier
-    if (threadIdx.x == 0) gate_s = gate_value(gate);
     typename TL::Post &T = *reinterpret_cast<typename TL::Post *>(post_smem);
     const int I0 = 1 + bx * TCX, J0 = 1 + by * TCY;
     const int X0 = 2 * I0 - 3, Y0 = 2 * J0 - 3;
@@ -958,22 +988,27 @@ __device__ __forceinline__ void prolong_post2_tile(const OpView<float> &o, float
     // 1 / D and u + P ec, whose coarse values each node reads itself (the four corner nodes
     // floor/ceil(x / 2), floor/ceil(y / 2) of an interior fine node lie in the coarse grid)
     tile_coef<RW, RH>(o, X0, Y0, T.tc);
+    float2 dv[TL::NP];
+    if (EARLY) {
+        tile_dinv<RW, RH, TL::NT>(o, X0, Y0, dv);
+        pdl_enter();
+    }
+    if (threadIdx.x == 0) gate_s = gate_value(gate);
     // u3 = u + P ec on the region
-    for_region<RW, RH, TL::NT>([&](int sx, int sy) {
+    for_region_k<RW, RH, TL::NT, TL::NP>([&](int sx, int sy, int k) {
         const int x = X0 + sx, y = Y0 + sy;
-        float2 bv = make_float2(0.f, 0.f), v = make_float2(0.f, 0.f);
-        float2 dv = make_float2(0.f, 0.f);
+        float2 bv = make_float2(0.f, 0.f), v = make_float2(0.f, 0.f), di = EARLY ? dv[k] : make_float2(0.f, 0.f);
         if (inside(x, y)) {
             const size_t p = (size_t)x + (size_t)nx * y;
             bv = b[p];
-            dv = o.dinv[p];
+            if (!EARLY) di = o.dinv[p];
             const size_t ya = (size_t)ncx * (y >> 1), yb = (size_t)ncx * ((y + 1) >> 1);
             const int xa = x >> 1, xb = (x + 1) >> 1;
             const float2 e = cadd(cadd(ec[ya + xa], ec[ya + xb]), cadd(ec[yb + xa], ec[yb + xb]));
             v = cadd(u_in[p], cscale(e, 0.25f));
         }
         T.b[sy][sx] = bv;
-        T.di[sy][sx] = dv;
+        T.di[sy][sx] = di;
         T.u3[sy][sx] = v;
     });
     __syncthreads();
@@ -998,8 +1033,7 @@ template <int TCX, int TCY>
 __global__ void __launch_bounds__(Tile<TCX, TCY>::NT, 4) k_prolong_post2(OpView<float> o, float omega, const float2 *__restrict__ b,
                                                        const float2 *__restrict__ u_in, float2 *__restrict__ u,
                                                        const float2 *__restrict__ ec, int ncx, int ncy) {
-    pdl_enter();
-    prolong_post2_tile<TCX, TCY>(o, omega, b, u_in, u, ec, ncx, ncy, blockIdx.x, blockIdx.y, o.gate);
+    prolong_post2_tile<TCX, TCY, true>(o, omega, b, u_in, u, ec, ncx, ncy, blockIdx.x, blockIdx.y, o.gate);
 }
 
 // Batched forms (many problems, one launch): blockIdx.z picks the table entry, whose level has
@@ -1010,7 +1044,7 @@ __global__ void __launch_bounds__(Tile<TCX, TCY>::NT, 4) k_pre2_restrict_b(const
     const BLevel &E = tab[blockIdx.z];
     if (*E.active == 0) return;
     const OpView<float> o = view(E.op);
-    pre2_restrict_tile<TCX, TCY>(o, omega, E.b, E.t, E.coarse, (o.nx + 1) / 2, (o.ny + 1) / 2, blockIdx.x, blockIdx.y);
+    pre2_restrict_tile<TCX, TCY, false>(o, omega, E.b, E.t, E.coarse, (o.nx + 1) / 2, (o.ny + 1) / 2, blockIdx.x, blockIdx.y);
 }
 
 template <int TCX, int TCY>
@@ -1019,7 +1053,7 @@ __global__ void __launch_bounds__(Tile<TCX, TCY>::NT, 4) k_prolong_post2_b(const
     const BLevel &E = tab[blockIdx.z];
     if (*E.active == 0) return;
     const OpView<float> o = view(E.op);
-    prolong_post2_tile<TCX, TCY>(o, omega, E.b, E.t, E.u + (size_t)j * E.ustride, E.coarse, (o.nx + 1) / 2,
+    prolong_post2_tile<TCX, TCY, false>(o, omega, E.b, E.t, E.u + (size_t)j * E.ustride, E.coarse, (o.nx + 1) / 2,
                                  (o.ny + 1) / 2, blockIdx.x, blockIdx.y);
 }
 
@@ -1066,12 +1100,13 @@ cudaError_t launch_jacobi(const DevOp<R> &op, int dim, R omega, const CB *bb, co
                           typename CT<R>::T *u_out, cudaStream_t s) {
     dim3 g = grid_for(op.n, dim), b(BX, BY);
     if (dim == 3) {
-        const int kc = z_chunk((size_t)g.x * g.y, op.n[2] - 2, KCHUNK, 152 * 10);
+        const int kc = z_chunk((size_t)g.x * g.y, op.n[2] - 2, 2 * KCHUNK, 152 * 10);
         g.z = cdiv(op.n[2] - 2, kc);
         typename CT<R>::T *none = nullptr;
         auto go = [&](auto kernel) { return launch_pdl(kernel, g, b, 0, s, view(op), omega, bb, u_in, u_out, none); };
         if (u_in == nullptr) {
             switch (kc) {
+            case 16: go(k_jacobi3<R, CB, true, 16>); break;
             case 8: go(k_jacobi3<R, CB, true, 8>); break;
             case 4: go(k_jacobi3<R, CB, true, 4>); break;
             case 2: go(k_jacobi3<R, CB, true, 2>); break;
@@ -1079,6 +1114,7 @@ cudaError_t launch_jacobi(const DevOp<R> &op, int dim, R omega, const CB *bb, co
             }
         } else {
             switch (kc) {
+            case 16: go(k_jacobi3<R, CB, false, 16>); break;
             case 8: go(k_jacobi3<R, CB, false, 8>); break;
             case 4: go(k_jacobi3<R, CB, false, 4>); break;
             case 2: go(k_jacobi3<R, CB, false, 2>); break;

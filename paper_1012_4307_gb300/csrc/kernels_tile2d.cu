@@ -22,7 +22,8 @@
 // the code is the same for every tile.
 // Measured on GB300: 641^2 complex128 F cycle with one sweep each way 755 -> 599 us, Bi-CGSTAB on 385^2
 // (two such cycles an iteration) 57.5 -> 42.0 ms; with the residual after one sweep from zero formed
-// without the diagonal and real coefficients taken as real (block-uniform), 599 -> 538 us.
+// without the diagonal and real coefficients taken as real (block-uniform), 599 -> 538 us; with the
+// coefficients staged before the wait for the kernel ahead, 525 -> 511 us.
 #include <algorithm>
 
 #include "helm_internal.h"
@@ -206,15 +207,15 @@ template <typename R, bool RB, bool REAL> __device__ __forceinline__ void tile_p
 
 template <typename R, bool RB>
 __global__ void __launch_bounds__(512) k_tile_pre(const __grid_constant__ T2<R> A) {
-    pdl_enter();
-    if (A.gate && *A.gate) return;
     extern __shared__ __align__(16) unsigned char t2_smem[];
     const int I0 = 1 + blockIdx.x * A.tcx, J0 = 1 + blockIdx.y * A.tcy;
     // residuals of the coarse nodes' neighbourhoods: owned fine nodes and one more row and column
     const Range res{2 * I0 - 1, 2 * I0 + 2 * A.tcx - 1, 2 * J0 - 1, 2 * J0 + 2 * A.tcy - 1};
     const int e = 1 + A.s;
     Region<R> G = region<R>(A, t2_smem, res.x0 - e, res.y0 - e, 2 * A.tcx + 1 + 2 * e, 2 * A.tcy + 1 + 2 * e);
-    G.stage();
+    G.stage();  // coefficients only, which no kernel writes: before the wait for the kernel ahead
+    pdl_enter();
+    if (A.gate && *A.gate) return;
     if constexpr (sizeof(R) == sizeof(double)) {
         if (G.real) {
             tile_pre<R, RB, true>(A, G, res);
@@ -268,14 +269,14 @@ template <typename R, bool RB, bool REAL> __device__ __forceinline__ void tile_p
 
 template <typename R, bool RB>
 __global__ void __launch_bounds__(512) k_tile_post(const __grid_constant__ T2<R> A) {
-    pdl_enter();
-    if (A.gate && *A.gate) return;
     extern __shared__ __align__(16) unsigned char t2_smem[];
     const int I0 = 1 + blockIdx.x * A.tcx, J0 = 1 + blockIdx.y * A.tcy;
     const Range own{2 * I0 - 1, 2 * I0 + 2 * A.tcx - 2, 2 * J0 - 1, 2 * J0 + 2 * A.tcy - 2};
     const int e = A.s;
     Region<R> G = region<R>(A, t2_smem, own.x0 - e, own.y0 - e, 2 * A.tcx + 2 * e, 2 * A.tcy + 2 * e);
-    G.stage();
+    G.stage();  // coefficients only, which no kernel writes: before the wait for the kernel ahead
+    pdl_enter();
+    if (A.gate && *A.gate) return;
     if constexpr (sizeof(R) == sizeof(double)) {
         if (G.real) {
             tile_post<R, RB, true>(A, G, own);
