@@ -459,8 +459,6 @@ cudaError_t launch_mdot2_pair(size_t n, const float4 *V, size_t ldv, int nv, con
 cudaError_t launch_reduce_dcgs2(const double2 *partials, int nblk, double2 *hv, unsigned *ticket, int j,
                                 const double2 *alpha2, double2 *H, int ldh, double2 *coef, int has_w,
                                 cudaStream_t s);
-cudaError_t launch_dcgs2_coef(int j, int has_w, const double2 *hv, const double2 *alpha2, double2 *H, int ldh,
-                              double2 *coef, cudaStream_t s);
 cudaError_t launch_update2_pair(size_t n, float4 *V, size_t ldv, int j, const double2 *coef, double2 *partials,
                                 unsigned *ticket, double2 *alpha_out, float2 *b_out, const int *gate, cudaStream_t s);
 // w <- w / beta->x (float pairs)

@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(NT, 6) k_mdot2_pair_b(const BVec *__restrict__
                    (int)(first[e + 1] - first[e]));
 }
 
-// One pass of the DCGS2 update for step j with coefficients coef (see k_dcgs2_coef):
+// One pass of the DCGS2 update for step j with coefficients coef (see dcgs2_coef_warps):
 //   x <- (x - sum_{i<j} V_i A_i) r             (x = basis slot j: its final vector v_j)
 //   w <- w rw - x_old s - sum_{i<j} V_i C_i    (w = slot j + 1: once orthogonalised, not
 //                                                normalised)
@@ -500,7 +500,7 @@ __device__ __forceinline__ void update2_body(size_t n, float4 *__restrict__ V, s
     block_sum_ff<1>(vals, sums);
     if (threadIdx.x == 0) partials[bx] = make_double2(sums[0], 0.0);
     if (!ticket || !last_block(ticket, nblk)) return;
-    reduce_partials_block(partials, nblk, 1, alpha_out, true);
+    reduce_norm_block<NT>(partials, nblk, alpha_out);
     if (threadIdx.x == 0) *ticket = 0u;
 }
 

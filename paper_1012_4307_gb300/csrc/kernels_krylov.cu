@@ -435,20 +435,33 @@ __global__ void k_givens_b(const BVec *__restrict__ tab, int j, double *out, con
     }
 }
 
-// The reduction of the two-vector inner-product pass (block v sums value v of the partials in
-// the fixed order of k_reduce) followed, in the last block to finish, by the DCGS2 coefficient
+// The reduction of the two-vector inner-product pass (block v sums value v of the partials in a
+// fixed tree) followed, in the last block to finish, by the DCGS2 coefficient
 // step of step j (see dcgs2_coef.cuh); the ticket returns to 0.
 __device__ __forceinline__ void reduce_dcgs2_body(const double2 *__restrict__ partials, int nblk, double2 *hv,
                                                   unsigned *ticket, int j, const double2 *alpha2, double2 *H, int ldh,
                                                   double2 *coef, int has_w) {
-    __shared__ double2 sums[1];
-    const int i = blockIdx.x;
-    double2 acc[1] = {make_double2(0.0, 0.0)};
-    for (int b = threadIdx.x; b < nblk; b += NT) acc[0] = cadd(acc[0], partials[(size_t)i * nblk + b]);
-    block_sum<1>(acc, sums);
-    if (threadIdx.x == 0) hv[i] = sums[0];
+    __shared__ double red[2 * NT / 32];
+    const int i = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double2 *p = partials + (size_t)i * nblk;
+    double v[2] = {0.0, 0.0};
+#pragma unroll 2
+    for (int b = threadIdx.x; b < nblk; b += NT) {
+        v[0] += p[b].x;
+        v[1] += p[b].y;
+    }
+    const int c = warp_transpose_sum<2>(v);
+    if ((lane & 15) == 0) red[2 * warp + c] = v[0];
+    __syncthreads();
+    if (warp == 0) {
+        // lane 2 w + c: component c of warp w
+        static_assert(2 * NT / 32 == 16, "");
+        double s = red[lane & 15];
+        for (int off = 8; off > 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (lane < 2) ((double *)(hv + i))[lane] = s;
+    }
     if (!last_block(ticket, gridDim.x)) return;
-    if (threadIdx.x < 32) dcgs2_coef_warp(j, has_w, hv, alpha2, H, ldh, coef);
+    if (threadIdx.x < 64) dcgs2_coef_warps(j, has_w, hv, alpha2, H, ldh, coef);
     if (threadIdx.x == 0) *ticket = 0u;
 }
 
@@ -467,13 +480,6 @@ __global__ void k_reduce_dcgs2_b(const BVec *__restrict__ tab, const unsigned *_
     if (*P.active == 0) return;
     const int nblk = (int)((first[blockIdx.z + 1] - first[blockIdx.z]) / groups);
     reduce_dcgs2_body(P.partials, nblk, P.hv, P.tickets, j, P.alpha2, P.H, P.ldh, P.dcoef, has_w);
-}
-
-// DCGS2 coefficient step as its own launch (one warp); see dcgs2_coef.cuh.
-__global__ void k_dcgs2_coef(int j, int has_w, const double2 *__restrict__ hv, const double2 *__restrict__ alpha2,
-                             double2 *__restrict__ H, int ldh, double2 *__restrict__ coef) {
-    pdl_enter();
-    dcgs2_coef_warp(j, has_w, hv, alpha2, H, ldh, coef);
 }
 
 // y = R^{-1} g for the k x k upper-triangular leading block R of H (column-major, leading
@@ -817,13 +823,6 @@ cudaError_t launch_reduce_dcgs2_batch(int count, const BVec *tab, const unsigned
 cudaError_t launch_givens_batch(int count, const BVec *tab, int j, double *est_out, const double *tol, cudaStream_t s) {
     if (count < 1 || count > 65535 || j < 0 || j > 63) return cudaErrorInvalidValue;
     launch_pdl(k_givens_b, dim3(1, 1, count), 32, 0, s, tab, j, est_out, tol);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_dcgs2_coef(int j, int has_w, const double2 *hv, const double2 *alpha2, double2 *H, int ldh,
-                              double2 *coef, cudaStream_t s) {
-    if (j < 0 || j > 64) return cudaErrorInvalidValue;
-    launch_pdl(k_dcgs2_coef, 1, 32, 0, s, j, has_w, hv, alpha2, H, ldh, coef);
     return cudaGetLastError();
 }
 
