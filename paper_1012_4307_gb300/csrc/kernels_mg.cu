@@ -176,8 +176,22 @@ __global__ void __launch_bounds__(BX *BY) k_apply(OpView<R> o, const CB *__restr
                 return;
             }
         }
+        apply_march<R, DIM, CX, CB, RES, false, false, false>(o, b, x, y, i, j, k0, k1);
+    } else {
+        // bound by memory: the coefficients come from L1 at every node, which leaves the loads of a
+        // plane more room (257 x 225 x 257 nodes: 70.5 us with the x and y coefficients in registers, 67.6 so)
+        typedef typename CT<R>::T C;
+        const size_t sz = (size_t)o.nx * o.ny;
+        size_t p = (size_t)i + (size_t)o.nx * ((size_t)j + (size_t)o.ny * k0);
+        C xm = mk(R(0), R(0)), xc = to_c(x[p], R()), xp = mk(R(0), R(0)), d;
+        if (DIM == 3) xm = to_c(x[p - sz], R());
+        for (int k = k0; k < k1; k++, p += sz) {
+            if (DIM == 3) xp = to_c(x[p + sz], R());
+            const C v = stencil<R, DIM>(o, x, p, i, j, k, xm, xc, xp, d);
+            y[p] = RES ? csub(to_c(b[p], R()), v) : v;
+            if (DIM == 3) { xm = xc; xc = xp; }
+        }
     }
-    apply_march<R, DIM, CX, CB, RES, false, false, false>(o, b, x, y, i, j, k0, k1);
 }
 
 // omega-Jacobi: every unknown from the previous iterate (ping-pong buffers).
@@ -1065,6 +1079,27 @@ static int z_chunk(size_t tiles_xy, int planes, int kmax, size_t target) {
     return kc;
 }
 
+// Planes per thread of an A x in 3D.  complex64: as above.  complex128 holds 100 registers, two blocks
+// per SM, and is bound by the FP64 units, so what counts is the block-planes of the busiest SM: whole
+// rounds of two blocks, each of kc planes and about 0.8 of one for its coefficients.  Measured, kc = 8 /
+// 4 / 2 / 1: 65 x 57 x 73 nodes - / 19.5 / - / 21.2 us, 81^3 36.2 / - / 37.9 / 44.0, 97^3 61.3 / 50.5 / 53.3 / -,
+// 129 x 97 x 113 80.6 / 73.8 / 78.3 / -, 129^3 111.7 / 108.6 / - / -, 161 x 129 x 161 162 / 165 / - / -, 193 x 161 x 193 276 / 288 / - / -.  (The
+// residual and the red-black sweep keep the shorter chunks: with this rule a red-black cycle on 193 x
+// 129 x 97 nodes took 518 instead of 469 us.)
+template <typename R> static int apply_chunk(size_t tiles_xy, int planes) {
+    if (sizeof(R) == sizeof(float)) return z_chunk(tiles_xy, planes, KCHUNK, 152 * 10);
+    int best = 1;
+    double least = 1e30;
+    for (int kc = KCHUNK; kc >= 1; kc /= 2) {
+        const double cost = (double)cdiv(tiles_xy * cdiv(planes, kc), 2 * 152) * (kc + 0.8);
+        if (cost < least) {
+            least = cost;
+            best = kc;
+        }
+    }
+    return best;
+}
+
 dim3 grid_for(const int n[3], int dim) {
     return dim3(cdiv(n[0] - 2, BX), cdiv(n[1] - 2, BY), dim == 3 ? cdiv(n[2] - 2, KCHUNK) : 1);
 }
@@ -1075,7 +1110,7 @@ dim3 grid_for(const int n[3], int dim) {
 template <typename R, typename CX>
 cudaError_t launch_apply(const DevOp<R> &op, int dim, const CX *x, typename CT<R>::T *y, cudaStream_t s) {
     dim3 g = grid_for(op.n, dim), b(BX, BY);
-    const int kc = dim == 3 ? z_chunk((size_t)g.x * g.y, op.n[2] - 2, KCHUNK, 152 * 10) : 1;
+    const int kc = dim == 3 ? apply_chunk<R>((size_t)g.x * g.y, op.n[2] - 2) : 1;
     if (dim == 3) g.z = cdiv(op.n[2] - 2, kc);
     const CX *none = nullptr;
     if (dim == 3) launch_pdl(k_apply<R, 3, CX, CX, false>, g, b, 0, s, view(op), none, x, y, kc);

@@ -100,3 +100,18 @@ def test_real_coefficients_outside_the_layers(helm, oracle, n, coarsest_n, smoot
     x = W.random_field(tuple(reversed(n)), 52)
     for which, op in (("A", A), ("M", M)):
         assert rel_l2(to_np(helm.helm_apply(h, to_gpu(x), which=which)), op.apply(x)) <= 1e-14
+
+
+@pytest.mark.parametrize("prec", ["c64", "c128"])
+@pytest.mark.parametrize("n", [(33, 17, 25), (65, 57, 73), (81, 73, 81)])
+def test_3d_apply_chunks(helm, oracle, n, prec):
+    """The 3D operator with chunks of one, four and eight planes per thread and a last chunk that is
+    not full.  complex128: 1e-14 as elsewhere; complex64: some 16 roundings of 6e-8 a node."""
+    P = problem(n, 10)
+    h = gpu_handle(helm, P, prec=prec)
+    A, _ = oracle_pair(oracle, P)
+    x = W.random_field(tuple(reversed(n)), 53)
+    v = to_gpu(x)
+    if prec == "c64":
+        v = v.to(torch.complex64)
+    assert rel_l2(to_np(helm.helm_apply(h, v)), A.apply(x)) <= (1e-6 if prec == "c64" else 1e-14)
