@@ -364,9 +364,11 @@ helm_status helm_profile_read(helm_handle *h, int ncls, int *launches, double *m
  *                  HELM_TILE_* (coarse nodes per block, or the register wavefront), or as
  *                  separate sweep / residual /
  *                  transfer launches (HELM_TILE_NONE).  Ignored where it does not apply (other
- *                  smoothers, complex128 cycles, 3D, levels inside the tail, grids the tile
- *                  does not fit: those use the separate launches).
- * Default: tail_levels = -1, HELM_TILE_32x8 on every level, cluster_levels = 0 (16 blocks, cluster_halo 3). */
+ *                  smoothers and complex128 cycles, whose 2D levels have blocked launches of
+ *                  their own; 3D, levels inside the tail, grids the tile does not fit).
+ * Default: tail_levels = -1, HELM_TILE_32x8 on every level, cluster_levels = 0 (16 blocks, cluster_halo 3).
+ * While no tuning was set or measured, a handle of its own (not one of a lockstep batch) runs each
+ * such level with the tile that suits the level's size instead of 32x8; the results are the same. */
 #define HELM_MAX_LEVELS 16
 typedef enum {
     HELM_TILE_NONE = -1,

@@ -1,8 +1,8 @@
 // Cycle tuning: which kernels carry out Algorithm 1 on each level (temporally blocked tiles or
 // separate sweep / residual / transfer launches, and how many coarse levels go into the fused
-// single-block tail or the thread-block-cluster tail), and an autotuner that times the choices
-// on the device.  The arithmetic
-// of the cycle does not depend on the choice (up to FP32 rounding order).
+// tail, on how many blocks and with how many halo rows), and an autotuner that times the choices
+// on the device.  The arithmetic of the cycle does not depend on the choice (up to FP32 rounding
+// order).
 #include <algorithm>
 #include <vector>
 
