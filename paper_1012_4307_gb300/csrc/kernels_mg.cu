@@ -12,6 +12,7 @@
 // keeping the x[p - nx ny], x[p], x[p + nx ny] column in registers.  Every launch covers the
 // interior only, so no thread touches a boundary node's value except as a stencil neighbour.
 #include "helm_internal.h"
+#include "restrict_turns.h"
 
 namespace {
 
@@ -466,11 +467,12 @@ __global__ void __launch_bounds__(BX *BY) k_prolong_add(int nx, int ny, int nz, 
 // own residuals by (1, 2, 1) along z in registers; once per coarse plane the weighted plane goes through
 // shared memory and the coarse nodes' threads apply (1, 2, 1) in x and y.  The four groups of four warps
 // take turns at that sum: a group waits for the plane in its own turn only and merely arrives at the
-// barrier in the others' (four buffers, four barriers), so that the sum does not hold up the march of
-// the other warps.  A buffer is written again four coarse planes later, when every warp has since waited
-// in a turn of its own, behind the group that read it.  (257^3 complex64 finest level: 141 us per launch
+// barrier in the others' (restrict_turns.h), so that the sum does not hold up the march of the other
+// warps.  Five shared planes for the four turns: every warp then waits in a turn of its own between a
+// group's reads of a plane and its own next store into it.  (257^3 complex64 finest level: 141 us per launch
 // with one barrier and the same four warps summing every fine plane, 128 us with the z sums in registers,
-// the cycle 725 -> 700 us with the turns; four lanes per coarse node in every warp instead: 141 us.)  An odd fine plane 2K + 1 completes coarse plane
+// the cycle 725 -> 700 us with the turns; four lanes per coarse node in every warp instead: 141 us.)  An odd
+// fine plane 2K + 1 completes coarse plane
 // K and starts K + 1.  Fine nodes outside the grid's interior hold zero
 // residuals.  Same weights as k_residual_restrict, applied per axis.
 constexpr int R3_TX = 16, R3_TY = 8, R3_KC = 8;
@@ -514,7 +516,7 @@ __global__ void __launch_bounds__(R3_NT, sizeof(R) == sizeof(float) ? 2 : 1)
     }
     if (gv) return;  // the same value in every thread: no barrier is left waiting
     // the coarse node this thread sums in its warp group's turns (warps 0 .. 15)
-    const int group = (t >> 7) & 3, cn = t & 127, cx = cn % R3_TX, cy = cn / R3_TX, I = I0 + cx, J = J0 + cy;
+    const int group = r3_group(t >> 5), cn = t & 127, cx = cn % R3_TX, cy = cn / R3_TX, I = I0 + cx, J = J0 + cy;
     const bool own = t < 512 && I <= ncx - 2 && J <= ncy - 2;
     C acc = zero;  // z sum of this fine column for the current coarse plane
     for (int z = zs; z <= ze; z++, p += sz) {
@@ -552,8 +554,8 @@ __global__ void __launch_bounds__(R3_NT, sizeof(R) == sizeof(float) ? 2 : 1)
         // fine plane 2K + 1 (K = (z - 1) / 2) completes coarse plane K and starts K + 1
         const int K = (z - 1) >> 1;
         if (K >= K0) {
-            const int turn = (K - K0) & 3;
-            C(*buf)[R3_FW] = rbuf[turn];
+            const int turn = r3_turn(K - K0);
+            C(*buf)[R3_FW] = rbuf[r3_plane(K - K0)];
             if (region) buf[ly][lx] = cadd(acc, r);
             if (turn != group) {
                 asm volatile("bar.arrive %0, %1;" ::"r"(1 + turn), "n"(R3_NT) : "memory");
@@ -1215,7 +1217,7 @@ cudaError_t launch_residual_restrict(const DevOp<R> &op, int dim, const CB *bb, 
         return cudaGetLastError();
     }
     if (dim == 3 && (size_t)op.n[0] * op.n[1] < ((size_t)1 << 31)) {  // 32-bit in-plane offsets
-        constexpr size_t smem = r3_smem_bytes<R>(4);
+        constexpr size_t smem = r3_smem_bytes<R>(R3_PLANES);
         static_assert(smem <= 48 * 1024, "");
         dim3 g(cdiv(nc[0] - 2, R3_TX), cdiv(nc[1] - 2, R3_TY), 1);
         const int kc = z_chunk((size_t)g.x * g.y, nc[2] - 2, R3_KC, 152 * 4);
