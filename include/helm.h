@@ -399,8 +399,8 @@ typedef struct {
 /* Sets / reads the handle's tuning (host struct).  Setting drops the handle's captured CUDA
  * graphs (they are re-captured on next use) and, when the tuning selects a cluster tail not
  * used before on this handle, allocates that tail's initial shared-memory image (every
- * block's, at most 3.2 MB; freed by helm_destroy) and fills it with one kernel on the handle's
- * stream.  Errors: HELM_ERR_ARG (null pointers, a tile index out of range, tail_levels < -1 or
+ * block's, at most 3.2 MB; freed by helm_destroy), fills it with one kernel on the handle's
+ * stream and waits for that stream.  Errors: HELM_ERR_ARG (null pointers, a tile index out of range, tail_levels < -1 or
  * == 1, cluster_levels < 0 or == 1, cluster_ctas not 8 or 16). */
 helm_status helm_set_tuning(helm_handle *h, const helm_tuning *t);
 helm_status helm_get_tuning(const helm_handle *h, helm_tuning *t);

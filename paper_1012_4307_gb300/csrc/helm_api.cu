@@ -414,7 +414,7 @@ helm_status helm_create_impl(const helm_grid *grid, double theta, const double *
             for (int k = 0; k < 2; k++)
                 for (int nt = 2; nt <= std::min(nlev, MAX_CT_LEVELS); nt++)
                     if (tail_bytes(nt, k ? 16 : 8, sizeof(float2)) <= CT_SMEM_BYTES) h->ctail_fit[k] = nt;
-        helm_refresh_tails(h, true);
+        CKC(helm_refresh_tails(h, true));
     }
     CKC(cudaStreamSynchronize(s));
     *out = h;
@@ -603,12 +603,13 @@ const void *ctail_image(const helm_handle *h, int prec, bool deep) {
     return nullptr;
 }
 
-// Builds the image of the selected tail unless the handle has it.  A failure leaves the tail without
-// an image: the deep-halo kernel is then not used, and the other builds its blocks' memory itself.
-template <typename R> static void build_image(helm_handle *h, bool deep) {
+// Builds the image of the selected tail unless the handle has it; true when it launched the build.  A
+// failure leaves the tail without an image: the deep-halo kernel is then not used, and the other builds
+// its blocks' memory itself.
+template <typename R> static bool build_image(helm_handle *h, bool deep) {
     const int prec = sizeof(R) == sizeof(float) ? 0 : 1;
     const helm_handle::Tail &T = h->tail[prec];
-    if (T.top < 0 || ctail_image(h, prec, deep)) return;
+    if (T.top < 0 || ctail_image(h, prec, deep)) return false;
     const int nt = (int)h->lv.size() - T.top;
     DevOp<R> ops[MAX_CT_LEVELS];
     for (int k = 0; k < nt; k++) ops[k] = LvBuf<R>::op(h->lv[T.top + k]);
@@ -621,7 +622,7 @@ template <typename R> static void build_image(helm_handle *h, bool deep) {
         e = build_mg_ctail_image<R>(h->dim, nt, ops, LvBuf<R>::minv(h), h->nu_c, (R)h->mg.omega, T.nc, &img, h->stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        return;
+        return false;
     }
     try {
         h->ctail_img.reserve(h->ctail_img.size() + 1);
@@ -629,14 +630,26 @@ template <typename R> static void build_image(helm_handle *h, bool deep) {
         h->ctail_img.push_back({image_key(T.top, T.nc, deep, prec), img});
     } catch (...) {
         cudaFree(img);
+        return false;
     }
+    return true;
 }
 
-void helm_refresh_tails(helm_handle *h, bool build) {
+// Whether work put on the handle's stream now would be captured into a graph instead of run.
+static bool stream_captures(const helm_handle *h) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+cudaError_t helm_refresh_tails(helm_handle *h, bool build) {
     const helm_mg_params &m = h->mg;
     const helm_tuning &t = h->tune;
     h->tail[0] = h->tail[1] = helm_handle::Tail{};
-    if (m.kind == HELM_PC_NONE) return;
+    if (m.kind == HELM_PC_NONE) return cudaSuccess;
     const int nlev = (int)h->lv.size();
     for (int prec = 0; prec < 2; prec++) {
         helm_handle::Tail &T = h->tail[prec];
@@ -658,13 +671,18 @@ void helm_refresh_tails(helm_handle *h, bool build) {
             T.deep = mg_chalo_bytes(nlev - T.top, ops, h->nu_c, T.nc) > 0;
         }
     }
-    if (!build) return;
+    if (!build) return cudaSuccess;
+    const bool can = !stream_captures(h);
+    bool built = false;
     if (h->tail[0].deep) {
-        build_image<float>(h, true);
+        if (can) built |= build_image<float>(h, true);
         if (!ctail_image(h, 0, true)) h->tail[0].deep = false;
     }
-    if (!h->tail[0].deep) build_image<float>(h, false);
-    build_image<double>(h, false);
+    if (can && !h->tail[0].deep) built |= build_image<float>(h, false);
+    if (can) built |= build_image<double>(h, false);
+    // The tails copy their image before they wait for the kernel ahead of them, and the next kernel on the
+    // stream can be a tail: nothing returns to the caller before the images are in memory.
+    return built ? cudaStreamSynchronize(h->stream) : cudaSuccess;
 }
 
 // u <- MG(l, M_l, b, u, nu1, nu2, C, gf, gc).  'zero' means u = 0 on entry (not read).

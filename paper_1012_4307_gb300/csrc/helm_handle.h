@@ -190,9 +190,9 @@ float2 *level0_rhs_c64(helm_handle *h);
 // The tile of level l: the tuning's, or without one a choice by the level's size.
 int helm_level_tile(const helm_handle *h, int l);
 // Recomputes h->tail for the handle's tuning; with build, also builds the initial shared-memory
-// images its cycles use (allocates device memory and launches on the handle's stream; outside graph
-// capture).
-void helm_refresh_tails(helm_handle *h, bool build);
+// images its cycles use (allocates device memory, launches on the handle's stream and waits for it; while
+// the stream is being captured nothing is built and the tails run without new images).
+cudaError_t helm_refresh_tails(helm_handle *h, bool build);
 // The initial shared-memory image of a complex64 (prec 0) or complex128 (1) tail (deep: of the
 // deep-halo kernel); null if it was not built.
 const void *ctail_image(const helm_handle *h, int prec, bool deep);

@@ -50,7 +50,7 @@ extern "C" helm_status helm_set_tuning(helm_handle *h, const helm_tuning *t) {
     h->tune = *t;
     h->tuned = true;
     helm_drop_graphs(h);
-    helm_refresh_tails(h, true);
+    CKR(helm_refresh_tails(h, true));
     return HELM_OK;
 }
 
@@ -92,12 +92,13 @@ extern "C" helm_status helm_autotune(helm_handle *h, helm_prec prec, int reps, h
     // skipped
     auto time_it = [&](const helm_tuning &t, bool soft = false) -> double {
         h->tune = t;
-        helm_refresh_tails(h, true);
+        cudaError_t e = helm_refresh_tails(h, true);
+        if (e != cudaSuccess) return fail(e, "tail images");
         cudaStream_t keep_s = h->stream;
         cudaGraph_t g = nullptr;
         cudaGraphExec_t ge = nullptr;
         h->stream = h->cap_stream;
-        cudaError_t e = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal);
+        e = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             pdl_capture_scope no_pdl;
             h->capturing = true;
@@ -205,7 +206,7 @@ extern "C" helm_status helm_autotune(helm_handle *h, helm_prec prec, int reps, h
         // per level above the tails, greedily from the finest: separate launches or a tile shape
         if (blockable) {
             h->tune = cur;
-            helm_refresh_tails(h, false);
+            (void)helm_refresh_tails(h, false);  // builds nothing
             const int stop = std::min(h->tail[0].top >= 0 ? h->tail[0].top : last, HELM_MAX_LEVELS);
             for (int l = 0; l < stop && st == HELM_OK; l++) {
                 for (int tile = HELM_TILE_NONE; tile < HELM_TILE_COUNT && st == HELM_OK; tile++) {
@@ -229,8 +230,9 @@ extern "C" helm_status helm_autotune(helm_handle *h, helm_prec prec, int reps, h
     h->tune = st == HELM_OK ? cur : keep;
     h->tuned = st == HELM_OK ? true : kept_tuned;
     helm_drop_graphs(h);
-    helm_refresh_tails(h, true);
+    const cudaError_t e = helm_refresh_tails(h, true);
     if (st != HELM_OK) return st;
+    CKR(e);
     if (best) *best = cur;
     if (best_ms) *best_ms = cur_ms;
     return HELM_OK;
