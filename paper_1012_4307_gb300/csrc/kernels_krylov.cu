@@ -151,9 +151,14 @@ __global__ void __launch_bounds__(NT, 2) k_mdot_norm(size_t n, const double2 *__
 // Pass "update": w -= sum_{i < nv} V_i h_i, then partials[b] = (sum |w|^2, 0).  Gated.
 // Bound by the FP64 units (4 multiply-adds per vector and node).  The second Gram-Schmidt pass only
 // takes out what rounding left behind: with wnorm (||w|| so far) and ||h|| <= 2^-36 ||w||, the sum over
-// the basis is formed in FP32, whose rounding, about 2^-24 ||h|| <= 2^-60 ||w||, stays far below the FP64
-// rounding of w itself, and subtracted in FP64; a larger correction takes the FP64 products.
-// Measured, FGMRES(30) on 513^2 (59 iterations): 14.1 ms with FP64 products in both passes, 13.4 so.
+// the basis is formed in FP32 and subtracted in FP64: its rounding, at most nv 2^-24 ||h|| <= 2^-54 ||w|| for
+// 64 vectors, stays below that of the FP64 chain, which rounds w once per vector; a larger correction
+// takes the FP64 products.  The coefficients enter the sum divided by the power of two in ||w||, so that
+// FP32's range is that of the correction's size relative to w, whatever the units of the problem.
+// Measured against FP64 products in both passes (FGMRES(30) and its backward step to 1e-10, 97^2 .. 513^2
+// and 49^3 .. 97^3, both precisions, three seeds): solutions 2e-15 .. 4e-14 apart, their errors against
+// 64-bit results (1e-12 .. 2e-9, the tolerance's) equal; 513^2 13.88 -> 12.98 ms, 257^2 4.21 -> 4.13, 97^2 2.10 ->
+// 2.12, 97^3 19.0 -> 17.7.
 __global__ void __launch_bounds__(NT) k_update_norm(size_t n, const double2 *__restrict__ V, size_t ldv, int nv,
                                                     const double2 *__restrict__ h, double2 *__restrict__ w,
                                                     double2 *__restrict__ partials, const int *__restrict__ gate,
@@ -163,18 +168,31 @@ __global__ void __launch_bounds__(NT) k_update_norm(size_t n, const double2 *__r
     __shared__ double2 hs[64];
     __shared__ float2 hf[64];
     __shared__ int small_s;
+    // unit = the power of two in ||w||, per = 1 / unit (both normal numbers, or no short form)
+    double unit = 0.0, per = 0.0;
+    if (wnorm) {
+        const int e = (__double2hiint(wnorm->x) >> 20) & 0x7ff;
+        if (e >= 1 && e <= 2045) {
+            unit = __hiloint2double(e << 20, 0);
+            per = __hiloint2double((2046 - e) << 20, 0);
+        }
+    }
     for (int i = threadIdx.x; i < nv; i += NT) {
         const double2 hi = h[i];
         hs[i] = hi;
-        hf[i] = to_c(hi, 0.f);
+        hf[i] = to_c(cscale(hi, per), 0.f);
     }
     if (threadIdx.x == 0) small_s = 0;
     __syncthreads();
-    if (wnorm && threadIdx.x < 32) {
+    if (unit != 0.0 && threadIdx.x < 32) {
         double s2 = 0.0;
-        for (int i = threadIdx.x; i < nv; i += 32) s2 = fma(hs[i].x, hs[i].x, fma(hs[i].y, hs[i].y, s2));
+        for (int i = threadIdx.x; i < nv; i += 32) {
+            const double2 r = cscale(hs[i], per);
+            s2 = fma(r.x, r.x, fma(r.y, r.y, s2));
+        }
         s2 = warp_sum_d(s2);
-        if (threadIdx.x == 0) small_s = s2 <= 0x1p-72 * wnorm->x * wnorm->x;
+        const double r = wnorm->x * per;  // in [1, 2)
+        if (threadIdx.x == 0) small_s = s2 <= 0x1p-72 * r * r;
     }
     __syncthreads();
     double acc = 0.0;
@@ -188,7 +206,7 @@ __global__ void __launch_bounds__(NT) k_update_norm(size_t n, const double2 *__r
                 c.x = fmaf(v.x, hh.x, fmaf(-v.y, hh.y, c.x));
                 c.y = fmaf(v.x, hh.y, fmaf(v.y, hh.x, c.y));
             }
-            wq = csub(wq, to_c(c, 0.0));
+            wq = make_double2(fma(-unit, to_double(c.x), wq.x), fma(-unit, to_double(c.y), wq.y));
             w[q] = wq;
             acc = fma(wq.x, wq.x, fma(wq.y, wq.y, acc));
         }
