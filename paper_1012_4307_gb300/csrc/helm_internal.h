@@ -41,8 +41,10 @@ template <typename C> __host__ __device__ __forceinline__ C cinv(C a) {
     const auto r = decltype(d)(1) / d;
     return mk(a.x * r, -a.y * r);
 }
-// 1 / a for complex64 with the fast approximate reciprocal (__fdividef, about 2 ulp): used
-// where the result only enters a complex64 smoother update.
+// 1 / a for complex64 with the fast approximate reciprocal (__fdividef: about 2 ulp, and 0 where |a|^2
+// exceeds 2^126): only where a kernel forms it at every node (the residual of the blocked pre-smoother, which
+// recovers D from 1 / D, and the wavefront).  What is formed once, 1 / D of the levels and tails, is
+// divided (cinv).
 __device__ __forceinline__ float2 cinv_fast(float2 a) {
     const float r = __fdividef(1.0f, fmaf(a.x, a.x, a.y * a.y));
     return make_float2(a.x * r, -a.y * r);

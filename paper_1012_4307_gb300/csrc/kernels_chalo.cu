@@ -45,7 +45,7 @@ struct HLevel {
     int B[MAX_CT_BLOCKS + 1];
     // byte offsets in shared memory (same in every block): right-hand side, iterate, second
     // iterate / residual, result copy for the finer level, diagonal of M and its reciprocal
-    // (cinv_fast, formed once), x and y coefficients
+    // (formed once), x and y coefficients
     unsigned ob, ou, ot, oe, od, oi, ocx, ocy;
 };
 
@@ -312,7 +312,7 @@ __device__ __noinline__ void hd_init(Ctx X, const HArgs *A) {
             const float k2 = G.k2[(size_t)(ja + r) * L.nx + i];
             const float2 d = cadd(cadd(cx[3 * i + 1], cy[3 * s + 1]), cadd(cscale(L.bk, k2), L.c));
             dg[(size_t)s * L.nx + i] = d;
-            di[(size_t)s * L.nx + i] = cinv_fast(d);
+            di[(size_t)s * L.nx + i] = cinv(d);
         }
     }
     if (A->mrow) {

@@ -463,8 +463,8 @@ __device__ __noinline__ void ct_init(Ctx X, const CArgs<R> *A) {
             const C d = cadd(cc, cadd(cscale(L.bk, k2), L.c));
             dg[p] = d;
             // (a boundary node's entries are never read)
-            if constexpr (sizeof(R) == sizeof(float)) di[p] = cinv_fast(d);
-            else di[p] = cscale(cinv(d), A->omega);
+            di[p] = cinv(d);
+            if constexpr (sizeof(R) == sizeof(double)) di[p] = cscale(di[p], A->omega);
         }
     }
     if (A->mrow) ph_stage_minv(X, A);

@@ -1447,8 +1447,8 @@ template <typename R> __global__ void k_diag_inv(OpView<R> o, int dim, R omega, 
             C d = cadd(o.cx[3 * x + 1], o.cy[3 * y + 1]);
             if (dim == 3) d = cadd(d, o.cz[3 * k + 1]);
             d = cadd(d, cadd(cscale(o.bk, o.k2[p]), o.c));
-            if constexpr (sizeof(R) == sizeof(float)) v = cinv_fast(d);
-            else v = cscale(cinv(d), omega);
+            v = cinv(d);
+            if constexpr (sizeof(R) == sizeof(double)) v = cscale(v, omega);
         }
         dinv[p] = v;
     }

@@ -71,3 +71,25 @@ def test_fp64_gram_schmidt_with_large_second_corrections(helm, power):
     ref = np.linalg.solve(A, f[1:-1, 1:-1].ravel())
     # condition number about 100, residual at most 1e-11
     assert rel_l2(to_np(x)[1:-1, 1:-1].ravel() * 2.0 ** (-2 * power), ref) <= 2e-9
+
+
+@pytest.mark.parametrize("n,power,smoother,nu,tail", [
+    ((49, 49), -26, "jacobi", (1, 2), 0), ((49, 49), -26, "rb", (1, 1), 0),       # level tiles
+    ((49, 49), -26, "jacobi", (1, 2), -1), ((49, 49), -26, "rb", (1, 1), -1),     # cluster tail
+    ((49, 49), -26, "jacobi", (2, 2), -1), ((21, 21, 21), -27, "jacobi", (1, 1), -1),
+])
+def test_complex64_diagonals_keep_their_range(helm, n, power, smoother, nu, tail):
+    """Diagonals of about 1e19, whose squared moduli are just below the largest float (between 2^126 and
+    2^128): their reciprocals are formed by a division, not by an approximation that gives 0 there.  The
+    scaled cycle is the unscaled one up to complex64 rounding (the reciprocal of a squared modulus is a
+    subnormal with 22 bits here): the bound of the other complex64 cycles, 2e-5."""
+    dim = len(n)
+    k2 = W.k2_well_growth(dim, n[0], kh_max=0.3)
+    v = to_gpu(W.random_field(tuple(reversed(n)), 7))
+    out = []
+    for p in (0, power):
+        h = handle(helm, n, k2, p, prec="c64", smoother=smoother, nu=nu, coarsest_n=13 if dim == 2 else 7)
+        if tail >= 0:
+            helm.helm_set_tuning(h, dict(tail_levels=tail))
+        out.append(to_np(helm.mg_precondition(h, v)).astype(np.complex128) * 2.0 ** (-2 * p))
+    assert rel_l2(out[1], out[0]) <= 2e-5
