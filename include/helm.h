@@ -157,7 +157,9 @@ helm_status helm_apply(helm_handle *h, helm_op which, helm_prec prec, const void
  * (nu1, nu2, omega, smoother, gamma_f, gamma_c).
  *   b   DEVICE right-hand side (precision prec), unchanged.
  *   x   DEVICE initial guess on entry, cycle result on exit (precision prec).
- * b and x must not overlap. */
+ * b and x must not overlap.  The first complex128 cycle on a handle with mg->prec HELM_C64 allocates what
+ * complex128 cycles need beside the levels (16 bytes per node) and waits for it; on a handle with
+ * mg->prec HELM_C128 helm_create has done so.  Errors: HELM_ERR_NOMEM among others. */
 helm_status mg_vcycle(helm_handle *h, const void *b, void *x, helm_prec prec);
 
 /* The preconditioner call of the outer solvers: z = one cycle of Algorithm 1 for M z = v from

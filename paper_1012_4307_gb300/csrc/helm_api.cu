@@ -205,6 +205,8 @@ helm_status helm_validate_create(const helm_grid *grid, const double *r0_lo, con
     return HELM_OK;
 }
 
+static cudaError_t form_c128(helm_handle *h, cudaStream_t s);
+
 helm_status helm_create_impl(const helm_grid *grid, double theta, const double *r0_lo, const double *r0_hi,
                              const std::vector<double> &k2h, const helm_mg_params *mg, cudaStream_t s,
                              helm_handle **out) {
@@ -311,15 +313,12 @@ helm_status helm_create_impl(const helm_grid *grid, double theta, const double *
             CKC(launch_diag_inv<float>(L.M32, dim, (float)mg->omega, di, s));
             L.M32.dinv = di;
         }
-        if (mg->kind != HELM_PC_NONE) {  // omega / diagonal for the complex128 sweeps
-            double2 *di = nullptr;
-            CKC(dalloc(&di, L.np, h->owned));
-            CKC(launch_diag_inv<double>(L.M64, dim, mg->omega, di, s));
-            L.M64.dinv = di;
-        }
         CKC(dalloc(&L.b64, L.np, h->owned)); CKC(dalloc(&L.u64, L.np, h->owned));
         CKC(dalloc(&L.t64, L.np, h->owned)); CKC(dalloc(&L.b32, L.np, h->owned));
-        CKC(dalloc(&L.u32, L.np, h->owned)); CKC(dalloc(&L.t32, L.np, h->owned));
+        // t32 and u32 side by side: together room for one complex128 vector (C128Borrowed)
+        const size_t t_len = (L.np + 1) & ~(size_t)1;
+        CKC(dalloc(&L.t32, t_len + L.np, h->owned));
+        L.u32 = L.t32 + t_len;
         CKC(cudaMemsetAsync(L.b64, 0, L.np * sizeof(double2), s)); CKC(cudaMemsetAsync(L.u64, 0, L.np * sizeof(double2), s));
         CKC(cudaMemsetAsync(L.t64, 0, L.np * sizeof(double2), s)); CKC(cudaMemsetAsync(L.b32, 0, L.np * sizeof(float2), s));
         CKC(cudaMemsetAsync(L.u32, 0, L.np * sizeof(float2), s)); CKC(cudaMemsetAsync(L.t32, 0, L.np * sizeof(float2), s));
@@ -415,6 +414,7 @@ helm_status helm_create_impl(const helm_grid *grid, double theta, const double *
                 for (int nt = 2; nt <= std::min(nlev, MAX_CT_LEVELS); nt++)
                     if (tail_bytes(nt, k ? 16 : 8, sizeof(float2)) <= CT_SMEM_BYTES) h->ctail_fit[k] = nt;
         CKC(helm_refresh_tails(h, true));
+        if (mg->prec == HELM_C128) CKC(form_c128(h, s));
     }
     CKC(cudaStreamSynchronize(s));
     *out = h;
@@ -606,7 +606,7 @@ const void *ctail_image(const helm_handle *h, int prec, bool deep) {
 // Builds the image of the selected tail unless the handle has it; true when it launched the build.  A
 // failure leaves the tail without an image: the deep-halo kernel is then not used, and the other builds
 // its blocks' memory itself.
-template <typename R> static bool build_image(helm_handle *h, bool deep) {
+template <typename R> static bool build_image(helm_handle *h, bool deep, cudaStream_t s) {
     const int prec = sizeof(R) == sizeof(float) ? 0 : 1;
     const helm_handle::Tail &T = h->tail[prec];
     if (T.top < 0 || ctail_image(h, prec, deep)) return false;
@@ -616,10 +616,10 @@ template <typename R> static bool build_image(helm_handle *h, bool deep) {
     void *img = nullptr;
     cudaError_t e = cudaErrorInvalidValue;
     if constexpr (sizeof(R) == sizeof(float)) {
-        if (deep) e = build_mg_chalo_image(nt, ops, h->minv32, h->nu_c, T.nc, &img, h->stream);
+        if (deep) e = build_mg_chalo_image(nt, ops, h->minv32, h->nu_c, T.nc, &img, s);
     }
     if (!deep)
-        e = build_mg_ctail_image<R>(h->dim, nt, ops, LvBuf<R>::minv(h), h->nu_c, (R)h->mg.omega, T.nc, &img, h->stream);
+        e = build_mg_ctail_image<R>(h->dim, nt, ops, LvBuf<R>::minv(h), h->nu_c, (R)h->mg.omega, T.nc, &img, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return false;
@@ -675,14 +675,79 @@ cudaError_t helm_refresh_tails(helm_handle *h, bool build) {
     const bool can = !stream_captures(h);
     bool built = false;
     if (h->tail[0].deep) {
-        if (can) built |= build_image<float>(h, true);
+        if (can) built |= build_image<float>(h, true, h->stream);
         if (!ctail_image(h, 0, true)) h->tail[0].deep = false;
     }
-    if (can && !h->tail[0].deep) built |= build_image<float>(h, false);
-    if (can) built |= build_image<double>(h, false);
+    if (can && !h->tail[0].deep) built |= build_image<float>(h, false, h->stream);
+    if (can && h->c128) built |= build_image<double>(h, false, h->stream);
     // The tails copy their image before they wait for the kernel ahead of them, and the next kernel on the
     // stream can be a tail: nothing returns to the caller before the images are in memory.
     return built ? cudaStreamSynchronize(h->stream) : cudaSuccess;
+}
+
+// omega / D of every level (16 bytes a node) and the image of the complex128 tail, formed on stream s, which
+// is waited for.
+static cudaError_t form_c128(helm_handle *h, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    try {
+        h->owned.reserve(h->owned.size() + h->lv.size());
+    } catch (...) {
+        return cudaErrorMemoryAllocation;
+    }
+    const size_t kept = h->owned.size();
+    for (LevelDev &L : h->lv) {
+        double2 *di = nullptr;
+        if (e == cudaSuccess) e = dalloc(&di, L.np, h->owned);
+        if (e == cudaSuccess) e = launch_diag_inv<double>(L.M64, h->dim, h->mg.omega, di, s);
+        L.M64.dinv = di;
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) {
+        for (LevelDev &L : h->lv) L.M64.dinv = nullptr;
+        for (size_t q = kept; q < h->owned.size(); q++) cudaFree(h->owned[q]);
+        h->owned.resize(kept);
+        return e;
+    }
+    h->c128 = true;
+    return build_image<double>(h, false, s) ? cudaStreamSynchronize(s) : cudaSuccess;
+}
+
+// A complex128 handle has them from its creation; another forms them in its first complex128 cycle, on a
+// stream of its own and with allocations allowed, since the handle's stream may be being captured.
+helm_status helm_need_c128(helm_handle *h) {
+    if (h->c128) return HELM_OK;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    CKR(cudaThreadExchangeStreamCaptureMode(&mode));
+    cudaStream_t s = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e == cudaSuccess) {
+        pdl_capture_scope plain;
+        e = form_c128(h, s);
+        cudaStreamDestroy(s);
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) return HELM_OK;
+    cudaGetLastError();
+    return helm_fail(e == cudaErrorMemoryAllocation ? HELM_ERR_NOMEM : HELM_ERR_CUDA, "complex128 diagonals: %s",
+                     cudaGetErrorString(e));
+}
+
+// A level's t32 and u32 lie side by side and hold nothing between cycles.
+C128Borrowed::C128Borrowed(helm_handle *h_, bool want) : h(h_), on(want && !h_->c128) {
+    if (!on) return;
+    for (LevelDev &L : h->lv) {
+        if (e == cudaSuccess) e = launch_diag_inv<double>(L.M64, h->dim, h->mg.omega, (double2 *)L.t32, h->stream);
+        L.M64.dinv = (double2 *)L.t32;
+    }
+    h->c128 = e == cudaSuccess;
+}
+C128Borrowed::~C128Borrowed() {
+    if (!on) return;
+    for (LevelDev &L : h->lv) {
+        L.M64.dinv = nullptr;
+        cudaMemsetAsync(L.t32, 0, L.np * sizeof(double2), h->stream);
+    }
+    h->c128 = false;
 }
 
 // u <- MG(l, M_l, b, u, nu1, nu2, C, gf, gc).  'zero' means u = 0 on entry (not read).
@@ -822,8 +887,10 @@ cudaError_t precondition(helm_handle *h, const double2 *v, typename CT<R>::T *z)
         ProfScope ps(h, HELM_K_VECTOR, h->np * (16 + es), 0);
         return launch_convert(h->np, v, z, h->stream);
     }
-    if (sizeof(R) == sizeof(double))
+    if (sizeof(R) == sizeof(double)) {
+        if (helm_need_c128(h) != HELM_OK) return cudaErrorMemoryAllocation;
         return cycle<R>(h, 0, (const typename CT<R>::T *)v, z, true, h->mg.gamma_f, h->mg.gamma_c);
+    }
     if (first_launch_rounds(h))
         return cycle<R>(h, 0, LvBuf<R>::b(h->lv[0]), z, true, h->mg.gamma_f, h->mg.gamma_c, v);
     {
@@ -850,6 +917,7 @@ cudaError_t precondition_pair(helm_handle *h, const float4 *v, const double2 *al
         else CKE(launch_pair_to_c128(h->np, v, alpha, dst, h->stream));
     }
     if (h->mg.kind == HELM_PC_NONE) return cudaSuccess;
+    if (sizeof(R) == sizeof(double) && helm_need_c128(h) != HELM_OK) return cudaErrorMemoryAllocation;
     return cycle<R>(h, 0, dst, z, true, h->mg.gamma_f, h->mg.gamma_c);
 }
 template cudaError_t precondition_pair<float>(helm_handle *, const float4 *, const double2 *, float2 *);
@@ -911,6 +979,7 @@ extern "C" helm_status mg_vcycle(helm_handle *h, const void *b, void *x, helm_pr
     helm_status st;
     if ((st = check_ptr(b, al, "b")) != HELM_OK || (st = check_ptr(x, al, "x")) != HELM_OK) return st;
     if (b == x) return helm_fail(HELM_ERR_ARG, "b and x must not overlap");
+    if (prec == HELM_C128 && (st = helm_need_c128(h)) != HELM_OK) return st;
     if (prec == HELM_C128)
         CKR(cycle<double>(h, 0, (const double2 *)b, (double2 *)x, false, h->mg.gamma_f, h->mg.gamma_c));
     else if (prec == HELM_C64)
@@ -928,6 +997,7 @@ extern "C" helm_status mg_precondition(helm_handle *h, const void *v, void *z, h
         (st = check_ptr(z, prec == HELM_C128 ? 16 : 8, "z")) != HELM_OK)
         return st;
     if (v == z) return helm_fail(HELM_ERR_ARG, "v and z must not overlap");
+    if (prec == HELM_C128 && (st = helm_need_c128(h)) != HELM_OK) return st;
     if (prec == HELM_C128)
         CKR(precondition<double>(h, (const double2 *)v, (double2 *)z));
     else if (prec == HELM_C64)

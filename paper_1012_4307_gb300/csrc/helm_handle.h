@@ -18,7 +18,7 @@ struct LevelDev {
     double *k2_64 = nullptr;
     float *k2_32 = nullptr;
     double2 *b64 = nullptr, *u64 = nullptr, *t64 = nullptr;
-    float2 *b32 = nullptr, *u32 = nullptr, *t32 = nullptr;
+    float2 *b32 = nullptr, *u32 = nullptr, *t32 = nullptr;  // u32 follows t32 in one allocation
 };
 
 // Opt-in launch timing: when on, every kernel launch of the drivers is bracketed by two CUDA
@@ -73,6 +73,7 @@ struct helm_handle {
     int tail_built[2] = {-1, -1}, tail_ctas[2] = {16, 16};
     helm_tuning tune{};                      // kernel choices (see helm_set_tuning)
     bool tuned = false;                      // set by helm_set_tuning or helm_autotune
+    bool c128 = false;                       // complex128 cycles have their omega / D (helm_need_c128)
     int ctail_fit[2] = {0, 0};               // most coarsest levels a cluster tail of 8 / 16 blocks holds
     // the fused tail that the tuning selects, per precision (helm_refresh_tails)
     struct Tail {
@@ -193,6 +194,19 @@ int helm_level_tile(const helm_handle *h, int l);
 // images its cycles use (allocates device memory, launches on the handle's stream and waits for it; while
 // the stream is being captured nothing is built and the tails run without new images).
 cudaError_t helm_refresh_tails(helm_handle *h, bool build);
+// Gives the handle what its complex128 cycles need and complex64 ones do not (allocates in the first call on a
+// complex64 handle, and then waits).
+helm_status helm_need_c128(helm_handle *h);
+// The same while it lives, if wanted, without an allocation: on a complex64 handle that has run no complex128 cycle,
+// omega / D of every level in its t32 and u32 (zeroed again at the end; no complex64 cycle may run meanwhile).
+struct C128Borrowed {
+    helm_handle *h;
+    bool on;
+    cudaError_t e = cudaSuccess;
+    C128Borrowed(helm_handle *h, bool want);
+    C128Borrowed(const C128Borrowed &) = delete;
+    ~C128Borrowed();
+};
 // The initial shared-memory image of a complex64 (prec 0) or complex128 (1) tail (deep: of the
 // deep-halo kernel); null if it was not built.
 const void *ctail_image(const helm_handle *h, int prec, bool deep);

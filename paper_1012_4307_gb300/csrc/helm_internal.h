@@ -129,7 +129,7 @@ template <typename R> struct DevOp {
     C bk, c;
     // formed once by launch_diag_inv (0 off the interior): 2D complex64 levels 1 / (diagonal of M)
     // for the temporally blocked smoothers; complex128 levels omega / (diagonal of M), which every
-    // complex128 sweep uses; null otherwise
+    // complex128 sweep uses (once the handle runs such cycles: helm_need_c128); null otherwise
     const C *dinv = nullptr;
     // device flag (null: none): when it is set at launch, this level's smoothing, residual and
     // transfer kernels return at once (the fused coarse-tail kernels do not test it).  Set only

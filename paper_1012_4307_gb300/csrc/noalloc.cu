@@ -91,6 +91,9 @@ extern "C" helm_status helm_mg_conv_noalloc(helm_handle *h, const void *b, void 
     if ((st = norm(b64, &bn)) != HELM_OK) return st;
     std::vector<double> res(1, bn);
     res.reserve((size_t)maxcyc + 1);
+    // a complex64 handle's first complex128 cycles would allocate their diagonals
+    const C128Borrowed borrowed(h, prec == HELM_C128);
+    CKR(borrowed.e);
     int c = 0;
     while (c < maxcyc) {
         if ((st = mg_vcycle(h, b, x, prec)) != HELM_OK) return st;

@@ -67,6 +67,10 @@ extern "C" helm_status helm_autotune(helm_handle *h, helm_prec prec, int reps, h
     if (reps < 1) return helm_fail(HELM_ERR_ARG, "reps must be >= 1");
     const size_t np = h->np;
     const bool c64 = prec == HELM_C64;
+    if (!c64) {
+        const helm_status need = helm_need_c128(h);
+        if (need != HELM_OK) return need;
+    }
     double2 *v = nullptr;
     void *z = nullptr;
     if (cudaMalloc((void **)&v, np * sizeof(double2)) != cudaSuccess ||
