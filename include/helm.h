@@ -357,8 +357,9 @@ helm_status helm_profile_read(helm_handle *h, int ncls, int *launches, double *m
  * kernels carry it out, and every choice gives the same cycle up to FP32 rounding order.
  *   tail_levels    the coarsest levels (>= 2, or 0 for none) fused into one launch of a thread-
  *                  block cluster, every level in distributed shared memory; -1 = as many as fit
- *                  (at most 6 levels, each with at most 8192 unknowns, 16384 in 2D complex64,
- *                  in 200 KB a block).
+ *                  (at most 6 levels in 200 KB a block, each with at most 8192 unknowns; in 2D
+ *                  complex64 16384, but 10000 in a V(2,2) omega-Jacobi cycle unless the whole grid
+ *                  fits the tail).
  *                  Values above what fits are clamped.
  *   level_tile[l]  level l (0 = finest) of a 2D complex64 V(2,2) omega-Jacobi cycle runs its
  *                  two pre-sweeps + residual + full weighting, and its prolongation + two
@@ -368,9 +369,9 @@ helm_status helm_profile_read(helm_handle *h, int ncls, int *launches, double *m
  *                  transfer launches (HELM_TILE_NONE).  Ignored where it does not apply (other
  *                  smoothers and complex128 cycles, whose 2D levels have blocked launches of
  *                  their own; 3D, levels inside the tail, grids the tile does not fit).
- * Default: tail_levels = -1, HELM_TILE_32x8 on every level, cluster_levels = 0 (16 blocks, cluster_halo 3).
- * While no tuning was set or measured, a handle of its own (not one of a lockstep batch) runs each
- * such level with the tile that suits the level's size instead of 32x8; the results are the same. */
+ * Default: tail_levels = -1, cluster_levels = 0 (16 blocks, cluster_halo 3), and on every level of a 2D
+ * grid the tile that suits the level's size (HELM_TILE_32x8 in a lockstep batch and where that tile does
+ * not fit).  helm_get_tuning reports the tiles in use, so that setting what it reported changes nothing. */
 #define HELM_MAX_LEVELS 16
 typedef enum {
     HELM_TILE_NONE = -1,

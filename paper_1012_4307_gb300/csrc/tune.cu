@@ -57,6 +57,7 @@ extern "C" helm_status helm_set_tuning(helm_handle *h, const helm_tuning *t) {
 extern "C" helm_status helm_get_tuning(const helm_handle *h, helm_tuning *t) {
     if (!h || !t) return helm_fail(HELM_ERR_ARG, "null argument");
     *t = h->tune;
+    for (int l = 0; l < std::min((int)h->lv.size(), HELM_MAX_LEVELS); l++) t->level_tile[l] = helm_level_tile(h, l);
     return HELM_OK;
 }
 
@@ -232,12 +233,12 @@ extern "C" helm_status helm_autotune(helm_handle *h, helm_prec prec, int reps, h
     cudaFree(z);
     h->prof.on = prof;
     h->tune = st == HELM_OK ? cur : keep;
-    h->tuned = st == HELM_OK ? true : kept_tuned;
+    h->tuned = (st == HELM_OK && c64) || kept_tuned;  // complex128 cycles have no such tiles to choose
     helm_drop_graphs(h);
     const cudaError_t e = helm_refresh_tails(h, true);
     if (st != HELM_OK) return st;
     CKR(e);
-    if (best) *best = cur;
+    if (best) helm_get_tuning(h, best);
     if (best_ms) *best_ms = cur_ms;
     return HELM_OK;
 }

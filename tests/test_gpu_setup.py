@@ -1,4 +1,6 @@
 """What the set-up calls leave behind: work in flight, memory, and the kernels that the cycles run."""
+import re
+
 import numpy as np
 import pytest
 
@@ -115,3 +117,40 @@ def test_noalloc_in_complex128_on_a_complex64_handle(helm):
     xr, cr, fr = helm.helm_mg_conv(h, v, tol=1e-6, maxcyc=30)
     assert cycles == cr and torch.equal(x, xr)
     assert torch.equal(helm.mg_precondition(h, v), z64)
+
+
+def kernel_names(fn):
+    """Names of the CUDA kernels fn launches (torch's profiler); None when it records none."""
+    from torch.profiler import ProfilerActivity, profile
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        fn()
+        torch.cuda.synchronize()
+    return {e.name for e in prof.events() if e.device_type == torch.autograd.DeviceType.CUDA} or None
+
+
+@pytest.mark.parametrize("change", ["round trip", "tail only", "autotuned in complex128"])
+def test_tiles_by_size_survive(helm, change):
+    """Reading a handle's tuning and setting it again, changing another field of it, or autotuning the
+    complex128 cycle (which has no such tiles) leaves the complex64 cycle on the tiles that suit its levels."""
+    h = handle(helm, (513, 513), prec="c64")
+    v = to_gpu(W.random_field((513, 513), 64))
+
+    def tiles():
+        names = kernel_names(lambda: helm.mg_precondition(h, v))
+        return names and set(re.findall(r"k_(?:pre2_restrict|prolong_post2)<[^>]*>", " ".join(sorted(names))))
+
+    tiles()  # the first profile of a process may record nothing
+    before, z = tiles(), helm.mg_precondition(h, v)
+    reported = helm.helm_get_tuning(h)
+    if change == "round trip":
+        helm.helm_set_tuning(h, reported)
+    elif change == "tail only":
+        helm.helm_set_tuning(h, dict(tail_levels=reported["tail_levels"]))
+    else:
+        tuning, _ = helm.helm_autotune(h, "c128", reps=2)
+        assert tuning == helm.helm_get_tuning(h) and tuning["level_tile"] == reported["level_tile"]
+        helm.helm_set_tuning(h, dict(tail_levels=reported["tail_levels"]))
+    assert helm.helm_get_tuning(h)["level_tile"] == reported["level_tile"]
+    after = tiles()
+    assert before is None or after is None or (after == before and len(before) >= 4)
+    assert torch.equal(helm.mg_precondition(h, v), z)
