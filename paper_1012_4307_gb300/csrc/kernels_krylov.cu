@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(NT) k_backsolve(const double2 *H, int ldh, int
 }
 
 // Bi-CGSTAB scalar block (device): 0 rho, 1 rho_old, 2 alpha, 3 omega, 4 beta, 5 <rh,v>,
-// 6 <t,s>, 7 <t,t>, 8 -alpha, 9 -omega, 10 one, 11 flags (x: breakdown)
+// 6 <t,s>, 7 <t,t>, 8 -alpha, 9 -omega, 11 flags (x: breakdown)
 __device__ __forceinline__ void bicg_stage(int stage, double2 *sc) {
     const double2 zero = make_double2(0.0, 0.0);
     auto isz = [](double2 v) { return v.x == 0.0 && v.y == 0.0; };
@@ -464,7 +464,7 @@ __device__ __forceinline__ void bicg_stage(int stage, double2 *sc) {
         sc[1] = sc[0];
         if (isz(sc[3])) sc[11].x = 1.0;
     } else {                     // init: rho_old = alpha = omega = 1, flags = 0
-        sc[1] = sc[2] = sc[3] = sc[10] = make_double2(1.0, 0.0);
+        sc[1] = sc[2] = sc[3] = make_double2(1.0, 0.0);
         sc[11] = zero;
     }
 }

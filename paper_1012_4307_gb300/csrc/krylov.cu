@@ -728,7 +728,7 @@ static helm_status bicgstab(helm_handle *h, const double2 *f, double2 *x, double
     if (s0 != HELM_OK) return s0;
     const size_t np = h->np;
     cudaStream_t s = h->stream;
-    double2 *sc = h->scal;  // 0 rho 1 rho_old 2 alpha 3 omega 4 beta 5 rv 6 ts 7 tt 8 -alpha 9 -omega 10 one 11 flags
+    double2 *sc = h->scal;  // 0 rho 1 rho_old 2 alpha 3 omega 4 beta 5 rv 6 ts 7 tt 8 -alpha 9 -omega 11 flags
     double2 *nrm = h->scal + 16;
     double2 hv[2];
     helm_status rs;
