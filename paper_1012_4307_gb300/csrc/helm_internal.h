@@ -149,11 +149,12 @@ struct DevOpDF {
 cudaError_t launch_apply_A_df(const DevOpDF &op, int dim, const float2 *z, float4 *y, cudaStream_t s,
                              const int *gate = nullptr);
 
-// Programmatic dependent launch.  Every kernel of the library begins with pdl_wait() (it returns
+// Programmatic dependent launch.  Every kernel of the library calls pdl_wait() (it returns
 // once the kernel before it in the stream has finished and its writes are visible; a no-op when
-// the kernel was launched without the attribute) and pdl_trigger() (the next kernel may be
-// scheduled as soon as all of this kernel's blocks have started, so its launch overlaps this
-// kernel's tail).  launch_pdl() launches with the attribute, except while the calling thread
+// the kernel was launched without the attribute) before it reads what another kernel may have written, and
+// pdl_trigger() (the next kernel may be scheduled as soon as all of this kernel's blocks have started, so
+// its launch overlaps this kernel's tail).  Most begin with both; the blocked pair, the level tiles and the
+// tails first load what only the set-up writes, which waits for it: operator coefficients, 1 / D, images.  launch_pdl() launches with the attribute, except while the calling thread
 // captures a CUDA graph (pdl_capture_scope): measured on GB300, replayed graphs of the FGMRES
 // steps ran about 4% slower with programmatic edges, while eager launch sequences (the cycle
 // alone) ran about 10% faster with them.

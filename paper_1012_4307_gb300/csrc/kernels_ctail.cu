@@ -27,8 +27,9 @@
 //
 // What bounds it: the latency of its dependent phases (a cluster barrier and a few shared-memory
 // round trips, about 0.8 us each) in complex64, and 16 SMs' FP64 units in complex128.  Measured per
-// cycle against a single block with the same levels in its shared memory: 129^2 complex64 V(2,2)
-// 72.9 -> 25.1 us, 641^2 complex128 F cycle (nine tails) 2404 -> 880 us, 257^3 complex64 876 -> 757 us.
+// cycle against a single block with the same levels in its shared memory (and, in complex128, its sweeps
+// with a division at every node): 129^2 complex64 V(2,2) 71.7 -> 24.6 us, 641^2 complex128 F cycle (nine
+// tails) 2396 -> 755 us, 257^3 complex64 876 -> 757 us.
 #include <cooperative_groups.h>
 
 #include <algorithm>

@@ -245,8 +245,8 @@ __global__ void __launch_bounds__(NT) k_update_norm_pair(size_t n, const float4 
 // problem's share of a batched launch).
 // gv != 0 (a gate flag's value): stop after the first loads (the partials are then meaningless).
 // STREAM: the basis is loaded as streaming data, so that x and w, which the other block rows read too,
-// stay cached (1025^2: 21.23 -> 21.05 ms per solve; over several problems, where it does not pay, 75.0 ->
-// 77.8 ms per batch of 12, it is off).
+// stay cached (1025^2: 20.4 ms per solve, 20.7 with plain loads; over several problems, where it does not
+// pay, 77.8 against 75.0 ms per batch of 12, it is off).
 template <int CH, bool STREAM>
 __device__ __forceinline__ void mdot2_body(size_t n, const float4 *__restrict__ V, size_t ldv, int nv,
                                            const float4 *__restrict__ x, const float4 *__restrict__ w,
@@ -362,9 +362,10 @@ __device__ __forceinline__ void update2_nodes(size_t n, float4 *__restrict__ V, 
                                               float2 *__restrict__ b_out, float &sn, float &cn, int bx, int nblk) {
     float4 *x = V + (size_t)j * ldv, *w = V + (size_t)(j + 1) * ldv;
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    // The dot pass before this one sweeps the nodes upwards, so L2 holds the top of every
-    // vector it read: this pass sweeps downwards and starts on those lines, and it ends at
-    // the bottom, where the next step's dot pass starts.
+    // The dot pass before this one sweeps the nodes upwards and ends at the top: this pass sweeps
+    // downwards, so that it starts where L2 may still hold what that pass read last (x and w, and of the
+    // basis what the streaming loads of a single problem have left there), and ends at the bottom, where the
+    // next step's dot pass starts (1025^2: 20.4 ms per solve, 20.55 sweeping upwards).
     const size_t stride = (size_t)nblk * NT, base = bx * (size_t)NT + threadIdx.x;
     for (size_t round = (n + stride - 1) / stride; round-- > 0;) {
         const size_t q = round * stride + base;

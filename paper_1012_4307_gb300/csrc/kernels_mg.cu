@@ -237,8 +237,8 @@ __global__ void __launch_bounds__(BX *BY) k_jacobi(OpView<R> o, R omega, const C
 // 3D omega-Jacobi: k_jacobi's arithmetic in the same order, with the x and y coefficient
 // triples loaded once per thread, the (z - 1, z, z + 1) column in registers, and the next plane's
 // operands (four in-plane neighbours, z + 2, b, k^2) loaded while this plane is computed.
-// KC: fine planes per thread (shorter chunks on small grids give more blocks; 16 against 8 on 257^3: 695
-// against 700 us per cycle).  ZERO with a complex128 b
+// KC: fine planes per thread (shorter chunks on small grids give more blocks; at most 16 against
+// at most 8 on 257^3: 690 against 694 us per cycle).  ZERO with a complex128 b
 // in a complex64 cycle: the sweep also writes b rounded to complex64 to b_out.
 template <typename R, typename CB, bool ZERO, int KC>
 __global__ void __launch_bounds__(BX *BY) k_jacobi3(OpView<R> o, R omega, const CB *__restrict__ b,
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(BX *BY) k_jacobi3(OpView<R> o, R omega, const 
             bn = to_c(b[q], R());
             kn = o.k2[q];
         }
-        // the lines two planes ahead into L2 (257^3: 733 us per cycle with them, 747 without; further
+        // the lines two planes ahead into L2 (257^3: 690 us per cycle with them, 734 without; further
         // ahead or in the residual kernel no gain)
         if (k + 2 < k1 && (threadIdx.x & 15) == 0) {
             const size_t q = p + 2 * sz;
@@ -469,12 +469,10 @@ __global__ void __launch_bounds__(BX *BY) k_prolong_add(int nx, int ny, int nz, 
 // take turns at that sum: a group waits for the plane in its own turn only and merely arrives at the
 // barrier in the others' (restrict_turns.h), so that the sum does not hold up the march of the other
 // warps.  Five shared planes for the four turns: every warp then waits in a turn of its own between a
-// group's reads of a plane and its own next store into it.  (257^3 complex64 finest level: 141 us per launch
-// with one barrier and the same four warps summing every fine plane, 128 us with the z sums in registers,
-// the cycle 725 -> 700 us with the turns; four lanes per coarse node in every warp instead: 141 us.)  An odd
-// fine plane 2K + 1 completes coarse plane
-// K and starts K + 1.  Fine nodes outside the grid's interior hold zero
-// residuals.  Same weights as k_residual_restrict, applied per axis.
+// group's reads of a plane and its own next store into it.  (257^3 complex64: 120 us
+// per launch on the finest level and 690 us per cycle; 702 us with every warp waiting at every plane.)  An
+// odd fine plane 2K + 1 completes coarse plane K and starts K + 1.  Fine nodes outside the grid's interior
+// hold zero residuals.  Same weights as k_residual_restrict, applied per axis.
 constexpr int R3_TX = 16, R3_TY = 8, R3_KC = 8;
 constexpr int R3_FW = 2 * R3_TX + 1, R3_FH = 2 * R3_TY + 1;  // fine region
 constexpr int R3_NT = ((R3_FW * R3_FH + 31) / 32) * 32;       // threads: one per region node
@@ -714,6 +712,7 @@ __global__ void __launch_bounds__(BX *BY) k_prolong3(int nx, int ny, int nz, con
         C sn = sb, un = uq;
         if (k + 1 < k1) {
             un = uf[p + (size_t)nx * ny];
+            // three planes ahead into L2 (257^3: 690 us per cycle with it, 702 without)
             if (k + 3 < k1 && (threadIdx.x & 15) == 0) l2_prefetch(&uf[p + 3 * (size_t)nx * ny]);
             if (((k + 2) >> 1) != ((k + 1) >> 1)) sn = corner_sum((k + 2) >> 1);
         }
@@ -895,7 +894,7 @@ __device__ __forceinline__ float2 tile_diag(const TC &tc, int sx, int sy, float 
 // CB double2: b is a complex128 vector; its owned nodes rounded to complex64 go to b_out too.
 // EARLY: the caller has not yet waited for the kernel before it in the stream: the operator's data
 // (coefficients and 1 / D, which no kernel writes) is loaded before the wait (1025^2 complex64 cycle, eager:
-// 74.3 -> 69.4 us; its FGMRES solve in replayed graphs 21.05 -> 20.84 ms).  The batched kernels fill the
+// 69.6 us, with the loads after it 74.8; its FGMRES solve in replayed graphs 20.4 against 20.8 ms).  The batched kernels fill the
 // chip and keep the plain order.
 template <int TCX, int TCY, bool EARLY, typename CB>
 __device__ __forceinline__ void pre2_restrict_tile(const OpView<float> &o, float omega, const CB *__restrict__ b,
