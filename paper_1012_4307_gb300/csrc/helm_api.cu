@@ -798,9 +798,10 @@ static cudaError_t cycle(helm_handle *h, int l, const typename CT<R>::T *b, type
             {
                 // fused: read b and 1/D, write u and the coarse residual; pass by pass: the
                 // first sweep from zero (b, k^2 -> u), the second (u, b, k^2 -> u), the
-                // residual with full weighting (u, b, k^2 -> coarse)
-                ProfScope ps(h, l == 0 ? HELM_K_SMOOTH_FINE : HELM_K_SMOOTH_COARSE, ni * (es + es + es + es / nd), 0,
-                             ni * ((2 * es + rs) + (3 * es + rs) + (2 * es + rs + es / nd)));
+                // residual with full weighting (u, b, k^2 -> coarse); from v, that is read and b written
+                const double vs = v ? 16.0 : 0.0;
+                ProfScope ps(h, l == 0 ? HELM_K_SMOOTH_FINE : HELM_K_SMOOTH_COARSE, ni * (vs + es + es + es + es / nd), 0,
+                             ni * (vs + (2 * es + rs) + (3 * es + rs) + (2 * es + rs + es / nd)));
                 if (v) CKE(launch_pre2_restrict_c128(L.M32, tile, (float)h->mg.omega, v, const_cast<float2 *>(b), L.t32, Lc.b32, h->stream));
                 else CKE(launch_pre2_restrict(L.M32, tile, (float)h->mg.omega, b, L.t32, Lc.b32, h->stream));
             }

@@ -365,7 +365,7 @@ static cudaError_t fgmres_step(helm_handle *h, int j, int m) {
     }
     if (fork) CKE(cudaEventRecord(h->ev_join, h->side));
     {
-        ProfScope ps(h, HELM_K_VECTOR, np * 32.0, df ? 0.0 : np * 2.0);
+        ProfScope ps(h, HELM_K_VECTOR, np * (fp64_fold(h) ? 40.0 : 32.0), df ? 0.0 : np * 2.0);
         const double2 *norm = h->scal + 20;  // ||w||, kept for this pass: the rotation replaces it in H
         if (df) CKE(launch_scale_inv_pair(np, (float4 *)w, norm, s));
         else CKE(launch_scale_inv(np, w, norm, w, fp64_fold(h) ? level0_rhs_c64(h) : nullptr, s));
@@ -761,31 +761,45 @@ static helm_status bicgstab(helm_handle *h, const double2 *f, double2 *x, double
         CKR(dev_dot(h, h->brh, h->br, sc + 0));                                   // rho
         CKR(launch_bicg_scalars(0, sc, s));                                       // beta
     }
+    // a vector pass that reads and writes `bytes` and takes `flops` per node
+    auto pass = [&](double bytes, double flops, auto launch) {
+        ProfScope ps(h, HELM_K_VECTOR, np * bytes, np * flops);
+        return launch();
+    };
+    const double b_bytes = c64 ? 8.0 : 0.0, y_bytes = c64 ? 8.0 : 16.0;
     while (status == HELM_ERR_NOCONV && it < maxit) {
-        CKR(launch_bicg_p(np, h->br, h->bv, sc, h->bp, b32, s));                  // p
+        CKR(pass(64.0 + b_bytes, 18.0, [&] { return launch_bicg_p(np, h->br, h->bv, sc, h->bp, b32, s); }));  // p
         CKR(precond_apply(h, c64 ? nullptr : h->bp, h->by, h->bv));               // y = M p, v = A y
-        CKR(launch_bicg_dots(1, np, h->brh, h->bv, sc, h->partials, ticket, s));  // <rh, v>, alpha
-        CKR(launch_bicg_s(np, h->br, h->bv, sc, h->bs, b32, h->partials, ticket, host, s));  // s = r - alpha v
+        CKR(pass(32.0, 8.0, [&] {                                                 // <rh, v>, alpha
+            return launch_bicg_dots(1, np, h->brh, h->bv, sc, h->partials, ticket, s);
+        }));
+        CKR(pass(48.0 + b_bytes, 12.0, [&] {                                      // s = r - alpha v
+            return launch_bicg_s(np, h->br, h->bv, sc, h->bs, b32, h->partials, ticket, host, s);
+        }));
         CKR(cudaStreamSynchronize(s));
         it++;
         if (host[1] != 0.0) { status = HELM_ERR_BREAKDOWN; break; }
         est = host[0] / fn;
         if (!std::isfinite(est)) { status = HELM_ERR_NONFINITE; break; }
         if (est <= tol) {                                                         // x += alpha y
-            if (c64) CKR(launch_axpy_mixed<float2>(np, sc + 2, (const float2 *)h->by, x, s));
-            else CKR(launch_axpy_mixed<double2>(np, sc + 2, (const double2 *)h->by, x, s));
+            CKR(pass(32.0 + y_bytes, 8.0, [&] {
+                return c64 ? launch_axpy_mixed<float2>(np, sc + 2, (const float2 *)h->by, x, s)
+                           : launch_axpy_mixed<double2>(np, sc + 2, (const double2 *)h->by, x, s);
+            }));
             status = HELM_OK;
             if (st && st->history && it - 1 < st->history_len) st->history[it - 1] = est;
             break;
         }
         CKR(precond_apply(h, c64 ? nullptr : h->bs, h->bz, h->bt));               // z = M s, t = A z
-        CKR(launch_bicg_dots(2, np, h->bt, h->bs, sc, h->partials, ticket, s));   // <t, s>, <t, t>, omega
-        if (c64)                                                                  // x, r = s - omega t, rho, beta
-            CKR(launch_bicg_xr<float2>(np, (const float2 *)h->by, (const float2 *)h->bz, h->bs, h->bt, h->brh, sc, x,
-                                       h->br, h->partials, ticket, host, s));
-        else
-            CKR(launch_bicg_xr<double2>(np, (const double2 *)h->by, (const double2 *)h->bz, h->bs, h->bt, h->brh, sc, x,
-                                        h->br, h->partials, ticket, host, s));
+        CKR(pass(32.0, 12.0, [&] {                                                // <t, s>, <t, t>, omega
+            return launch_bicg_dots(2, np, h->bt, h->bs, sc, h->partials, ticket, s);
+        }));
+        CKR(pass(96.0 + 2 * y_bytes, 36.0, [&] {                                  // x, r = s - omega t, rho, beta
+            return c64 ? launch_bicg_xr<float2>(np, (const float2 *)h->by, (const float2 *)h->bz, h->bs, h->bt, h->brh,
+                                                sc, x, h->br, h->partials, ticket, host, s)
+                       : launch_bicg_xr<double2>(np, (const double2 *)h->by, (const double2 *)h->bz, h->bs, h->bt,
+                                                 h->brh, sc, x, h->br, h->partials, ticket, host, s);
+        }));
         CKR(cudaStreamSynchronize(s));
         est = host[0] / fn;
         if (st && st->history && it - 1 < st->history_len) st->history[it - 1] = est;
