@@ -653,7 +653,8 @@ int gs_df_dot2_nblocks(size_t n, int nv) {
 
 cudaError_t launch_mdot2_pair(size_t n, const float4 *V, size_t ldv, int nv, const float4 *x, const float4 *w,
                               double2 *partials, const int *gate, cudaStream_t s) {
-    if (nv < 1 || nv > 64) return cudaErrorInvalidValue;
+    // 64 basis vectors, and at the end of a cycle of 64 steps the vector that closes it
+    if (nv < 1 || nv > 65) return cudaErrorInvalidValue;
     const unsigned g = (unsigned)gs_df_dot2_nblocks(n, nv) * (unsigned)((nv + DF_CH2 - 1) / DF_CH2);
     launch_pdl(k_mdot2_pair<DF_CH2>, dim3(g), NT, 0, s, n, V, ldv, nv, x, w, partials, gate);
     return cudaGetLastError();
