@@ -289,17 +289,17 @@ def run_reference(args):
 # source file is the one that was captured (same SHA-1); otherwise null.
 NCU_TRAFFIC = {
     ("2d-well-n1025", "update_norm"): dict(kernel="k_update2_pair", source="paper_1012_4307_gb300/csrc/kernels_gs_df.cu",
-                                           sha1="41d6b963621c0f6663226836034cff765733672b", bytes=314204160,
+                                           sha1="3f3e363a23433a0b6f2e06050b39513c6ac34ad7", bytes=314169088,
                                            launch="basis slot j = 15, the mean over a restart cycle being 14.5",
                                            profile="profiles/gram_schmidt_dcgs2_kernels_n1025.md"),
     ("2d-well-n1025", "mdot"): dict(kernel="k_mdot2_pair", source="paper_1012_4307_gb300/csrc/kernels_gs_df.cu",
-                                    sha1="41d6b963621c0f6663226836034cff765733672b", bytes=289714944,
+                                    sha1="3f3e363a23433a0b6f2e06050b39513c6ac34ad7", bytes=289831680,
                                     launch="basis slot j = 15, the mean over a restart cycle being 14.5",
                                     profile="profiles/gram_schmidt_dcgs2_kernels_n1025.md"),
     # captured at 161^3 (whose basis vectors, 67 MB each, also stream from DRAM: traffic 0.98 x the
     # algorithmic bytes) and scaled to 257^3 by the node count
     ("3d-well-n257", "update_norm"): dict(kernel="k_update2_pair", source="paper_1012_4307_gb300/csrc/kernels_gs_df.cu",
-                                          sha1="41d6b963621c0f6663226836034cff765733672b", bytes=3870680573,
+                                          sha1="3f3e363a23433a0b6f2e06050b39513c6ac34ad7", bytes=3870826351,
                                           launch="basis slot j = 10 of FGMRES(20), captured at 161^3 and scaled by "
                                                  "the node count",
                                           profile="profiles/update_pass_3d_well_n161.md"),
